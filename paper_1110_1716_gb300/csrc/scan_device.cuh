@@ -1553,7 +1553,10 @@ __device__ void process_tile(const OView &ov, const MView &mv, const TileView &t
                             const uint32_t i = iw + r;
                             if (static_cast<uint32_t>(r) < gown && i + mm <= n) {
                                 const uint32_t idx = memo_index<SB>(lo, hi, p2, r, mm, mv.sbits, mmask);
-                                if (!((sm.surv[idx >> 5] >> (idx & 31)) & 1u)) keep &= ~(1u << r);
+                                const uint32_t bit = SB == 8 && sm.survb
+                                                         ? pfsm_dyn_smem[idx]   // one byte per 2-gram
+                                                         : (sm.surv[idx >> 5] >> (idx & 31)) & 1u;
+                                if (!bit) keep &= ~(1u << r);
                             }
                         }
                     }
