@@ -329,8 +329,11 @@ int pfsm_test_hold_tiles(pfsm_ctx *ctx, int32_t enable);
  * queue of later chained single-text scans at `entries` instances and, for
  * NFAs, its pool at `pool_states` states of sets larger than 8; instances
  * that find no room continue in place (lazy), as they do when the real
- * queue fills. 0 restores the library's capacities (2^20 DFA entries;
- * 2^18 NFA entries and 2^21 pool states); values above them are clamped.
+ * queue fills. `entries` also caps the candidate list of the sieve (scans
+ * with default parameters); a list that overflows is replaced by every start
+ * of the text. 0 restores the library's capacities (2^20 DFA entries; 2^18
+ * NFA entries and 2^21 pool states; 2^22 candidates); values above them are
+ * clamped.
  * For tests only. Errors: E_INVAL (NULL ctx). */
 int pfsm_test_carry_cap(pfsm_ctx *ctx, uint32_t entries, uint32_t pool_states);
 

@@ -422,9 +422,14 @@ void build_survival(Machine &m) {
     m.sm_m = 0;
     m.sm_m2 = 0;
     const int m1 = std::min(9, 18 / m.sbits);
-    if (m1 >= 1 && survival_bits(m, m1, m.surv)) m.sm_m = m1;
+    auto bits = [&](int mm, std::vector<uint32_t> &to) {
+        return m.kind == 1 && m.sbits == 2 ? survival_bits_dna(m, mm, to) : survival_bits(m, mm, to);
+    };
+    if (m1 >= 1 && bits(m1, m.surv)) m.sm_m = m1;
     const int m2 = std::min(13, 26 / m.sbits);
-    if (m2 > m1 && survival_bits(m, m2, m.surv2)) m.sm_m2 = m2;
+    if (m2 > m1 && bits(m2, m.surv2)) m.sm_m2 = m2;
+    build_sieve(m);
+    build_level3(m);
 }
 
 // ---- residency --------------------------------------------------------------
@@ -432,7 +437,9 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 size_t device_bytes(const Machine &m) {
     size_t b = align256(m.memo.size() * 2 + 4) + align256(m.surv.size() * 4 + 4) +
-               align256(m.surv2.size() * 4 + 4) + align256(m.tail.size() * 2 + 4);
+               align256(m.surv2.size() * 4 + 4) + align256(m.tail.size() * 2 + 4) +
+               align256(m.sv_near.size() * 4) + align256(m.sv_deep.size() * 4) + align256(m.sv_l3.size() * 4) +
+               align256(m.chain.size() * 4) + align256(m.sv_strand.size() * 2 + 4);
     if (m.kind == 0) {
         b += align256(m.dtab.size() * 2 + 4) + align256(m.pool.size() * 4);
     } else {
@@ -557,6 +564,11 @@ static int build_host_image(Machine &m) {
     m.o_tail = put(m.tail.data(), m.tail.size() * 2, 4);
     m.o_surv = put(m.surv.data(), m.surv.size() * 4, 4);
     m.o_surv2 = put(m.surv2.data(), m.surv2.size() * 4, 4);
+    m.o_near = put(m.sv_near.data(), m.sv_near.size() * 4, 0);
+    m.o_deep = put(m.sv_deep.data(), m.sv_deep.size() * 4, 0);
+    m.o_l3 = put(m.sv_l3.data(), m.sv_l3.size() * 4, 0);
+    m.o_chain = put(m.chain.data(), m.chain.size() * 4, 0);
+    m.o_strand = put(m.sv_strand.data(), m.sv_strand.size() * 2, 4);
     if (m.kind == 0) {
         m.o_tab = put(m.dtab.data(), m.dtab.size() * 2, 4);
         m.o_pool = put(m.pool.data(), m.pool.size() * 4, 0);
@@ -599,6 +611,11 @@ static DevMachine dev_view(const Machine &m, uint8_t *base) {
     dm.surv_words = static_cast<uint32_t>(m.surv.size());
     dm.surv2 = m.surv2.empty() ? nullptr : reinterpret_cast<const uint32_t *>(base + m.o_surv2);
     dm.surv2_m = m.sm_m2;
+    dm.sv_near = m.sv_kind ? reinterpret_cast<const uint32_t *>(base + m.o_near) : nullptr;
+    dm.chain = m.chain.empty() ? nullptr : reinterpret_cast<const uint4 *>(base + m.o_chain);
+    dm.sv_strand = m.sv_strand.empty() ? nullptr : reinterpret_cast<const uint16_t *>(base + m.o_strand);
+    dm.sv_l3 = m.sv_l3.empty() ? nullptr : reinterpret_cast<const uint32_t *>(base + m.o_l3);
+    dm.sv_deep = m.sv_deep.empty() ? nullptr : reinterpret_cast<const uint32_t *>(base + m.o_deep);
     if (m.kind == 0) {
         dm.dtab = reinterpret_cast<const uint16_t *>(base + m.o_tab);
         dm.pool = reinterpret_cast<const uint32_t *>(base + m.o_pool);
@@ -630,9 +647,13 @@ int make_resident(pfsm_ctx *ctx, int id, Machine &m, cudaStream_t s) {
         return PFSM_E_CUDA;
     }
     if (m.dev) {
-        if (cudaEventQuery(m.ready) != cudaSuccess) {
-            cudaGetLastError();
-            cudaStreamWaitEvent(s, m.ready, 0);
+        if (!m.uploaded) {
+            if (cudaEventQuery(m.ready) == cudaSuccess) {
+                m.uploaded = true;
+            } else {
+                cudaGetLastError();
+                cudaStreamWaitEvent(s, m.ready, 0);
+            }
         }
         return PFSM_OK;
     }
@@ -653,6 +674,7 @@ int make_resident(pfsm_ctx *ctx, int id, Machine &m, cudaStream_t s) {
         return PFSM_E_CUDA;
     }
     m.dev = p;
+    m.uploaded = false;
     m.dev_bytes = bytes;
     m.dm = dev_view(m, static_cast<uint8_t *>(p));
     ctx->resident_bytes += bytes;
@@ -710,14 +732,18 @@ Slot *get_slot(pfsm_ctx *ctx, cudaStream_t s) {
     if (it != ctx->slots.end()) return &it->second;
     Slot sl;
     void *p = nullptr;
-    const size_t bytes = 64 + static_cast<size_t>(kCarryCap) * 16;
+    constexpr size_t head = 128;   // status, carry counters, the sieve's counters
+    const size_t bytes = head + static_cast<size_t>(kCarryCap) * 16 + static_cast<size_t>(kCandCap) * sizeof(uint2);
     if (cudaMalloc(&p, bytes) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
     sl.status = static_cast<unsigned long long *>(p);
     sl.carry_n = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(p) + 16);
-    sl.carry = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(p) + 64);
+    sl.sv_status = reinterpret_cast<unsigned long long *>(static_cast<uint8_t *>(p) + 64);
+    sl.sv_count = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(p) + 80);
+    sl.carry = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(p) + head);
+    sl.cand = reinterpret_cast<uint2 *>(sl.carry + static_cast<size_t>(kCarryCap) * 4);
     if (cudaMallocHost(&sl.host_status, 2 * sizeof(unsigned long long)) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(p);
@@ -778,6 +804,7 @@ int apply_k(pfsm_ctx *ctx, Machine &m, bool may_lower) {
         }
         --m.k;   // k = 0 always builds (no table)
     }
+    build_level3(m);   // its rows follow the second-level records
     m.params.prefix_k = m.k > 0 ? m.k : -1;
     return PFSM_OK;
 }
@@ -787,6 +814,35 @@ struct Plan {
     int threads, grid;
     uint32_t smem;
 };
+
+// The machine's part of the scan arguments.
+static void machine_args(const Machine &m, ScanArgs &a) {
+    a.Q = m.Q;
+    a.S = m.S;
+    a.q0 = m.q0;
+    a.k = m.k;
+    a.sbits = m.sbits;
+    a.memo_n = m.dm.memo_n;
+    a.memo = m.dm.memo;
+    a.tail = m.dm.tail;
+    a.ecl_off = m.dm.ecl_off;
+    a.ecl_tgt = m.dm.ecl_tgt;
+    a.dtab = m.dm.dtab;
+    a.off = m.dm.off;
+    a.tgt = m.dm.tgt;
+    a.pool = m.dm.pool;
+    a.l2tab = m.dm.l2tab;
+    a.memox = m.dm.memox;
+    a.pool2 = m.dm.pool2;
+    a.pool_n = m.dm.pool_n;
+    a.band = m.dm.band;
+    a.surv = m.dm.surv;
+    a.surv_m = m.dm.surv_m;
+    a.surv_words = m.dm.surv_words;
+    a.surv2 = m.dm.surv2;
+    a.surv2_m = m.dm.surv2_m;
+    a.Wq = m.kind == 1 ? m.dm.Wq : 0;
+}
 
 // Launch geometry and shared-memory layout of one scan.
 int plan_scan(pfsm_ctx *ctx, const Machine &m, const uint8_t *text, uint64_t n, Plan &pl) {
@@ -832,31 +888,7 @@ int plan_scan(pfsm_ctx *ctx, const Machine &m, const uint8_t *text, uint64_t n, 
     // memory for CTAs
     a.nbuf = spt == 8 ? 2 : 3;
     a.shift = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(text) & 15);
-    a.Q = m.Q;
-    a.S = m.S;
-    a.q0 = m.q0;
-    a.k = m.k;
-    a.sbits = m.sbits;
-    a.memo_n = m.dm.memo_n;
-    a.memo = m.dm.memo;
-    a.tail = m.dm.tail;
-    a.ecl_off = m.dm.ecl_off;
-    a.ecl_tgt = m.dm.ecl_tgt;
-    a.dtab = m.dm.dtab;
-    a.off = m.dm.off;
-    a.tgt = m.dm.tgt;
-    a.pool = m.dm.pool;
-    a.l2tab = m.dm.l2tab;
-    a.memox = m.dm.memox;
-    a.pool2 = m.dm.pool2;
-    a.pool_n = m.dm.pool_n;
-    a.band = m.dm.band;
-    a.surv = m.dm.surv;
-    a.surv_m = m.dm.surv_m;
-    a.surv_words = m.dm.surv_words;
-    a.surv2 = m.dm.surv2;
-    a.surv2_m = m.dm.surv2_m;
-    a.Wq = m.kind == 1 ? m.dm.Wq : 0;
+    machine_args(m, a);
     uint32_t tab_bytes = m.kind == 0 ? ((static_cast<uint32_t>(m.Q) * m.S + 1) / 2) * 4 : 0;
     // table placement: shared memory when asked, or (auto) when small
     a.tab_smem = 0;
@@ -931,14 +963,125 @@ void collect_timing(pfsm_ctx *ctx, Slot *slot, int keep) {
     }
 }
 
+// A machine's scans take the sieve (sieve.cu) when it has the tables and all
+// its parameters are the defaults: any other setting shapes the tile kernel,
+// which then runs. (Positions within 256 of 2^32 would wrap in the sieve.)
+// A scan that is being captured takes the tile kernel: the sieve's counters
+// belong to the stream, and a graph may be replayed on others.
+static bool takes_sieve(const pfsm_ctx *ctx, const Machine &m, uint64_t n, cudaStream_t s) {
+    if (!m.sv_kind || m.k <= 0 || ctx->hold_tiles || n >= (1ull << 32) - 256) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    pfsm_params d{};
+    d.prefix_k = m.params.prefix_k;   // lowered at load where the records did not fit
+    fill_defaults(m, d);
+    return memcmp(&d, &m.params, sizeof(d)) == 0;
+}
+
+// The launches of a sieved scan.
+static int sieve_enqueue(pfsm_ctx *ctx, const Machine &m, const uint8_t *text, uint64_t n, uint32_t *out,
+                         uint64_t cap, unsigned long long *status, Slot *slot, cudaStream_t s) {
+    SieveArgs a{};
+    a.text = text;
+    a.n = static_cast<uint32_t>(n);
+    a.Q = m.Q;
+    a.S = m.S;
+    a.q0 = m.q0;
+    a.near = m.dm.sv_near;
+    a.deep = m.dm.sv_deep;
+    // (bytes: single starts are tested by their 3-gram)
+    a.surv2 = m.sv_kind == SIEVE_DNA || (m.sbits == 8 && m.sm_m2 == 3) ? m.dm.surv2 : nullptr;
+    a.dtab = m.dm.dtab;
+    a.memo = m.dm.memo;
+    a.chain = m.dm.chain;
+    a.sbits = m.sbits;
+    a.memox = m.dm.memox;
+    a.l2tab = m.dm.l2tab;
+    a.l3 = m.dm.sv_l3;
+    a.strand = m.dm.sv_strand;
+    a.k = m.k;
+    a.cand = slot->cand;
+    a.cand_n = slot->sv_count;
+    a.done = slot->sv_count + 1;
+    a.cand_cap = ctx->test_carry_cap ? std::min(kCandCap, ctx->test_carry_cap) : kCandCap;
+    a.out = out;
+    a.cap = cap;
+    a.status = slot->sv_status;
+    a.status_out = status;
+    // the sieve, then the kernel that finishes its candidates and leaves the
+    // counters zero; they are cleared here before the stream's first scan
+    // and after one that was not wholly launched
+    auto launch = [&](auto &&finish) {
+        if (!slot->sv_ready && cudaMemsetAsync(slot->sv_status, 0, 32, s) != cudaSuccess) return PFSM_E_CUDA;
+        slot->sv_ready = false;
+        if (launch_sieve(a, m.sv_kind, ctx->nsm, ctx->smem_set, s) != cudaSuccess || finish() != cudaSuccess)
+            return PFSM_E_CUDA;
+        slot->sv_ready = true;
+        return PFSM_OK;
+    };
+    if (m.kind == 0) return launch([&] { return launch_finish_dfa(a, ctx->nsm, s); });
+    // the finishing kernel, in half an SM's shared memory: band rows and
+    // warp-wide bitsets as far as they fit
+    ScanArgs f;
+    memset(&f, 0, sizeof(f));
+    f.text = text;
+    f.n = a.n;
+    machine_args(m, f);
+    f.out = out;
+    f.cap = cap;
+    f.status = slot->sv_status;
+    f.stage_n = 32;
+    f.settle_steps = m.params.settle > 0 ? m.params.settle : 0;
+    constexpr int warps = kFinishThreads / 32;
+    const uint32_t most = ctx->smem_sm / 2 - ctx->smem_rsv;
+    const uint32_t band = static_cast<uint32_t>(m.band.size() * 4);
+    const uint32_t coop = static_cast<uint32_t>(warps * 2 * m.dm.Wq * 4);
+    uint32_t smem = layout_finish_nfa(f, band, coop);
+    if (smem > most) smem = layout_finish_nfa(f, band, 0);
+    if (smem > most) smem = layout_finish_nfa(f, 0, 0);
+    if (!f.coop_smem) {
+        const size_t words = static_cast<size_t>(2 * ctx->nsm) * warps * 2 * m.dm.Wq;
+        if (ensure_words(&slot->coop, &slot->coop_words, words)) return PFSM_E_NOMEM;
+        f.coop_g = slot->coop;
+    }
+    return launch([&] { return launch_finish_nfa(f, a, smem, ctx->nsm, ctx->smem_set, s); });
+}
+
 int scan_enqueue(pfsm_ctx *ctx, pfsm_aut aut, const uint8_t *text, uint64_t n, uint32_t *out,
-                 uint64_t cap, unsigned long long *status, Slot *slot, cudaStream_t s) {
+                 uint64_t cap, unsigned long long *status, Slot *slot, cudaStream_t s,
+                 bool *in_host = nullptr) {
     NvtxRange nr("pfsm scan (plan, tile kernel, carry)");
     auto it = ctx->machines.find(aut);
     if (it == ctx->machines.end()) return PFSM_E_NOENT;
     Machine &m = it->second;
     int st = make_resident(ctx, aut, m, s);
     if (st) return st;
+    int ev = -1;
+    auto time_begin = [&]() {
+        if (!ctx->timing) return;
+        collect_timing(ctx, slot, kEventRing - 1);
+        ev = slot->ev_head;
+        cudaEventRecord(slot->ev[2 * ev], s);
+    };
+    auto time_end = [&]() {
+        if (ev < 0) return;
+        cudaEventRecord(slot->ev[2 * ev + 1], s);
+        slot->ev_head = (slot->ev_head + 1) % kEventRing;
+        slot->ev_pending++;
+    };
+    if (n > 0 && takes_sieve(ctx, m, n, s)) {
+        time_begin();
+        // a scan that is waited for gets its status written to host memory
+        if (in_host) *in_host = true;
+        st = sieve_enqueue(ctx, m, text, n, out, cap, in_host ? slot->host_status : status, slot, s);
+        time_end();
+        if (st) return st;
+        Machine *mp = &m;
+        return mark_use(ctx, s, &mp, 1);
+    }
     if (cudaMemsetAsync(status, 0, 2 * sizeof(unsigned long long), s) != cudaSuccess)
         return PFSM_E_CUDA;
     if (n == 0) return PFSM_OK;
@@ -972,18 +1115,9 @@ int scan_enqueue(pfsm_ctx *ctx, pfsm_aut aut, const uint8_t *text, uint64_t n, u
     }
     if (pl.a.carry_cap && cudaMemsetAsync(slot->carry_n, 0, 8 * sizeof(uint32_t), s) != cudaSuccess)
         return PFSM_E_CUDA;
-    int ev = -1;
-    if (ctx->timing) {
-        collect_timing(ctx, slot, kEventRing - 1);
-        ev = slot->ev_head;
-        cudaEventRecord(slot->ev[2 * ev], s);
-    }
+    time_begin();
     cudaError_t e = launch_scan(pl.a, m.kind, pl.threads, pl.grid, pl.smem, s);
-    if (ev >= 0) {
-        cudaEventRecord(slot->ev[2 * ev + 1], s);
-        slot->ev_head = (slot->ev_head + 1) % kEventRing;
-        slot->ev_pending++;
-    }
+    time_end();
     if (e != cudaSuccess) return PFSM_E_CUDA;
     if (m.kind == 0 && pl.a.carry_cap > 0) {
         NvtxRange nr("pfsm carry_dfa launch");
@@ -1332,10 +1466,12 @@ int pfsm_scan(pfsm_ctx *ctx, pfsm_aut aut, const uint8_t *text_dev, uint64_t n,
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     Slot *slot = get_slot(ctx, s);
     if (!slot) return PFSM_E_NOMEM;
+    bool in_host = false;
     int st = scan_enqueue(ctx, aut, text_dev, n, reinterpret_cast<uint32_t *>(out_dev), cap,
-                          slot->status, slot, s);
+                          slot->status, slot, s, &in_host);
     if (st) return st;
-    if (cudaMemcpyAsync(slot->host_status, slot->status, 2 * sizeof(unsigned long long),
+    if (!in_host &&
+        cudaMemcpyAsync(slot->host_status, slot->status, 2 * sizeof(unsigned long long),
                         cudaMemcpyDeviceToHost, s) != cudaSuccess)
         return PFSM_E_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return PFSM_E_CUDA;

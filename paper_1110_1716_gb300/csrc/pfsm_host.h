@@ -15,6 +15,7 @@ namespace pfsm {
 
 constexpr uint64_t kDefaultBudget = 8ull << 30;
 constexpr uint32_t kCarryCap = 1u << 20;     // carry entries per stream slot
+constexpr uint32_t kCandCap = 1u << 22;      // sieve candidates per stream slot (32 MB)
 constexpr uint32_t kSmemMax = 232448;        // opt-in shared memory per CTA
 constexpr uint32_t kSmemStatic = 1024;       // room left for static shared memory (single-text kernels: none)
 constexpr uint32_t kBatchSmemStatic = 2048;  // the batch class kernels' static shared memory (1.5 KB)
@@ -45,6 +46,13 @@ struct Machine {
     // survival bitmap over m-grams (m = 0: none)
     int sm_m = 0, sm_m2 = 0;
     std::vector<uint32_t> surv, surv2;   // shallow (shared memory) and deep (global) bitmaps
+    // sieve tables (see SIEVE_DNA_STEP): kind, near and deep bitmaps
+    int sv_kind = 0;
+    std::vector<uint32_t> sv_near, sv_deep, sv_l3;
+    std::vector<uint32_t> chain;      // DFA with a sieve: four words per state
+    // NFA with a sieve whose states but q0 all have band rows and none leads
+    // back to q0: the weakly connected part (without q0) of every state
+    std::vector<uint16_t> sv_strand;
     pfsm_params params{};
     // residency: the device image is built once in pinned host memory and
     // copied in on the scan's stream whenever the machine becomes resident
@@ -54,8 +62,9 @@ struct Machine {
     size_t img_bytes = 0;
     size_t o_memo = 0, o_tail = 0, o_surv = 0, o_surv2 = 0, o_tab = 0, o_off = 0,
            o_tgt = 0, o_pool = 0, o_band = 0, o_eoff = 0, o_etgt = 0, o_l2tab = 0,
-           o_pool2 = 0, o_memox = 0;   // section offsets
+           o_pool2 = 0, o_memox = 0, o_near = 0, o_deep = 0, o_l3 = 0, o_chain = 0, o_strand = 0;   // section offsets
     cudaEvent_t ready = nullptr;      // recorded after the last upload
+    bool uploaded = false;            // ... and seen to have completed
     // last use per stream (an event recorded after a launch that read the
     // image); an eviction orders its free after every one of them
     std::vector<std::pair<cudaStream_t, cudaEvent_t>> uses;
@@ -69,6 +78,12 @@ struct Slot {   // per-stream scratch
     unsigned long long *status = nullptr;   // device [2]
     uint32_t *carry_n = nullptr;
     uint32_t *carry = nullptr;              // kCarryCap entries of 4 words
+    uint2 *cand = nullptr;                  // kCandCap candidates of the sieve
+    // the sieve's counters, zero between scans: {matches, error bits} and
+    // {candidates, CTAs done}
+    unsigned long long *sv_status = nullptr;
+    uint32_t *sv_count = nullptr;
+    bool sv_ready = false;                  // the counters are zero
     unsigned long long *host_status = nullptr;   // pinned [2]
     uint32_t *coop = nullptr;               // warp-wide NFA bitsets
     size_t coop_words = 0;
@@ -151,6 +166,7 @@ struct pfsm_ctx {
     pfsm::BatchShape batch_shape[pfsm::kBatchClasses];
     uint32_t smem_sm = 233472;    // shared memory per SM
     uint32_t smem_rsv = 1024;     // shared memory the system reserves per CTA
+    std::atomic<uint32_t> smem_set{0};   // see launch_sieve
 };
 
 namespace pfsm {
@@ -158,6 +174,9 @@ namespace pfsm {
 int ceil_log2(int S);
 bool build_memo(Machine &m);
 void build_survival(Machine &m);
+void build_sieve(Machine &m);                                              // sieve_tables.cu
+void build_level3(Machine &m);
+bool survival_bits_dna(const Machine &m, int mm, std::vector<uint32_t> &bits);
 size_t align256(size_t x);
 void release(pfsm_ctx *ctx, Machine &m);
 void drop_host_image(Machine &m);

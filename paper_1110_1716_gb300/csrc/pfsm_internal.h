@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "pfsm.h"
 
 namespace pfsm {
@@ -51,6 +53,13 @@ constexpr uint32_t L2_GRAMS = 1u << (2 * L2_SYMS);
 constexpr uint16_t L2_NONE = 0xFFFF;
 constexpr uint16_t L2_EMPTY = 0xFFFF;
 constexpr uint32_t L2_MAX_SETS = 4096;   // at most 8 MB of second-level tables
+// Third level (machines with a sieve): one row of 4^L3_SYMS bits per word of
+// the second-level pool; in the row of a record, the bit of the next L3_SYMS
+// symbols is set when the record has matches, or its set meets a final state
+// within them or still holds a state after them.
+constexpr int L3_SYMS = 6;
+constexpr uint32_t L3_GRAMS = 1u << (2 * L3_SYMS);
+constexpr uint32_t L3_MAX_ROWS = 1u << 14;   // 8 MB
 constexpr uint32_t L2_NO_REC = 0xFFFFFFFFu;   // (device) a start without a second-level record
 // memox[w] (beside the prefix table, same index): the survivor-set index x
 // of k-gram w's first-level record when that record has survivors, no
@@ -75,6 +84,30 @@ __host__ __device__ inline uint32_t tail_base(int j, int sbits) {
 // marks a state with a target outside that window: its rows are read from
 // the CSR arrays instead.
 constexpr uint32_t BAND_CSR = 0xFFFFFFFFu;
+
+// Sieve (sieve.cu, sieve_tables.cu): bitmaps tested once per few starts.
+// SIEVE_DNA (2-bit symbols): `near` one bit per SIEVE_NEAR_M-gram, `deep` one
+// bit per SIEVE_DEEP_M-gram, both of the gram that begins at the last of
+// SIEVE_DNA_STEP starts. SIEVE_BYTES (DFAs over wider symbols): `near` one
+// bit per hash of four bytes, the gram that begins at the last of
+// SIEVE_BYTE_STEP starts. Bit x of a word is stored at 31 - x.
+constexpr int SIEVE_DNA_STEP = 2, SIEVE_BYTE_STEP = 4;
+constexpr int SIEVE_NONE = 0, SIEVE_DNA = 1, SIEVE_BYTES = 2;
+constexpr int SIEVE_NEAR_M = 10;     // 128 KB: what a CTA's shared memory holds
+constexpr int SIEVE_DEEP_M = 13;     // 8 MB in L2
+constexpr int SIEVE_HASH_BITS = 19;  // 64 KB: three CTAs per SM
+constexpr uint32_t SIEVE_NO_RECORD = 0xFFFFFFFFu;   // a candidate without a second-level record
+constexpr uint32_t SIEVE_HASH_MAX = 1u << (SIEVE_HASH_BITS - 4);   // most bits set
+// A sieved DFA's chains, one uint4 per state: where exactly one symbol leads
+// on from the state, and so on, up to eight symbols or the first final state:
+// x, y the symbols, z their number | 1 << 8 when the last state is final, w
+// the last state. z = 0: the state branches (or leads nowhere).
+
+// The word of a four-byte gram; its bit there is 31 - (low five bits of the
+// gram), so that a left shift by the gram brings it to the top.
+__host__ __device__ inline uint32_t sieve_hash_word(uint32_t four_bytes) {
+    return (four_bytes * 0x9E3779B1u) >> (32 - (SIEVE_HASH_BITS - 5));
+}
 
 // Survival bitmap (optional): one bit per m-gram, set when an instance
 // started at q0 meets a final state within those m symbols or still holds a
@@ -165,6 +198,31 @@ struct ScanArgs {
     int32_t spt;            // starts per thread per filter round: 8 or 32 (0 = 32)
 };
 
+// Arguments of the sieve and of the kernels that finish its candidates.
+struct SieveArgs {
+    const uint8_t *text;
+    uint32_t n;
+    int32_t Q, S, q0;
+    const uint32_t *near, *deep;   // sampled bitmaps (see SIEVE_DNA_STEP)
+    const uint32_t *surv2;         // deep survival bitmap of single starts, or null (bytes)
+    const uint16_t *dtab, *memo;   // DFA: table, prefix table (k symbols of sbits)
+    const uint4 *chain;            // DFA: chains (see "A sieved DFA's chains")
+    int32_t sbits;
+    const uint16_t *memox, *l2tab; // NFA with l3: second level (see L2_SYMS)
+    const uint32_t *l3;            // NFA: third level (see L3_SYMS), or null
+    const uint16_t *strand;        // NFA: strand of every state (see sv_strand), or null
+    int32_t k;
+    uint2 *cand;                   // candidates, cand_cap of them: start and second-level
+                                   // record (or SIEVE_NO_RECORD)
+    uint32_t *cand_n;              // their number (past cand_cap: the list is incomplete)
+    uint32_t cand_cap;
+    uint32_t *out;
+    uint64_t cap;
+    unsigned long long *status;      // the stream's own counters, zero between scans
+    unsigned long long *status_out;  // where the scan's status goes
+    uint32_t *done;                  // CTAs that ended, zero between scans
+};
+
 // Dynamic shared memory of the NFA carry kernel with `nw` warps: band rows
 // (when the scan stages them), then per warp the lane slots, the match
 // staging buffer and (when the scan keeps them in shared memory) the two
@@ -227,6 +285,9 @@ struct DevMachine {
     uint32_t surv_words;
     int32_t surv2_m;
     const uint32_t *surv2;
+    const uint32_t *sv_near, *sv_deep, *sv_l3;   // sieve tables, or null
+    const uint4 *chain;
+    const uint16_t *sv_strand;
     // batch: byte offsets of the tables copied into the CTA's shared-memory
     // table arena when this machine's tiles run (kNotStaged: read from
     // global memory; for the survival bitmap: not used)
@@ -273,6 +334,16 @@ int max_ctas_per_sm(int kind, int sbits, int threads, uint32_t smem, bool tab_sm
 cudaError_t launch_scan_spt8(const ScanArgs &a, int kind, int threads, int grid, uint32_t smem,
                              cudaStream_t s);
 int max_ctas_per_sm_spt8(int kind, int sbits, int threads, uint32_t smem, bool tab_smem);
+
+// the sieve and its finishing kernels (sieve.cu)
+// (smem_set: which kernels' shared-memory limits this context has raised)
+cudaError_t launch_sieve(const SieveArgs &a, int kind, int nsm, std::atomic<uint32_t> &smem_set, cudaStream_t s);
+cudaError_t launch_finish_dfa(const SieveArgs &a, int nsm, cudaStream_t s);
+constexpr int kFinishThreads = 256;   // of finish_nfa, two CTAs per SM
+// Fills the offsets of `a` (stage_n set) for finish_nfa; returns the bytes.
+uint32_t layout_finish_nfa(ScanArgs &a, uint32_t band_bytes, uint32_t coop_bytes);
+cudaError_t launch_finish_nfa(const ScanArgs &a, const SieveArgs &sv, uint32_t smem, int nsm,
+                              std::atomic<uint32_t> &smem_set, cudaStream_t s);
 
 // ---- batch launch helpers (batch_kernels.cu) -----------------------------
 int batch_class(int kind, int sbits, int k, bool tab_smem);

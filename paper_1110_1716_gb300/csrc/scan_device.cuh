@@ -260,12 +260,16 @@ __device__ __forceinline__ uint32_t bytes_ge32(uint32_t x, uint32_t S) {
 // other partial product lands at bit 32 or above (dropped) or below bit 24,
 // and those lower ones sum to less than 2^24, so nothing carries into the
 // top byte. Three byte permutations gather the four top bytes.
-__device__ __forceinline__ uint32_t pack16(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
+// (pack16_sym takes bytes that are symbols; pack16 drops their upper bits.)
+__device__ __forceinline__ uint32_t pack16_sym(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
     constexpr uint32_t M = 0x01041040u;
-    constexpr uint32_t K = 0x03030303u;
-    const uint32_t lo = __byte_perm((w0 & K) * M, (w1 & K) * M, 0x0073);
-    const uint32_t hi = __byte_perm((w2 & K) * M, (w3 & K) * M, 0x0073);
+    const uint32_t lo = __byte_perm(w0 * M, w1 * M, 0x0073);
+    const uint32_t hi = __byte_perm(w2 * M, w3 * M, 0x0073);
     return __byte_perm(lo, hi, 0x5410);
+}
+__device__ __forceinline__ uint32_t pack16(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
+    constexpr uint32_t K = 0x03030303u;
+    return pack16_sym(w0 & K, w1 & K, w2 & K, w3 & K);
 }
 
 // Packs the staged tile (len bytes at tsm) to 2-bit symbols, 16 per word,

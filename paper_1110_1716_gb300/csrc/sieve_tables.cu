@@ -1,0 +1,441 @@
+// Load-time tables of the sieve (sieve.cu): which grams can occur a few
+// symbols into an instance that still matters.
+//
+// A start i is dead when its instance meets no final state and holds no state
+// any more after some symbols; only the others can report. One lookup at a
+// sampled position answers for `step` starts at once: for the gram w read at
+// position p, the bit of w is set when, for some offset o < step and some o
+// symbols before p, an instance started at p - o is still alive after w or
+// meets a final state inside w. A clear bit settles all `step` starts. This
+// needs every final state to lie at least `step` symbols from q0 (a shorter
+// match would end before the gram); other machines have no sieve.
+#include <stdint.h>
+#include <string.h>
+
+#include <algorithm>
+#include <atomic>
+#include <thread>
+#include <vector>
+
+#include "pfsm_host.h"
+
+namespace pfsm {
+
+namespace {
+
+// delta as edges, in the order of their states and symbols; targets as
+// state | FINAL_BIT, epsilon closures among them.
+struct Delta {
+    int Q = 0, S = 0;
+    std::vector<uint32_t> row;     // first edge of every state
+    std::vector<uint8_t> sym;      // per edge
+    std::vector<uint16_t> tgt;
+    std::vector<uint32_t> off;     // alphabets of at most 4: first edge of every (state, symbol)
+    std::vector<uint16_t> start;   // the states an instance starts with
+    void add(int a, uint16_t t) {
+        sym.push_back(static_cast<uint8_t>(a));
+        tgt.push_back(t);
+    }
+};
+
+void flatten(const Machine &m, Delta &d) {
+    d.Q = m.Q;
+    d.S = m.S;
+    d.row.assign(static_cast<size_t>(m.Q) + 1, 0);
+    d.start.assign(1, static_cast<uint16_t>(m.q0));
+    const bool small = m.S <= 4;
+    if (small) d.off.assign(static_cast<size_t>(m.Q) * m.S + 1, 0);
+    std::vector<uint16_t> ts;
+    constexpr uint64_t DEAD4 = 0x0001000100010001ull * DEAD16;
+    for (int q = 0; q < m.Q; ++q) {
+        d.row[q] = static_cast<uint32_t>(d.tgt.size());
+        const size_t r = static_cast<size_t>(q) * m.S;
+        for (int a = 0; a < m.S; ++a) {
+            if (small) d.off[r + a] = static_cast<uint32_t>(d.tgt.size());
+            if (m.kind == 0) {
+                const uint16_t *e = m.dtab.data() + r + a;
+                if (!small && (a & 3) == 0 && a + 4 <= m.S) {   // wide rows are mostly dead
+                    uint64_t four;
+                    memcpy(&four, e, sizeof(four));
+                    if (four == DEAD4) {
+                        a += 3;
+                        continue;
+                    }
+                }
+                if (*e != DEAD16) d.add(a, *e);
+                continue;
+            }
+            const uint32_t lo = m.off[r + a], hi = m.off[r + a + 1];
+            if (m.ecl_off.empty()) {
+                for (uint32_t e = lo; e < hi; ++e) d.add(a, m.tgt[e]);
+                continue;
+            }
+            ts.clear();
+            for (uint32_t e = lo; e < hi; ++e) {
+                const uint32_t t = m.tgt[e] & 0x7FFF;
+                ts.push_back(m.tgt[e]);
+                ts.insert(ts.end(), m.ecl_tgt.begin() + m.ecl_off[t], m.ecl_tgt.begin() + m.ecl_off[t + 1]);
+            }
+            std::sort(ts.begin(), ts.end());
+            ts.erase(std::unique(ts.begin(), ts.end()), ts.end());
+            for (uint16_t t : ts) d.add(a, t);
+        }
+    }
+    d.row[m.Q] = static_cast<uint32_t>(d.tgt.size());
+    if (small) d.off[static_cast<size_t>(m.Q) * m.S] = static_cast<uint32_t>(d.tgt.size());
+    if (!m.ecl_off.empty())
+        for (uint32_t x = m.ecl_off[m.q0]; x < m.ecl_off[m.q0 + 1]; ++x)
+            d.start.push_back(static_cast<uint16_t>(m.ecl_tgt[x] & 0x7FFF));
+}
+
+// The states an instance can hold after 0 .. step - 1 symbols; false when one
+// of them, past the start, is final.
+bool sampled_states(const Delta &d, int step, std::vector<uint16_t> &u) {
+    std::vector<uint8_t> in(d.Q, 0);
+    std::vector<uint16_t> cur = d.start;
+    u = cur;
+    for (uint16_t q : cur) in[q] = 1;
+    for (int o = 1; o < step; ++o) {
+        std::vector<uint8_t> seen(d.Q, 0);
+        std::vector<uint16_t> nxt;
+        for (uint16_t q : cur)
+            for (uint32_t e = d.row[q]; e < d.row[q + 1]; ++e) {
+                const uint16_t t = d.tgt[e];
+                if (t & FINAL_BIT) return false;
+                if (!seen[t]) {
+                    seen[t] = 1;
+                    nxt.push_back(t);
+                }
+            }
+        for (uint16_t q : nxt)
+            if (!in[q]) {
+                in[q] = 1;
+                u.push_back(q);
+            }
+        cur.swap(nxt);
+    }
+    return true;
+}
+
+// ---- 2-bit symbols: one bit per m-gram (symbol j at bits 2j of the index) ----
+// Depth-first over the grams. The subtrees are split by symbol 5 and the
+// high bit of symbol 4 (index bits 9 .. 11) into 8 parts, one per thread:
+// those bits choose the cache line, so no two threads write one line.
+constexpr int kParts = 8;
+
+struct GramWalk {
+    const Delta &d;
+    const std::vector<uint8_t> &next;   // per state: the symbols it has successors on
+    int mm;
+    uint32_t *bits;
+    uint64_t limit;      // give up past this many set bits
+    int part;            // -1: the whole tree
+    uint64_t ones = 0;
+    std::vector<uint32_t> mark;
+    uint32_t stamp = 0;
+    std::vector<std::vector<uint16_t>> lv;
+
+    GramWalk(const Delta &dd, const std::vector<uint8_t> &nx, int m, uint32_t *b, uint64_t lim, int p)
+        : d(dd), next(nx), mm(m), bits(b), limit(lim), part(p), mark(dd.Q, 0), lv(m + 1) {}
+
+    bool mine(int depth, uint32_t prefix) const {
+        if (part < 0) return true;
+        if (depth > 5) return ((prefix >> 9) & 7u) == static_cast<uint32_t>(part);
+        if (depth == 5) return ((prefix >> 9) & 1u) == static_cast<uint32_t>(part & 1);
+        return true;
+    }
+    void set_range(uint32_t p, int depth) {   // every extension of a depth-long prefix
+        const uint32_t rest = static_cast<uint32_t>(mm - depth) * 2;
+        for (uint32_t hw = 0; hw < (1u << rest); ++hw) {
+            const uint32_t w = p | (hw << (2 * depth));
+            if (depth < 6 && !mine(6, w)) continue;
+            bits[w >> 5] |= 1u << (w & 31);
+            ++ones;
+        }
+    }
+    void run(int depth, uint32_t prefix) {
+        const std::vector<uint16_t> &s = lv[depth];
+        if (ones > limit) return;
+        if (depth + 1 == mm) {   // the last symbol: alive when any state has a successor
+            uint32_t any = 0;
+            for (uint16_t q : s) any |= next[q];
+            for (int a = 0; a < 4; ++a)
+                if ((any >> a) & 1u) {
+                    const uint32_t w = prefix | (static_cast<uint32_t>(a) << (2 * depth));
+                    bits[w >> 5] |= 1u << (w & 31);
+                    ++ones;
+                }
+            return;
+        }
+        for (int a = 0; a < d.S; ++a) {
+            const uint32_t p = prefix | (static_cast<uint32_t>(a) << (2 * depth));
+            if (!mine(depth + 1, p)) continue;
+            std::vector<uint16_t> &n = lv[depth + 1];
+            n.clear();
+            bool hit = false;
+            ++stamp;
+            for (uint16_t q : s) {
+                const size_t r = static_cast<size_t>(q) * d.S + a;
+                for (uint32_t e = d.off[r]; e < d.off[r + 1]; ++e) {
+                    const uint16_t t = d.tgt[e], ts = t & 0x7FFF;
+                    hit |= (t & FINAL_BIT) != 0;
+                    if (mark[ts] == stamp) continue;
+                    mark[ts] = stamp;
+                    n.push_back(ts);
+                }
+            }
+            if (hit) set_range(p, depth + 1);
+            else if (!n.empty()) run(depth + 1, p);
+        }
+    }
+};
+
+// Per state: the symbols it has successors on.
+std::vector<uint8_t> successor_symbols(const Delta &d) {
+    std::vector<uint8_t> next(d.Q, 0);
+    for (int q = 0; q < d.Q; ++q)
+        for (int a = 0; a < d.S; ++a)
+            if (d.off[static_cast<size_t>(q) * d.S + a] != d.off[static_cast<size_t>(q) * d.S + a + 1])
+                next[q] |= static_cast<uint8_t>(1u << a);
+    return next;
+}
+
+// The m-gram bitmap of instances that hold `from`; false (and no bitmap)
+// when more than `limit` grams are set.
+bool gram_bits(const Delta &d, const std::vector<uint16_t> &from, int mm, uint64_t limit,
+               std::vector<uint32_t> &bits) {
+    const std::vector<uint8_t> next = successor_symbols(d);
+    bits.assign((size_t(1) << (2 * mm)) / 32, 0);
+    const bool split = mm >= 10;
+    const int parts = split ? kParts : 1;
+    // (a part may hold four times its share before it gives up on its own)
+    const uint64_t part_limit = split ? limit / kParts * 4 : limit;
+    std::vector<uint64_t> ones(parts, 0);
+    auto work = [&](int p) {
+        GramWalk w(d, next, mm, bits.data(), part_limit, split ? p : -1);
+        w.lv[0] = from;
+        w.run(0, 0);
+        ones[p] = w.ones;
+    };
+    const int threads = std::min<int>(parts, std::max(1u, std::thread::hardware_concurrency()));
+    if (threads <= 1) {
+        for (int p = 0; p < parts; ++p) work(p);
+    } else {
+        std::atomic<int> at{0};
+        std::vector<std::thread> pool;
+        auto loop = [&]() {
+            for (int p; (p = at.fetch_add(1)) < parts;) work(p);
+        };
+        for (int t = 1; t < threads; ++t) {
+            try {
+                pool.emplace_back(loop);
+            } catch (...) {
+                break;   // no more threads: the others share the parts
+            }
+        }
+        loop();
+        for (std::thread &t : pool) t.join();
+    }
+    uint64_t total = 0;
+    bool over = false;
+    for (uint64_t o : ones) {
+        total += o;
+        over |= o > part_limit;
+    }
+    if (over || total > limit) {
+        bits.clear();
+        return false;
+    }
+    return true;
+}
+
+// ---- wider symbols: the 4-grams as bytes, hashed to SIEVE_HASH_BITS bits ----
+struct ByteWalk {
+    const Delta &d;
+    std::vector<uint32_t> &bits;
+    uint32_t ones = 0;
+    uint64_t steps = 0;
+    bool over = false;
+
+    void add(uint32_t gram) {
+        uint32_t &w = bits[sieve_hash_word(gram)];
+        const uint32_t bit = 0x80000000u >> (gram & 31);
+        ones += (w & bit) ? 0u : 1u;
+        w |= bit;
+        if (++steps > (1u << 21) || ones > SIEVE_HASH_MAX) over = true;
+    }
+    void all(int depth, uint32_t gram) {   // every extension
+        if (over) return;
+        if (depth == 4) {
+            add(gram);
+            return;
+        }
+        for (int a = 0; a < d.S && !over; ++a) all(depth + 1, gram | (static_cast<uint32_t>(a) << (8 * depth)));
+    }
+    void run(uint16_t q, int depth, uint32_t gram) {
+        if (over) return;
+        if (depth == 4) {
+            add(gram);
+            return;
+        }
+        for (uint32_t e = d.row[q]; e < d.row[q + 1] && !over; ++e) {
+            const uint16_t t = d.tgt[e];
+            const uint32_t g = gram | (static_cast<uint32_t>(d.sym[e]) << (8 * depth));
+            if (t & FINAL_BIT) all(depth + 1, g);
+            else run(t, depth + 1, g);
+        }
+    }
+};
+
+}  // namespace
+
+// The chains of a sieved DFA (see pfsm_internal.h).
+static void build_chains(Machine &m, const Delta &d) {
+    constexpr uint32_t NONE = 0xFFFFFFFFu;
+    std::vector<uint32_t> only(d.Q, NONE);   // symbol << 16 | target of a state with one way on
+    for (int q = 0; q < d.Q; ++q) {
+        if (d.row[q + 1] - d.row[q] == 1) only[q] = (static_cast<uint32_t>(d.sym[d.row[q]]) << 16) | d.tgt[d.row[q]];
+    }
+    m.chain.assign(static_cast<size_t>(d.Q) * 4, 0u);
+    for (int q = 0; q < d.Q; ++q) {
+        uint32_t *c = m.chain.data() + static_cast<size_t>(q) * 4;
+        uint32_t s = static_cast<uint32_t>(q), len = 0;
+        bool fin = false;
+        while (len < 8 && !fin && only[s] != NONE) {
+            c[len >> 2] |= (only[s] >> 16) << (8 * (len & 3));
+            fin = (only[s] & FINAL_BIT) != 0;
+            s = only[s] & 0x7FFFu;
+            ++len;
+        }
+        c[2] = len | (fin ? 256u : 0u);
+        c[3] = s;
+    }
+}
+
+// Bit x of a word to bit 31 - x.
+static uint32_t top_down(uint32_t w) {
+    w = ((w >> 1) & 0x55555555u) | ((w & 0x55555555u) << 1);
+    w = ((w >> 2) & 0x33333333u) | ((w & 0x33333333u) << 2);
+    w = ((w >> 4) & 0x0F0F0F0Fu) | ((w & 0x0F0F0F0Fu) << 4);
+    return __builtin_bswap32(w);
+}
+
+// The strands of a sieved NFA (see sv_strand): parts of the machine that no
+// edge joins once q0 is left.
+static void build_strands(Machine &m) {
+    m.sv_strand.clear();
+    if (m.kind != 1 || m.band.empty()) return;
+    std::vector<int> up(m.Q);
+    for (int q = 0; q < m.Q; ++q) up[q] = q;
+    auto root = [&](int q) {
+        while (up[q] != q) q = up[q] = up[up[q]];
+        return q;
+    };
+    for (int q = 0; q < m.Q; ++q) {
+        if (q != m.q0 && m.band[q] == BAND_CSR) return;
+        for (uint32_t e = m.off[static_cast<size_t>(q) * m.S]; e < m.off[static_cast<size_t>(q + 1) * m.S]; ++e) {
+            const int t = m.tgt[e] & 0x7FFF;
+            if (t == m.q0) return;
+            if (q != m.q0) up[root(q)] = root(t);
+        }
+    }
+    // numbered so that equal neighbours are one strand: a strand's states need
+    // not be consecutive, but those of a set must not alternate
+    m.sv_strand.resize(m.Q);
+    for (int q = 0; q < m.Q; ++q) m.sv_strand[q] = static_cast<uint16_t>(root(q));
+    int last = -1;
+    std::vector<uint8_t> closed(m.Q, 0);
+    for (int q = 0; q < m.Q; ++q) {
+        if (q == m.q0) continue;
+        const int r = m.sv_strand[q];
+        if (r == last) continue;
+        if (closed[r]) {   // two strands alternate: their sets would split wrongly
+            m.sv_strand.clear();
+            return;
+        }
+        if (last >= 0) closed[last] = 1;
+        last = r;
+    }
+}
+
+// Fills m.sv_kind and the sieve's tables. The limits only keep out machines
+// whose bitmaps drop next to nothing: with 1 start in 25 left by the deep
+// bitmap (760 motifs) the sieve still takes 1.74 against the tile kernel's
+// 2.74 ms per 16 MiB, with 1 in 98 (256 motifs) 33 against 66 us.
+void build_sieve(Machine &m) {
+    m.sv_kind = SIEVE_NONE;
+    m.sv_near.clear();
+    m.sv_deep.clear();
+    m.chain.clear();
+    m.sv_strand.clear();
+    const bool dna = m.sbits == 2 && m.sm_m2 == SIEVE_DEEP_M;
+    const bool bytes = m.kind == 0 && m.sbits > 2;
+    if (!dna && !bytes) return;
+    if (dna) {
+        uint64_t direct = 0;
+        for (uint32_t w : m.surv2) direct += static_cast<uint64_t>(__builtin_popcount(w));
+        if (direct * 8 > (1ull << (2 * SIEVE_DEEP_M))) return;
+    }
+    Delta d;
+    flatten(m, d);
+    std::vector<uint16_t> u;
+    if (!sampled_states(d, dna ? SIEVE_DNA_STEP : SIEVE_BYTE_STEP, u)) return;
+    if (dna) {
+        if (!gram_bits(d, u, SIEVE_NEAR_M, (1ull << (2 * SIEVE_NEAR_M)) * 3 / 4, m.sv_near)) return;
+        if (!gram_bits(d, u, SIEVE_DEEP_M, (1ull << (2 * SIEVE_DEEP_M)) / 8, m.sv_deep)) {
+            m.sv_near.clear();
+            return;
+        }
+        for (std::vector<uint32_t> *v : {&m.sv_near, &m.sv_deep})
+            for (uint32_t &w : *v) w = top_down(w);
+        m.sv_kind = SIEVE_DNA;
+        if (m.kind == 0) build_chains(m, d);
+        else build_strands(m);
+        return;
+    }
+    m.sv_near.assign((1u << SIEVE_HASH_BITS) / 32, 0);
+    ByteWalk w{d, m.sv_near};
+    for (uint16_t q : u) w.run(q, 0, 0);
+    if (w.over) {
+        m.sv_near.clear();
+        return;
+    }
+    m.sv_kind = SIEVE_BYTES;
+    build_chains(m, d);
+}
+
+// The third level of a sieved NFA (see L3_SYMS); rebuilt with the records.
+void build_level3(Machine &m) {
+    m.sv_l3.clear();
+    if (m.kind != 1 || m.sv_kind != SIEVE_DNA || m.l2tab.empty() || m.pool2.empty() ||
+        m.pool2.size() > L3_MAX_ROWS)
+        return;
+    Delta d;
+    flatten(m, d);
+    m.sv_l3.assign(m.pool2.size() * (L3_GRAMS / 32), 0u);
+    const std::vector<uint8_t> next = successor_symbols(d);
+    GramWalk w(d, next, L3_SYMS, nullptr, ~0ull, -1);
+    for (size_t at = 0; at < m.pool2.size();) {
+        const uint32_t nm = m.pool2[at] & 0xFFFFu, ns = m.pool2[at] >> 16;
+        uint32_t *to = m.sv_l3.data() + at * (L3_GRAMS / 32);
+        if (nm) {
+            std::fill(to, to + L3_GRAMS / 32, 0xFFFFFFFFu);
+        } else {
+            w.lv[0].assign(m.pool2.begin() + at + 1, m.pool2.begin() + at + 1 + ns);
+            w.bits = to;
+            w.run(0, 0);
+        }
+        at += 1 + nm + ns;
+    }
+}
+
+// The survival bitmap of an NFA over 2-bit symbols (bit set: an instance
+// started at q0 meets a final state within the m symbols or still holds a
+// state after them); false when fewer than half of the m-grams are clear.
+bool survival_bits_dna(const Machine &m, int mm, std::vector<uint32_t> &bits) {
+    Delta d;
+    flatten(m, d);
+    return gram_bits(d, d.start, mm, (1ull << (2 * mm)) / 2, bits);
+}
+
+}  // namespace pfsm
