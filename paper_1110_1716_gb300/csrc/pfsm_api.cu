@@ -430,6 +430,7 @@ void build_survival(Machine &m) {
     if (m2 > m1 && bits(m2, m.surv2)) m.sm_m2 = m2;
     build_sieve(m);
     build_level3(m);
+    build_walk(m);
 }
 
 // ---- residency --------------------------------------------------------------
@@ -439,7 +440,8 @@ size_t device_bytes(const Machine &m) {
     size_t b = align256(m.memo.size() * 2 + 4) + align256(m.surv.size() * 4 + 4) +
                align256(m.surv2.size() * 4 + 4) + align256(m.tail.size() * 2 + 4) +
                align256(m.sv_near.size() * 4) + align256(m.sv_deep.size() * 4) + align256(m.sv_l3.size() * 4) +
-               align256(m.chain.size() * 4) + align256(m.sv_strand.size() * 2 + 4);
+               align256(m.chain.size() * 4) + align256(m.sv_strand.size() * 2 + 4) +
+               align256(m.walk_tab.size() * 4);
     if (m.kind == 0) {
         b += align256(m.dtab.size() * 2 + 4) + align256(m.pool.size() * 4);
     } else {
@@ -569,6 +571,7 @@ static int build_host_image(Machine &m) {
     m.o_l3 = put(m.sv_l3.data(), m.sv_l3.size() * 4, 0);
     m.o_chain = put(m.chain.data(), m.chain.size() * 4, 0);
     m.o_strand = put(m.sv_strand.data(), m.sv_strand.size() * 2, 4);
+    m.o_walk = put(m.walk_tab.data(), m.walk_tab.size() * 4, 0);
     if (m.kind == 0) {
         m.o_tab = put(m.dtab.data(), m.dtab.size() * 2, 4);
         m.o_pool = put(m.pool.data(), m.pool.size() * 4, 0);
@@ -614,6 +617,7 @@ static DevMachine dev_view(const Machine &m, uint8_t *base) {
     dm.sv_near = m.sv_kind ? reinterpret_cast<const uint32_t *>(base + m.o_near) : nullptr;
     dm.chain = m.chain.empty() ? nullptr : reinterpret_cast<const uint4 *>(base + m.o_chain);
     dm.sv_strand = m.sv_strand.empty() ? nullptr : reinterpret_cast<const uint16_t *>(base + m.o_strand);
+    dm.walk = m.walk_tab.empty() ? nullptr : base + m.o_walk;
     dm.sv_l3 = m.sv_l3.empty() ? nullptr : reinterpret_cast<const uint32_t *>(base + m.o_l3);
     dm.sv_deep = m.sv_deep.empty() ? nullptr : reinterpret_cast<const uint32_t *>(base + m.o_deep);
     if (m.kind == 0) {
@@ -963,22 +967,66 @@ void collect_timing(pfsm_ctx *ctx, Slot *slot, int keep) {
     }
 }
 
-// A machine's scans take the sieve (sieve.cu) when it has the tables and all
-// its parameters are the defaults: any other setting shapes the tile kernel,
-// which then runs. (Positions within 256 of 2^32 would wrap in the sieve.)
-// A scan that is being captured takes the tile kernel: the sieve's counters
-// belong to the stream, and a graph may be replayed on others.
-static bool takes_sieve(const pfsm_ctx *ctx, const Machine &m, uint64_t n, cudaStream_t s) {
-    if (!m.sv_kind || m.k <= 0 || ctx->hold_tiles || n >= (1ull << 32) - 256) return false;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return false;
-    }
+// A machine's scans take the sieve (sieve.cu) or the direct scan (walk.cu)
+// when it has the tables for one of them and all its parameters are the
+// defaults: any other setting shapes the tile kernel, which then runs.
+// (Positions within 256 of 2^32 would wrap.) A scan that is being captured
+// takes the tile kernel too: the counters of the other two belong to the
+// stream, and a graph may be replayed on others.
+enum Route { ROUTE_TILES, ROUTE_SIEVE, ROUTE_WALK };
+static Route route_of(const pfsm_ctx *ctx, const Machine &m, uint64_t n, cudaStream_t s) {
+    const bool sieve = m.sv_kind && m.k > 0;
+    if ((!sieve && !m.walks) || ctx->hold_tiles || n == 0 || n >= (1ull << 32) - 256) return ROUTE_TILES;
     pfsm_params d{};
     d.prefix_k = m.params.prefix_k;   // lowered at load where the records did not fit
     fill_defaults(m, d);
-    return memcmp(&d, &m.params, sizeof(d)) == 0;
+    if (d.prefix_k < 0 || memcmp(&d, &m.params, sizeof(d)) != 0) return ROUTE_TILES;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return ROUTE_TILES;
+    }
+    return sieve ? ROUTE_SIEVE : ROUTE_WALK;
+}
+
+// Runs `launch` (a scan whose last kernel leaves the stream's counters zero)
+// with the counters zero: they are cleared before the stream's first such
+// scan and after one that was not wholly launched.
+template <class F>
+static int with_counters(Slot *slot, cudaStream_t s, F &&launch) {
+    if (!slot->sv_ready && cudaMemsetAsync(slot->sv_status, 0, 32, s) != cudaSuccess) return PFSM_E_CUDA;
+    slot->sv_ready = false;
+    if (!launch()) return PFSM_E_CUDA;
+    slot->sv_ready = true;
+    return PFSM_OK;
+}
+
+static int walk_enqueue(pfsm_ctx *ctx, const Machine &m, const uint8_t *text, uint64_t n, uint32_t *out, uint64_t cap,
+                        unsigned long long *status, Slot *slot, cudaStream_t s) {
+    WalkArgs a{};
+    a.text = text;
+    a.n = static_cast<uint32_t>(n);
+    a.Q = m.Q;
+    a.S = m.S;
+    a.q0 = m.q0;
+    a.tab = m.dm.walk;
+    a.tab_bytes = static_cast<uint32_t>(m.walk_tab.size() * 4);
+    for (int w = 0; w < 2; ++w) {
+        a.first[w] = m.walk_first[w];
+        a.finals[w] = m.walk_finals[w];
+    }
+    a.out = out;
+    a.cap = cap;
+    a.status = slot->sv_status;
+    a.status_out = status;
+    a.done = slot->sv_count + 1;
+    // (the scratch of long-lived instances is the candidates' buffer)
+    const bool longs = m.lives && n >= kLongText &&
+                       long_scratch_words(a.n, a.Q) <= static_cast<size_t>(kCandCap) * 2;
+    return with_counters(slot, s, [&] {
+        return (longs ? launch_long(a, reinterpret_cast<uint32_t *>(slot->cand), ctx->nsm, ctx->smem_set, s)
+                      : launch_walk(a, m.kind == 1 || m.lives ? 1 : 0, ctx->nsm, ctx->smem_set, s)) == cudaSuccess;
+    });
 }
 
 // The launches of a sieved scan.
@@ -1011,16 +1059,11 @@ static int sieve_enqueue(pfsm_ctx *ctx, const Machine &m, const uint8_t *text, u
     a.cap = cap;
     a.status = slot->sv_status;
     a.status_out = status;
-    // the sieve, then the kernel that finishes its candidates and leaves the
-    // counters zero; they are cleared here before the stream's first scan
-    // and after one that was not wholly launched
+    // the sieve, then the kernel that finishes its candidates
     auto launch = [&](auto &&finish) {
-        if (!slot->sv_ready && cudaMemsetAsync(slot->sv_status, 0, 32, s) != cudaSuccess) return PFSM_E_CUDA;
-        slot->sv_ready = false;
-        if (launch_sieve(a, m.sv_kind, ctx->nsm, ctx->smem_set, s) != cudaSuccess || finish() != cudaSuccess)
-            return PFSM_E_CUDA;
-        slot->sv_ready = true;
-        return PFSM_OK;
+        return with_counters(slot, s, [&] {
+            return launch_sieve(a, m.sv_kind, ctx->nsm, ctx->smem_set, s) == cudaSuccess && finish() == cudaSuccess;
+        });
     };
     if (m.kind == 0) return launch([&] { return launch_finish_dfa(a, ctx->nsm, s); });
     // the finishing kernel, in half an SM's shared memory: band rows and
@@ -1072,11 +1115,13 @@ int scan_enqueue(pfsm_ctx *ctx, pfsm_aut aut, const uint8_t *text, uint64_t n, u
         slot->ev_head = (slot->ev_head + 1) % kEventRing;
         slot->ev_pending++;
     };
-    if (n > 0 && takes_sieve(ctx, m, n, s)) {
+    const Route route = route_of(ctx, m, n, s);
+    if (route != ROUTE_TILES) {
         time_begin();
         // a scan that is waited for gets its status written to host memory
         if (in_host) *in_host = true;
-        st = sieve_enqueue(ctx, m, text, n, out, cap, in_host ? slot->host_status : status, slot, s);
+        st = (route == ROUTE_SIEVE ? sieve_enqueue : walk_enqueue)(ctx, m, text, n, out, cap,
+                                                                   in_host ? slot->host_status : status, slot, s);
         time_end();
         if (st) return st;
         Machine *mp = &m;
@@ -1252,8 +1297,15 @@ int pfsm_load_dfa(pfsm_ctx *ctx, const int16_t *delta, int32_t Q, int32_t S, int
     if (Q < 1 || Q > 32767 || S < 1 || S > 256) return PFSM_E_INVAL;
     if (q0 < 0 || q0 >= Q || dead < -1 || dead >= Q) return PFSM_E_INVAL;
     if (dead == q0) return PFSM_E_INVAL;
-    for (size_t i = 0; i < (size_t)Q * S; ++i)
-        if (delta[i] < 0 || delta[i] >= Q) return PFSM_E_INVAL;
+    // every entry's code by its target, one pass over the table
+    std::vector<uint16_t> code(Q);
+    for (int t = 0; t < Q; ++t)
+        code[t] = t == dead ? DEAD16 : static_cast<uint16_t>(t | (is_final[t] ? FINAL_BIT : 0));
+    std::vector<uint16_t> dtab((size_t)Q * S + ((size_t)Q * S & 1));
+    for (size_t i = 0; i < (size_t)Q * S; ++i) {
+        if (static_cast<uint16_t>(delta[i]) >= Q) return PFSM_E_INVAL;
+        dtab[i] = code[delta[i]];
+    }
     if (dead >= 0) {
         if (is_final[dead]) return PFSM_E_INVAL;
         for (int a = 0; a < S; ++a)
@@ -1266,12 +1318,7 @@ int pfsm_load_dfa(pfsm_ctx *ctx, const int16_t *delta, int32_t Q, int32_t S, int
     m.q0 = q0;
     m.dead = dead;
     m.fin.assign(is_final, is_final + Q);
-    m.dtab.resize((size_t)Q * S + ((size_t)Q * S & 1));
-    for (size_t i = 0; i < (size_t)Q * S; ++i) {
-        const int t = delta[i];
-        m.dtab[i] = t == dead ? DEAD16
-                              : static_cast<uint16_t>(t | (is_final[t] ? FINAL_BIT : 0));
-    }
+    m.dtab = std::move(dtab);
     return finish_load(ctx, std::move(m), out_id);
 }
 

@@ -53,6 +53,11 @@ struct Machine {
     // NFA with a sieve whose states but q0 all have band rows and none leads
     // back to q0: the weakly connected part (without q0) of every state
     std::vector<uint16_t> sv_strand;
+    // direct scans (walk.cu): taken at all, the table, an NFA's sets
+    // and whether its instances live long (the table is then an NFA's)
+    bool walks = false, lives = false;
+    std::vector<uint32_t> walk_tab;
+    uint32_t walk_first[2] = {0, 0}, walk_finals[2] = {0, 0};
     pfsm_params params{};
     // residency: the device image is built once in pinned host memory and
     // copied in on the scan's stream whenever the machine becomes resident
@@ -62,7 +67,7 @@ struct Machine {
     size_t img_bytes = 0;
     size_t o_memo = 0, o_tail = 0, o_surv = 0, o_surv2 = 0, o_tab = 0, o_off = 0,
            o_tgt = 0, o_pool = 0, o_band = 0, o_eoff = 0, o_etgt = 0, o_l2tab = 0,
-           o_pool2 = 0, o_memox = 0, o_near = 0, o_deep = 0, o_l3 = 0, o_chain = 0, o_strand = 0;   // section offsets
+           o_pool2 = 0, o_memox = 0, o_near = 0, o_deep = 0, o_l3 = 0, o_chain = 0, o_strand = 0, o_walk = 0;   // section offsets
     cudaEvent_t ready = nullptr;      // recorded after the last upload
     bool uploaded = false;            // ... and seen to have completed
     // last use per stream (an event recorded after a launch that read the
@@ -176,6 +181,7 @@ bool build_memo(Machine &m);
 void build_survival(Machine &m);
 void build_sieve(Machine &m);                                              // sieve_tables.cu
 void build_level3(Machine &m);
+void build_walk(Machine &m);
 bool survival_bits_dna(const Machine &m, int mm, std::vector<uint32_t> &bits);
 size_t align256(size_t x);
 void release(pfsm_ctx *ctx, Machine &m);

@@ -223,6 +223,29 @@ struct SieveArgs {
     uint32_t *done;                  // CTAs that ended, zero between scans
 };
 
+// Arguments of the direct scan (walk.cu).
+struct WalkArgs {
+    const uint8_t *text;
+    uint32_t n;
+    int32_t Q, S, q0;
+    const void *tab;            // DFA: uint16 [Q + 1][S], the dead state as state Q; NFA: uint32 [ceil(Q / 8)][S][256][W]
+    uint32_t tab_bytes;
+    uint32_t first[2], finals[2];   // NFA: the set an instance starts with, the final states
+    uint32_t *out;
+    uint64_t cap;
+    unsigned long long *status;      // the stream's own counters, zero between scans
+    unsigned long long *status_out;  // where the scan's status goes
+    uint32_t *done;                  // CTAs that ended, zero between scans
+    // long-lived instances (launch_long fills them): the set that each start
+    // enters the segment after its own with; per segment and state the set
+    // after the segment and the final states met at each of its positions
+    uint32_t *entry, *exit, *met;
+    uint32_t start_ctas;        // CTAs of long_walk that walk starts
+    // filled by the launch
+    uint32_t range;             // starts per warp
+    uint32_t sm_stage;          // shared-memory offset of the match buffers
+};
+
 // Dynamic shared memory of the NFA carry kernel with `nw` warps: band rows
 // (when the scan stages them), then per warp the lane slots, the match
 // staging buffer and (when the scan keeps them in shared memory) the two
@@ -288,6 +311,7 @@ struct DevMachine {
     const uint32_t *sv_near, *sv_deep, *sv_l3;   // sieve tables, or null
     const uint4 *chain;
     const uint16_t *sv_strand;
+    const void *walk;   // direct scan: the table (walk.cu), or null
     // batch: byte offsets of the tables copied into the CTA's shared-memory
     // table arena when this machine's tiles run (kNotStaged: read from
     // global memory; for the survival bitmap: not used)
@@ -344,6 +368,13 @@ constexpr int kFinishThreads = 256;   // of finish_nfa, two CTAs per SM
 uint32_t layout_finish_nfa(ScanArgs &a, uint32_t band_bytes, uint32_t coop_bytes);
 cudaError_t launch_finish_nfa(const ScanArgs &a, const SieveArgs &sv, uint32_t smem, int nsm,
                               std::atomic<uint32_t> &smem_set, cudaStream_t s);
+
+// the direct scan (walk.cu); words of an NFA set
+cudaError_t launch_walk(WalkArgs a, int kind, int nsm, std::atomic<uint32_t> &smem_set, cudaStream_t s);
+uint32_t walk_nfa_words(int Q);
+cudaError_t launch_long(WalkArgs a, uint32_t *scratch, int nsm, std::atomic<uint32_t> &smem_set, cudaStream_t s);
+size_t long_scratch_words(uint32_t n, int Q);
+constexpr uint32_t kLongText = 512;   // symbols from which launch_long is taken
 
 // ---- batch launch helpers (batch_kernels.cu) -----------------------------
 int batch_class(int kind, int sbits, int k, bool tab_smem);

@@ -464,6 +464,26 @@ __device__ __forceinline__ void warp_emit(bool has, uint32_t s, uint32_t e, uint
     sn += c;
 }
 
+// The last CTA of a scan's last kernel to end writes the scan's status out
+// and clears the stream's counters for the next scan on it (which starts
+// after this kernel), so that no scan needs a memset before it. Every thread
+// of the CTA calls this at its end.
+__device__ __forceinline__ void scan_status_out(unsigned long long *status, unsigned long long *status_out,
+                                                uint32_t *done, uint32_t *also) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(done, 1u) == gridDim.x - 1) {
+            __threadfence();
+            status_out[0] = atomicExch(&status[0], 0ull);
+            status_out[1] = atomicExch(&status[1], 0ull);
+            if (also) *also = 0;
+            *done = 0;
+            __threadfence_system();   // (status_out may be host memory)
+        }
+    }
+}
+
 // Direct append for divergent callers (warp-cooperative sets, carried runs).
 template <int OUTW>
 __device__ __forceinline__ void emit_direct(const OView &ov, uint32_t orig, uint32_t s,

@@ -452,23 +452,8 @@ __global__ void __launch_bounds__(512, NEAR_SM ? 2 : 1) sieve_bytes(const SieveA
     if (bad) atomicOr(&a.status[1], ERR_SYMBOL);
 }
 
-// The last CTA of a finishing kernel to end writes the scan's status out and
-// clears the counters for the next scan on this stream (which starts after
-// this kernel), so that no scan needs a memset before it. Every thread of the
-// CTA calls this at its end.
 __device__ __forceinline__ void finish_status_out(const SieveArgs &a) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(a.done, 1u) == gridDim.x - 1) {
-            __threadfence();
-            a.status_out[0] = atomicExch(&a.status[0], 0ull);
-            a.status_out[1] = atomicExch(&a.status[1], 0ull);
-            *a.cand_n = 0;
-            *a.done = 0;
-            __threadfence_system();   // (status_out may be host memory)
-        }
-    }
+    scan_status_out(a.status, a.status_out, a.done, a.cand_n);
 }
 
 // ------------------------------------------------------------ candidates: DFA

@@ -429,6 +429,98 @@ void build_level3(Machine &m) {
     }
 }
 
+// The bitset form of a machine of at most 64 states (see WalkArgs::tab).
+static bool bitset_table(Machine &m, const Delta &d) {
+    const uint32_t W = walk_nfa_words(m.Q), groups = (m.Q + 7) / 8;
+    const size_t words = static_cast<size_t>(groups) * m.S * 256 * W;
+    if (m.Q > 64 || words * 4 > 64 * 1024) return false;
+    m.walk_tab.assign(words, 0u);
+    std::vector<uint64_t> to(static_cast<size_t>(m.Q) * m.S, 0);
+    for (int q = 0; q < m.Q; ++q)
+        for (uint32_t e = d.row[q]; e < d.row[q + 1]; ++e)
+            to[static_cast<size_t>(q) * m.S + d.sym[e]] |= 1ull << (d.tgt[e] & 0x7FFF);
+    for (uint32_t g = 0; g < groups; ++g)
+        for (int a = 0; a < m.S; ++a)
+            for (uint32_t sub = 0; sub < 256; ++sub) {
+                uint64_t t = 0;
+                for (int b = 0; b < 8; ++b)
+                    if ((sub >> b & 1u) && static_cast<int>(8 * g) + b < m.Q)
+                        t |= to[static_cast<size_t>(8 * g + b) * m.S + a];
+                for (uint32_t w = 0; w < W; ++w)
+                    m.walk_tab[((static_cast<size_t>(g) * m.S + a) * 256 + sub) * W + w] =
+                        static_cast<uint32_t>(t >> (32 * w));
+            }
+    uint64_t first = 0, fin = 0;
+    for (uint16_t q : d.start) first |= 1ull << q;
+    for (int q = 0; q < m.Q; ++q)
+        if (m.fin[q]) fin |= 1ull << q;
+    for (int w = 0; w < 2; ++w) {
+        m.walk_first[w] = static_cast<uint32_t>(first >> (32 * w));
+        m.walk_finals[w] = static_cast<uint32_t>(fin >> (32 * w));
+    }
+    return true;
+}
+
+// Whether 1 in 16 or more of the instances live for 256 uniform symbols
+// (tried on 256 fixed texts).
+static bool lives_long(const Machine &m, const Delta &d) {
+    std::vector<uint64_t> to(static_cast<size_t>(m.Q) * m.S, 0);
+    for (int q = 0; q < m.Q; ++q)
+        for (uint32_t e = d.row[q]; e < d.row[q + 1]; ++e)
+            to[static_cast<size_t>(q) * m.S + d.sym[e]] |= 1ull << (d.tgt[e] & 0x7FFF);
+    uint64_t first = 0, x = 0x9E3779B97F4A7C15ull;
+    for (uint16_t q : d.start) first |= 1ull << q;
+    int alive = 0;
+    for (int t = 0; t < 256; ++t) {
+        uint64_t s = first;
+        for (int j = 0; j < 256 && s; ++j) {
+            x = x * 6364136223846793005ull + 1442695040888963407ull;
+            const uint32_t a = static_cast<uint32_t>(((x >> 32) * static_cast<uint64_t>(m.S)) >> 32);
+            uint64_t n = 0;
+            for (; s; s &= s - 1) n |= to[static_cast<size_t>(__builtin_ctzll(s)) * m.S + a];
+            s = n;
+        }
+        alive += s != 0;
+    }
+    return alive >= 16;
+}
+
+// Whether the machine's scans walk every start (walk.cu), and the tables for
+// it. DFAs: tables that L1 can hold, where the shallow survival bitmap would
+// pass at least 1 start in 8. NFAs: at most 64 states, tables of at most 64 KB.
+void build_walk(Machine &m) {
+    m.walks = m.lives = false;
+    m.walk_tab.clear();
+    if (m.sv_kind != SIEVE_NONE) return;
+    if (m.kind == 0) {
+        if (static_cast<size_t>(m.Q) * m.S * 2 > 160 * 1024) return;
+        uint64_t ones = 0;
+        for (uint32_t w : m.surv) ones += static_cast<uint64_t>(__builtin_popcount(w));
+        if (!m.surv.empty() && ones * 8 < (1ull << (m.sm_m * m.sbits))) return;
+    } else if (m.Q > 64) {
+        return;
+    }
+    Delta d;
+    if (m.Q <= 64) {
+        flatten(m, d);
+        m.lives = lives_long(m, d);
+        if ((m.kind == 1 || m.lives) && bitset_table(m, d)) {
+            m.walks = true;
+            return;
+        }
+        m.lives = false;
+        if (m.kind == 1) return;
+    }
+    // a DFA's table with the dead state as state Q, a row that leads to itself
+    const size_t cells = static_cast<size_t>(m.Q) * m.S;
+    std::vector<uint16_t> t(cells + m.S + 1, static_cast<uint16_t>(m.Q));
+    for (size_t i = 0; i < cells; ++i)
+        if (m.dtab[i] != DEAD16) t[i] = m.dtab[i];
+    m.walk_tab.assign((cells + m.S + 1) / 2, 0u);
+    memcpy(m.walk_tab.data(), t.data(), m.walk_tab.size() * 4);
+    m.walks = true;
+}
+
 // The survival bitmap of an NFA over 2-bit symbols (bit set: an instance
 // started at q0 meets a final state within the m symbols or still holds a
 // state after them); false when fewer than half of the m-grams are clear.
