@@ -29,6 +29,15 @@ constexpr uint32_t kMinArena = 8192;     // smallest table arena worth a class s
 constexpr int kUnitTilesMax = 8;        // tiles per work unit, at most
 constexpr int kCarryCtr = 15;           // counter word holding the carry count
 constexpr uint32_t kAllClasses = (1u << kBatchClasses) - 1;
+constexpr int kFlatCtr = 16;            // counter words holding the flat batches' candidate counts
+// symbols of a batch's sieved texts from which the kernel with the near
+// bitmaps in shared memory is taken (each of its CTAs copies 128 KB per
+// machine it meets). 64 texts, 4 motif sets, whole calls: 4 MiB 64 us (62
+// without), 8 MiB 63 (74), 64 MiB 138 (197); bytes 50 us (50), 50 (50), 62 (75)
+constexpr uint64_t kFlatBig = 8ull << 20;
+// least cost of a group of machines, 25 us of the whole chip: every group
+// copies its bitmaps and starts its warps anew (5 us)
+constexpr uint64_t kFlatGroupCost = 306000;
 
 struct BatchGraph {
     cudaGraphExec_t exec = nullptr;
@@ -47,6 +56,9 @@ struct BatchState {
     unsigned long long *status = nullptr;       // device: total, errors, per-job counts
     unsigned long long *host_status = nullptr;  // pinned copy of status
     uint32_t *carry = nullptr;
+    uint8_t *flat_dev = nullptr;      // flat batches: jobs | machines, and their pinned staging
+    uint8_t *flat_host = nullptr;
+    uint4 *cand = nullptr;            //   candidates, two lists of kFlatCand
     uint32_t *coop = nullptr;         // warp-wide NFA bitsets of every NFA class
     size_t coop_words = 0;
     cudaEvent_t staged = nullptr;     // previous staging copy has been consumed
@@ -73,6 +85,9 @@ static void state_free(BatchState *b) {
     cudaFree(b->dev);
     cudaFree(b->ctr);
     cudaFree(b->coop);
+    cudaFree(b->flat_dev);
+    cudaFree(b->cand);
+    cudaFreeHost(b->flat_host);
     cudaFreeHost(b->host);
     cudaFreeHost(b->host_status);
     delete b;
@@ -98,6 +113,11 @@ static int state_reserve(pfsm_ctx *ctx, cudaStream_t s, size_t njobs, size_t nma
             cudaGetLastError();
             return PFSM_E_CUDA;
         }
+        if (cudaMalloc(&b->cand, 2ull * kFlatCand * sizeof(uint4)) != cudaSuccess) {
+            cudaGetLastError();
+            b->cand = nullptr;
+            return PFSM_E_NOMEM;
+        }
     }
     if (njobs <= b->cap_jobs && nmachs <= b->cap_machs) {
         *out = b;
@@ -112,6 +132,10 @@ static int state_reserve(pfsm_ctx *ctx, cudaStream_t s, size_t njobs, size_t nma
     cudaFree(b->ctr);
     cudaFreeHost(b->host);
     cudaFreeHost(b->host_status);
+    cudaFree(b->flat_dev);
+    cudaFreeHost(b->flat_host);
+    b->flat_dev = nullptr;
+    b->flat_host = nullptr;
     b->dev = nullptr;
     b->ctr = nullptr;
     b->host = nullptr;
@@ -125,6 +149,8 @@ static int state_reserve(pfsm_ctx *ctx, cudaStream_t s, size_t njobs, size_t nma
     if (cudaMalloc(&b->dev, b->block_bytes) != cudaSuccess ||
         cudaMalloc(&b->ctr, ctr_bytes) != cudaSuccess ||
         cudaMallocHost(&b->host, b->block_bytes) != cudaSuccess ||
+        cudaMalloc(&b->flat_dev, b->block_bytes) != cudaSuccess ||
+        cudaMallocHost(&b->flat_host, b->block_bytes) != cudaSuccess ||
         cudaMallocHost(&b->host_status, (b->cap_jobs + 2) * 8) != cudaSuccess) {
         cudaGetLastError();
         b->cap_jobs = b->cap_machs = 0;
@@ -236,7 +262,19 @@ static int place_tables(const Machine &m, uint32_t arena, int warps, DevMachine 
     return batch_class(m.kind, m.sbits, m.k, m.kind == 0 && d.a_tab != kNotStaged);
 }
 
+// The flat part of a batch (flat_batch.cu).
+struct FlatPlan {
+    std::vector<BatchJob> jobs;
+    std::vector<DevMachine> machs;
+    uint32_t job_lo[FLAT_CLASSES] = {}, job_hi[FLAT_CLASSES] = {};
+    uint64_t steps[FLAT_CLASSES] = {};
+    uint64_t group_end[kFlatGroups] = {};
+    uint32_t groups = 0;
+    bool big = false;
+};
+
 struct BatchPlan {
+    FlatPlan flat;
     std::vector<BatchJob> jobs;
     std::vector<DevMachine> machs;
     std::vector<Machine *> used;            // the machines the batch reads
@@ -245,6 +283,96 @@ struct BatchPlan {
     uint32_t nunits[kBatchClasses] = {}, unit_tiles[kBatchClasses] = {};
     int32_t wq[kBatchClasses] = {};         // NFA: widest bitset kept in global scratch (words)
 };
+
+// The class of a machine whose texts run flat, or -1: machines with sieve or
+// direct-scan tables and nothing but default parameters (other settings shape
+// the class kernels, which then run).
+static int flat_class(const pfsm_ctx *ctx, const Machine &m) {
+    if (ctx->batch_threads || ctx->batch_ctas || ctx->batch_tile != kBatchTile || !default_params(m)) return -1;
+    if (m.sv_kind == SIEVE_DNA && m.k > 0 && (m.kind == 0 || m.sv_lean)) return FLAT_DNA;
+    if (m.sv_kind == SIEVE_BYTES && m.k > 0) return FLAT_BYTES;
+    return m.walks ? FLAT_WALK : -1;
+}
+
+// Groups of machines (in `order`) that the whole chip scans one after the
+// other, in flat_cost units.
+static void plan_groups(const std::vector<uint32_t> &order, FlatPlan &pl) {
+    uint64_t total = 0, base = 0;
+    for (int c = 0; c < FLAT_CLASSES; ++c) total += pl.steps[c] * flat_cost(c, pl.big);
+    const uint64_t least = pl.big ? std::max<uint64_t>(kFlatGroupCost, total / (kFlatGroups - 1) + 1) : total;
+    uint64_t from = 0;
+    int last = FLAT_DNA;
+    for (uint32_t s : order) {
+        const int c = pl.machs[s].flat;
+        for (; last < c; ++last) base += pl.steps[last] * flat_cost(last, pl.big);
+        const uint64_t end = base + pl.machs[s].flat_end * static_cast<uint64_t>(flat_cost(c, pl.big));
+        if (end - from >= least && total - end >= least) {
+            pl.group_end[pl.groups++] = end;
+            from = end;
+        }
+    }
+    pl.group_end[pl.groups++] = total;
+}
+
+// Cuts the flat texts (jobs of machine slots with a class in flat_of) into
+// steps, sorted by class, machine and the caller's order.
+static int plan_flat(const pfsm_job *jobs, int32_t k, const std::vector<uint32_t> &job_slot,
+                     const std::vector<int> &flat_of, const std::vector<Machine *> &machines, FlatPlan &pl) {
+    uint64_t sieved = 0;
+    std::vector<uint32_t> first(flat_of.size(), 0), order;
+    for (int32_t i = 0; i < k; ++i) {
+        const int c = flat_of[job_slot[i]];
+        if (c < 0) continue;
+        first[job_slot[i]]++;
+        if (c != FLAT_WALK) sieved += jobs[i].n;
+    }
+    pl.big = sieved >= kFlatBig;
+    uint32_t at = 0;
+    for (int c = 0; c < FLAT_CLASSES; ++c) {
+        pl.job_lo[c] = at;
+        for (size_t s = 0; s < flat_of.size(); ++s) {
+            if (flat_of[s] != c) continue;
+            const uint32_t n = first[s];
+            first[s] = at;
+            at += n;
+            order.push_back(static_cast<uint32_t>(s));
+        }
+        pl.job_hi[c] = at;
+    }
+    pl.jobs.resize(at);
+    pl.machs.resize(flat_of.size());
+    for (int32_t i = 0; i < k; ++i) {
+        const uint32_t s = job_slot[i];
+        const int c = flat_of[s];
+        if (c < 0) continue;
+        BatchJob &b = pl.jobs[first[s]++];
+        b.text = jobs[i].text;
+        b.n = static_cast<uint32_t>(jobs[i].n);
+        b.mach = s;
+        b.orig = static_cast<uint32_t>(i);
+        const uint64_t step = flat_step(c, pl.big);
+        // (the sieves' steps begin at 16-byte boundaries of the address space)
+        const uint64_t shift = c == FLAT_WALK ? 0 : reinterpret_cast<uintptr_t>(b.text) & 15;
+        b.ntiles = b.n ? static_cast<uint32_t>((b.n + shift + step - 1) / step) : 0u;
+    }
+    for (uint32_t s : order) {
+        DevMachine &d = pl.machs[s];
+        d = machines[s]->dm;
+        d.flat = flat_of[s];
+    }
+    for (int c = 0; c < FLAT_CLASSES; ++c) {
+        for (uint32_t j = pl.job_lo[c]; j < pl.job_hi[c]; ++j) {
+            BatchJob &b = pl.jobs[j];
+            const uint64_t steps = b.ntiles ? static_cast<uint64_t>(b.ntiles) + flat_pad(pl.big) : 0u;
+            if (pl.steps[c] + steps >= (1ull << 31)) return PFSM_E_INVAL;
+            b.unit_begin = static_cast<uint32_t>(pl.steps[c]);
+            pl.steps[c] += steps;
+            pl.machs[b.mach].flat_end = static_cast<uint32_t>(pl.steps[c]);
+        }
+    }
+    plan_groups(order, pl);
+    return PFSM_OK;
+}
 
 // Validate the jobs, make their machines resident, classify them and cut
 // every class's texts into work units.
@@ -280,6 +408,23 @@ static int plan_batch(pfsm_ctx *ctx, const pfsm_job *jobs, int32_t k, BatchPlan 
         int st = make_resident(ctx, id, ctx->machines[id], s);
         if (st) return st;
     }
+    // machines whose texts run flat, and the texts that keep to the classes
+    std::vector<int> flat_of(ids.size());
+    int32_t rest = k;
+    for (size_t i = 0; i < ids.size(); ++i) {
+        Machine &m = ctx->machines[ids[i]];
+        pl.used.push_back(&m);
+        flat_of[i] = flat_class(ctx, m);
+    }
+    for (int32_t i = 0; i < k; ++i) {
+        if (jobs[i].n >= (1ull << 32) - 256) flat_of[job_slot[i]] = -1;   // positions would wrap
+    }
+    for (int32_t i = 0; i < k; ++i) rest -= flat_of[job_slot[i]] >= 0;
+    if (rest < k) {
+        int fs = plan_flat(jobs, k, job_slot, flat_of, pl.used, pl.flat);
+        if (fs) return fs;
+    }
+    if (rest == 0) return PFSM_OK;
     // the DFA classes share one shape (threads, arena), as do the NFA classes
     int st = class_shape(ctx, 0);
     if (!st) st = class_shape(ctx, 6);
@@ -292,7 +437,6 @@ static int plan_batch(pfsm_ctx *ctx, const pfsm_job *jobs, int32_t k, BatchPlan 
         Machine &m = ctx->machines[ids[i]];
         DevMachine d = m.dm;
         const BatchShape &sh = ctx->batch_shape[m.kind == 1 ? 6 : 0];
-        pl.used.push_back(&m);
         cls_of[i] = place_tables(m, sh.arena, sh.threads / 32, d);
         if (m.kind == 1 && d.a_coop == kNotStaged) pl.wq[cls_of[i]] = std::max(pl.wq[cls_of[i]], d.Wq);
         pl.machs.push_back(d);
@@ -306,7 +450,8 @@ static int plan_batch(pfsm_ctx *ctx, const pfsm_job *jobs, int32_t k, BatchPlan 
         return cls_of[x] != cls_of[y] ? cls_of[x] < cls_of[y] : x < y;
     });
     std::vector<uint32_t> first(ids.size() + 1, 0);
-    for (int32_t i = 0; i < k; ++i) first[job_slot[i] + 1]++;
+    for (int32_t i = 0; i < k; ++i)
+        if (flat_of[job_slot[i]] < 0) first[job_slot[i] + 1]++;
     {
         std::vector<uint32_t> count(first.begin() + 1, first.end());
         uint32_t at = 0;
@@ -315,10 +460,12 @@ static int plan_batch(pfsm_ctx *ctx, const pfsm_job *jobs, int32_t k, BatchPlan 
             at += count[sl];
         }
     }
-    std::vector<uint32_t> key(static_cast<size_t>(k));   // job indices in (class, slot, index) order
-    for (int32_t i = 0; i < k; ++i) key[first[job_slot[i]]++] = static_cast<uint32_t>(i);
+    std::vector<uint32_t> key(static_cast<size_t>(rest));   // job indices in (class, slot, index) order
+    for (int32_t i = 0; i < k; ++i)
+        if (flat_of[job_slot[i]] < 0) key[first[job_slot[i]]++] = static_cast<uint32_t>(i);
     uint64_t tiles_of[kBatchClasses] = {};
     for (int32_t i = 0; i < k; ++i) {
+        if (flat_of[job_slot[i]] >= 0) continue;
         const int c = cls_of[job_slot[i]];
         tiles_of[c] += (jobs[i].n + ctx->batch_shape[c].layout.tile - 1) / ctx->batch_shape[c].layout.tile;
     }
@@ -329,8 +476,8 @@ static int plan_batch(pfsm_ctx *ctx, const pfsm_job *jobs, int32_t k, BatchPlan 
         pl.unit_tiles[c] = static_cast<uint32_t>(std::min<uint64_t>(kUnitTilesMax, std::max<uint64_t>(1, per)));
     }
     int cur = -1;
-    pl.jobs.reserve(static_cast<size_t>(k));
-    for (int32_t r = 0; r < k; ++r) {
+    pl.jobs.reserve(static_cast<size_t>(rest));
+    for (int32_t r = 0; r < rest; ++r) {
         const int32_t x = static_cast<int32_t>(key[r]);
         const pfsm_job &j = jobs[x];
         const uint32_t slot = job_slot[x];
@@ -420,9 +567,75 @@ static int batch_enqueue(pfsm_ctx *ctx, const pfsm_job *jobs, int32_t k, pfsm_bm
     ctx->epoch++;
     if (st) return st;
     BatchState *b = nullptr;
-    st = state_reserve(ctx, s, std::max<size_t>(1, pl.jobs.size()), std::max<size_t>(1, pl.machs.size()), &b);
+    // (the status block has one count per job of the caller)
+    st = state_reserve(ctx, s, std::max<size_t>(1, static_cast<size_t>(k)),
+                       std::max<size_t>(1, pl.used.size()), &b);
     if (st) return st;
-    if (b->staged_pending) cudaEventSynchronize(b->staged);   // staging buffer is free again
+    if (b->staged_pending) cudaEventSynchronize(b->staged);   // staging buffers are free again
+    b->staged_pending = false;
+    int ev = -1;
+    Slot *slot = ctx->timing ? get_slot(ctx, s) : nullptr;
+    auto time_begin = [&]() {
+        if (!slot) return;
+        collect_timing(ctx, slot, kEventRing - 1);
+        ev = slot->ev_head;
+        cudaEventRecord(slot->ev[2 * ev], s);
+    };
+    auto time_end = [&]() {
+        if (ev < 0) return;
+        cudaEventRecord(slot->ev[2 * ev + 1], s);
+        slot->ev_head = (slot->ev_head + 1) % kEventRing;
+        slot->ev_pending++;
+    };
+    const bool flat = !pl.flat.jobs.empty();
+    if (flat) {
+        // one copy: the flat jobs, then their machines
+        const size_t jb = align256(pl.flat.jobs.size() * sizeof(BatchJob));
+        memcpy(b->flat_host, pl.flat.jobs.data(), pl.flat.jobs.size() * sizeof(BatchJob));
+        memcpy(b->flat_host + jb, pl.flat.machs.data(), pl.flat.machs.size() * sizeof(DevMachine));
+        if (cudaMemcpyAsync(b->flat_dev, b->flat_host, jb + pl.flat.machs.size() * sizeof(DevMachine),
+                            cudaMemcpyHostToDevice, s) != cudaSuccess)
+            return PFSM_E_CUDA;
+    }
+    // the flat kernels, after the classes when the batch has both (those
+    // clear the status block)
+    auto launch_flat_part = [&]() -> int {
+        FlatArgs f{};
+        f.jobs = reinterpret_cast<const BatchJob *>(b->flat_dev);
+        f.machs = reinterpret_cast<const DevMachine *>(b->flat_dev + align256(pl.flat.jobs.size() * sizeof(BatchJob)));
+        for (int c = 0; c < FLAT_CLASSES; ++c) {
+            f.job_lo[c] = pl.flat.job_lo[c];
+            f.job_hi[c] = pl.flat.job_hi[c];
+            f.steps[c] = pl.flat.steps[c];
+        }
+        std::copy(pl.flat.group_end, pl.flat.group_end + kFlatGroups, f.group_end);
+        f.groups = pl.flat.groups;
+        f.out = reinterpret_cast<uint32_t *>(out);
+        f.cap = cap;
+        f.status = b->status;
+        f.job_counts = b->status + 2;
+        f.cand[0] = b->cand;
+        f.cand[1] = b->cand + kFlatCand;
+        f.cand_n = b->ctr + kFlatCtr;
+        f.cand_cap = ctx->test_carry_cap ? std::min(kFlatCand, ctx->test_carry_cap) : kFlatCand;
+        return launch_flat(f, pl.flat.big, ctx->nsm, ctx->smem_set, s) == cudaSuccess ? PFSM_OK : PFSM_E_CUDA;
+    };
+    if (pl.jobs.empty()) {
+        // nothing for the class kernels: clear the counters and the counts
+        if (cudaMemsetAsync(b->ctr, 0, 256 + (static_cast<size_t>(k) + 2) * 8, s) != cudaSuccess) return PFSM_E_CUDA;
+        time_begin();
+        if (flat) {
+            cudaEventRecord(b->staged, s);
+            b->staged_pending = true;
+            st = launch_flat_part();
+            if (st) return st;
+        }
+        time_end();
+        st = mark_use(ctx, s, pl.used.data(), pl.used.size());
+        if (st) return st;
+        *bs = b;
+        return PFSM_OK;
+    }
     // warp bitsets of the NFA classes, one region per class
     size_t coop_need = 0, coop_off[kBatchClasses] = {};
     for (int c = 6; c < kBatchClasses; ++c) {
@@ -471,21 +684,15 @@ static int batch_enqueue(pfsm_ctx *ctx, const pfsm_job *jobs, int32_t k, pfsm_bm
     cudaGraphExec_t exec = nullptr;
     st = graph_for(ctx, b, kAllClasses, &exec);
     if (st) return st;
-    int ev = -1;
-    Slot *slot = ctx->timing ? get_slot(ctx, s) : nullptr;
-    if (slot) {
-        collect_timing(ctx, slot, kEventRing - 1);
-        ev = slot->ev_head;
-        cudaEventRecord(slot->ev[2 * ev], s);
-    }
+    time_begin();
     if (cudaGraphLaunch(exec, s) != cudaSuccess) return PFSM_E_CUDA;
+    if (flat) {
+        st = launch_flat_part();
+        if (st) return st;
+    }
+    time_end();
     st = mark_use(ctx, s, pl.used.data(), pl.used.size());
     if (st) return st;
-    if (slot) {
-        cudaEventRecord(slot->ev[2 * ev + 1], s);
-        slot->ev_head = (slot->ev_head + 1) % kEventRing;
-        slot->ev_pending++;
-    }
     *bs = b;
     return PFSM_OK;
 }

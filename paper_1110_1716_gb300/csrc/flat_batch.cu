@@ -1,0 +1,469 @@
+// Flat batches: the texts of a batch whose machines the sieve (sieve.cuh) or
+// the direct scan (walk.cuh) takes, in two launches whatever the number of
+// texts and machines.
+//
+// `flat_front` runs over the steps of all texts, sorted by class (2-bit
+// sieve, byte sieve, direct scan) and machine: every CTA takes an equal share
+// of their cost and every warp consecutive steps of it, so no step is claimed
+// and nobody waits. `flat_finish` runs the sieves' candidates of all texts,
+// each lane with its own text and machine.
+//
+// Measured, whole calls, against one tile kernel per class and shape plus the
+// carry kernel in a graph: 64 requests over 24 machines 450 -> 69 us, of which
+// flat_front takes 25 and flat_finish 12 (chains of dependent loads: a request
+// is a few steps long); 10,000 texts over 16 machines, 1.1 GB, 4.7 -> 1.28 ms;
+// 8 machines over 8 MiB each 350 -> 109 us. With full warps of steps flat_front
+// is bound like the single-text kernels: 64 MiB of DNA 72 us against 60,
+// 256 MiB of bytes 61 us against 50; the rest is the start of a share (its
+// job, arguments and first loads) and arguments read from shared memory
+// instead of the constant bank. Steps of 512 bytes of DNA (1 KB, as the
+// single-text kernel takes: spills beside the arguments, 80 us); the text loop
+// as a call of its own 87 us.
+#include <algorithm>
+#include <atomic>
+
+#include "sieve.cuh"
+#include "walk.cuh"
+
+namespace pfsm {
+
+constexpr uint32_t kFlatStage = 96;   // direct scans: staged matches per warp and half
+
+// Last job of [lo, hi) whose first step is <= x (every lane calls it).
+__device__ __forceinline__ uint32_t flat_job(const BatchJob *jobs, uint32_t lo, uint32_t hi, uint32_t x, int lane) {
+    while (hi - lo > 1) {
+        const uint32_t each = (hi - lo + 31) / 32, at = lo + lane * each;
+        const uint32_t m = __ballot_sync(FULLMASK, at < hi && jobs[at].unit_begin <= x);
+        const uint32_t r = 31 - __clz(m);   // lane 0 always holds (lo's first step is <= x)
+        lo += r * each;
+        hi = min(hi, lo + each);
+    }
+    return lo;
+}
+
+// A warp's arguments for one text: the building blocks take them by reference.
+union FlatWarp {
+    SieveArgs sieve;
+    WalkArgs walk;
+};
+
+// Steps [s0, s1) of class CLS by the calling warp.
+template <int CLS, bool BIG>
+__device__ __forceinline__ void flat_steps(const FlatArgs &A, FlatWarp &wa, uint32_t s0, uint32_t s1, int wid, int lane,
+                                           uint64_t pol_keep) {
+    if (s0 >= s1) return;
+    // the near bitmap at offset 0 of the shared memory, then the warps' lists;
+    // direct scans have their match buffers there instead
+    const uint8_t *near = pfsm_dyn_smem;
+    constexpr uint32_t lists = BIG && CLS != FLAT_WALK ? (1u << (2 * SIEVE_NEAR_M)) / 8 : 0u;
+    constexpr uint32_t each = CLS == FLAT_WALK ? 2 * kFlatStage * 16 : kSieveList * 16;
+    uint8_t *own = pfsm_dyn_smem + lists + wid * each;
+    uint32_t *list = reinterpret_cast<uint32_t *>(own);
+    uint2 *list2 = reinterpret_cast<uint2 *>(list + kSieveList * 2);
+    uint32_t cnt = 0, cnt2 = 0;
+    bool bad = false;
+    WalkOut<4, kFlatStage> out{reinterpret_cast<uint32_t *>(own), 0u, 0u, 0u, 0ull};
+    for (uint32_t j = flat_job(A.jobs, A.job_lo[CLS], A.job_hi[CLS], s0, lane); s0 < s1; ++j) {
+        const BatchJob &J = A.jobs[j];
+        const DevMachine &M = A.machs[J.mach];
+        const uint32_t b0 = s0 - J.unit_begin, b1 = min(J.ntiles, b0 + (s1 - s0));
+        s0 = min(s1, J.unit_begin + J.ntiles + flat_pad(BIG));
+        if (b0 >= b1) continue;   // an empty text, or the padding after one
+        __syncwarp();
+        if (lane == 0) {
+            if (CLS == FLAT_WALK) {
+                WalkArgs &a = wa.walk;
+                a.text = J.text;
+                a.n = J.n;
+                a.Q = M.Q;
+                a.S = M.S;
+                a.q0 = M.q0;
+                a.tab = M.walk;
+                for (int w = 0; w < 2; ++w) {
+                    a.first[w] = M.walk_first[w];
+                    a.finals[w] = M.walk_finals[w];
+                }
+                a.out = A.out;
+                a.cap = A.cap;
+                a.status = A.status;
+                a.job_counts = A.job_counts;
+                a.orig = J.orig;
+            } else {
+                SieveArgs &a = wa.sieve;
+                a.text = J.text;
+                a.n = J.n;
+                a.S = M.S;
+                a.near = M.sv_near;
+                a.deep = M.sv_deep;
+                a.surv2 = CLS == FLAT_DNA || (M.sbits == 8 && M.surv2_m == 3) ? M.surv2 : nullptr;
+                a.memox = M.memox;
+                a.l2tab = M.l2tab;
+                a.l3 = M.kind == 1 ? M.sv_l3 : nullptr;
+                a.k = M.k;
+                a.min_match = M.min_match;
+                a.job = j;
+                a.cand = reinterpret_cast<uint2 *>(A.cand[M.kind]);
+                a.cand_n = A.cand_n + M.kind;
+                a.cand_cap = A.cand_cap;
+            }
+        }
+        __syncwarp();
+        if (CLS == FLAT_DNA) {
+            dna_steps<BIG, 1, true>(wa.sieve, near, list, list2, b0, b1, 1, cnt, cnt2, bad, lane, pol_keep);
+            sieve_rest<SIEVE_DNA, true>(wa.sieve, list, list2, cnt, cnt2, lane, pol_keep);
+        } else if (CLS == FLAT_BYTES) {
+            byte_steps<BIG, true>(wa.sieve, near, list, b0, b1, 1, cnt, bad, lane, pol_keep);
+            sieve_rest<SIEVE_BYTES, true>(wa.sieve, list, list2, cnt, cnt2, lane, pol_keep);
+        } else {
+            constexpr uint32_t R = flat_step(FLAT_WALK, BIG);
+            const uint32_t head = b0 * R;
+            const uint32_t stop = b1 == J.ntiles ? J.n : b1 * R;
+            const uint8_t *tab = reinterpret_cast<const uint8_t *>(wa.walk.tab);
+            const int words = M.walk_words;
+            if (words == 0) walk_range<WalkDfa<false>, false>(wa.walk, tab, head, stop, out, bad, lane);
+            else if (words == 1) walk_range<WalkNfa<1>, false>(wa.walk, tab, head, stop, out, bad, lane);
+            else walk_range<WalkNfa<2>, false>(wa.walk, tab, head, stop, out, bad, lane);
+            out.finish(wa.walk, lane);
+        }
+    }
+    if (bad) atomicOr(&A.status[1], ERR_SYMBOL);
+}
+
+// BIG: one CTA of 32 warps per SM with the machine's near bitmap in shared
+// memory (copied again where the CTA's share passes to the next machine);
+// otherwise small CTAs that read the bitmaps through L1 and L2.
+//
+// The CTAs share the steps group by group: the deep bitmaps of the machines
+// they test with at one time have to stay in L2 (8 MB each, read at random).
+// 10,000 texts over 8 motif and 8 signature sets: all machines at once 1.63 ms
+// for the kernel, 1.16 ms with two sets to a group, 0.90 ms with one.
+template <bool BIG>
+__global__ void __launch_bounds__(BIG ? 1024 : 128, 1) flat_front(const __grid_constant__ FlatArgs A) {
+    __shared__ FlatWarp warps[BIG ? 32 : 4];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const uint32_t nw = blockDim.x >> 5;
+    const uint64_t pol_keep = policy_evict_last();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    uint64_t from = 0;
+    for (uint32_t g = 0; g < A.groups; ++g) {
+        // this CTA's share of the group's cost, as steps of each class
+        const uint64_t part = A.group_end[g] - from;
+        const uint64_t x0 = from + part * blockIdx.x / gridDim.x, x1 = from + part * (blockIdx.x + 1) / gridDim.x;
+        from += part;
+        uint64_t base = 0;
+#pragma unroll
+        for (int c = 0; c < FLAT_CLASSES; ++c) {
+            const uint32_t cost = flat_cost(c, BIG);
+            auto step_at = [&](uint64_t x) -> uint32_t {
+                return static_cast<uint32_t>(x <= base ? 0 : min(A.steps[c], (x - base + cost - 1) / cost));
+            };
+            uint32_t s0 = step_at(x0);
+            const uint32_t s1 = step_at(x1);
+            base += A.steps[c] * cost;
+            while (s0 < s1) {
+                uint32_t e = s1;
+                if (BIG && c != FLAT_WALK) {
+                    // one machine at a time: its near bitmap, then its steps
+                    const BatchJob &J = A.jobs[flat_job(A.jobs, A.job_lo[c], A.job_hi[c], s0, lane)];
+                    const DevMachine &M = A.machs[J.mach];
+                    e = min(s1, M.flat_end);
+                    __syncthreads();   // every warp is done with the bitmap before
+                    if (c == FLAT_DNA) stage_near<(1u << (2 * SIEVE_NEAR_M)) / 8, 1024>(pfsm_dyn_smem, M.sv_near, tid);
+                    else stage_near<(1u << SIEVE_HASH_BITS) / 8, 1024>(pfsm_dyn_smem, M.sv_near, tid);
+                    __syncthreads();
+                } else if (BIG) {
+                    __syncthreads();   // the match buffers lie where the bitmap was
+                }
+                const uint32_t per = (e - s0 + nw - 1) / nw;
+                const uint32_t w0 = min(e, s0 + wid * per), w1 = min(e, w0 + per);
+                if (c == FLAT_DNA) flat_steps<FLAT_DNA, BIG>(A, warps[wid], w0, w1, wid, lane, pol_keep);
+                else if (c == FLAT_BYTES) flat_steps<FLAT_BYTES, BIG>(A, warps[wid], w0, w1, wid, lane, pol_keep);
+                else flat_steps<FLAT_WALK, BIG>(A, warps[wid], w0, w1, wid, lane, pol_keep);
+                s0 = e;
+            }
+        }
+    }
+}
+
+// ------------------------------------------------------------ candidates
+// The match (start, end, st) of every lane with `has`, to the output and the
+// counts.
+__device__ __forceinline__ void flat_emit(const FlatArgs &A, bool has, uint32_t orig, uint32_t start, uint32_t end,
+                                          uint32_t st, int lane) {
+    const uint32_t m = __ballot_sync(FULLMASK, has);
+    if (m == 0) return;
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(&A.status[0], static_cast<unsigned long long>(__popc(m)));
+    base = __shfl_sync(FULLMASK, base, 0) + __popc(m & lanemask_lt());
+    if (has) {
+        atomicAdd(&A.job_counts[orig], 1ull);
+        if (base < A.cap) reinterpret_cast<uint4 *>(A.out)[base] = make_uint4(orig, start, end, st);
+    }
+}
+
+// One DFA candidate per lane (see finish_dfa).
+__device__ __forceinline__ void flat_dfa(const FlatArgs &A, bool act, uint32_t job, uint32_t start, int lane,
+                                         uint64_t pol_keep) {
+    const BatchJob &J = A.jobs[job];
+    const DevMachine &M = A.machs[J.mach];
+    const uint32_t n = J.n, S = M.S, orig = J.orig;
+    const uintptr_t text = reinterpret_cast<uintptr_t>(J.text), end = text + n;
+    const uint4 *chain = M.chain;
+    const uint16_t *dtab = M.dtab;
+    uint32_t pos = start, s = M.q0;
+    const uint32_t kk = static_cast<uint32_t>(M.k);
+    if (act && n - start >= kk) {
+        const uint64_t w = bytes8_at(text, end, pos);
+        uint32_t gi = 0;
+        bool in = true;
+        for (uint32_t j = 0; j < kk; ++j) {
+            const uint32_t c = static_cast<uint32_t>(w >> (8 * j)) & 0xFFu;
+            in &= c < S;
+            gi |= c << (j * M.sbits);
+        }
+        if (in) {
+            const uint32_t e = ldg_u16_keep(M.memo + gi, pol_keep);
+            if (e == PT_SKIP) {
+                act = false;
+            } else if (!(e & PT_REC)) {   // a state; records and walks step from q0
+                s = e;
+                pos += kk;
+                if (pos >= n) act = false;
+            }
+        }
+    }
+    while (__any_sync(FULLMASK, act)) {
+        bool hit = false;
+        if (act) {
+            if (!PFSM_OK_IDX(s < static_cast<uint32_t>(M.Q), A.status)) s = 0;
+            const uint4 ch = __ldg(chain + s);
+            const uint64_t w = bytes8_at(text, end, pos);
+            const uint32_t len = ch.z & 0xFFu;
+            if (len) {
+                const uint64_t want = ch.x | (static_cast<uint64_t>(ch.y) << 32);
+                if (n - pos < len || ((w ^ want) << (64 - 8 * len)) != 0) {
+                    act = false;
+                } else {
+                    s = ch.w;
+                    pos += len;
+                    hit = (ch.z >> 8) & 1u;
+                }
+            } else {
+                const uint32_t c = static_cast<uint32_t>(w) & 0xFFu;
+                const uint32_t e = c < S ? ldg_u16_keep(dtab + s * S + c, pol_keep) : DEAD16;
+                if (e == DEAD16) {
+                    act = false;
+                } else {
+                    s = e & 0x7FFFu;
+                    hit = (e & FINAL_BIT) != 0;
+                    ++pos;
+                }
+            }
+            if (pos >= n) act = false;
+        }
+        flat_emit(A, hit, orig, start, pos - 1, s, lane);
+    }
+}
+
+// One NFA candidate per lane with its second-level record: the record's
+// matches, then its set by strands (see run_items; a strand of at most 64
+// states always fits its mask).
+__device__ __forceinline__ void flat_nfa(const FlatArgs &A, bool act, uint32_t job, uint32_t start, uint32_t rec,
+                                         uint4 *items, int lane) {
+    const BatchJob &J = A.jobs[job];
+    const DevMachine &M = A.machs[J.mach];
+    const uint32_t n = J.n, orig = J.orig;
+    uint32_t matches = 0, parts = 0;
+    uint32_t pb[SIEVE_PARTS];
+    uint64_t pm[SIEVE_PARTS];
+    const uint32_t *r = M.pool2 + (act ? rec : 0u);
+    if (act) {
+        // the header and the words after it in one round trip (16 bytes of
+        // slack follow the records)
+        const uint32_t hdr = __ldg(r), w1 = __ldg(r + 1), w2 = __ldg(r + 2), w3 = __ldg(r + 3);
+        matches = hdr & 0xFFFFu;
+        uint32_t strand = 0xFFFFFFFFu;
+        for (uint32_t x = 0; x < (hdr >> 16); ++x) {
+            const uint32_t at = matches + x;
+            const uint32_t q = at == 0 ? w1 : at == 1 ? w2 : at == 2 ? w3 : __ldg(r + 1 + at);
+            const uint32_t st = __ldg(M.sv_strand + q);
+            const bool first = st != strand;
+            strand = st;
+            parts += first;
+#pragma unroll
+            for (int p = 0; p < SIEVE_PARTS; ++p)
+                if (static_cast<uint32_t>(p) + 1 == parts) {
+                    if (first) {
+                        pb[p] = q;
+                        pm[p] = 0;
+                    }
+                    pm[p] |= 1ull << ((q - pb[p]) & 63);
+                }
+        }
+    }
+    // the record's matches (a record of a start near the end of its text may
+    // hold some past it)
+    for (uint32_t x = 0; __any_sync(FULLMASK, x < matches); ++x) {
+        const uint32_t w = x < matches ? __ldg(r + 1 + x) : 0u;
+        const uint32_t step = w >> 16;
+        flat_emit(A, x < matches && step < n - start, orig, start, start + step, w & 0xFFFFu, lane);
+    }
+    uint32_t incl = parts;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t t = __shfl_up_sync(FULLMASK, incl, d);
+        if (lane >= d) incl += t;
+    }
+    const uint32_t runs = __shfl_sync(FULLMASK, incl, 31);
+#pragma unroll
+    for (int p = 0; p < SIEVE_PARTS; ++p)
+        if (static_cast<uint32_t>(p) < parts)
+            items[incl - parts + p] = make_uint4(lane, pb[p], static_cast<uint32_t>(pm[p]), static_cast<uint32_t>(pm[p] >> 32));
+    __syncwarp();
+    for (uint32_t r0 = 0; r0 < runs; r0 += 32) {
+        bool on = r0 + lane < runs;
+        const uint4 v = on ? items[r0 + lane] : make_uint4(lane, 0u, 0u, 0u);
+        // the item's candidate: its text and machine
+        const uint32_t ijob = __shfl_sync(FULLMASK, job, v.x), istart = __shfl_sync(FULLMASK, start, v.x);
+        const BatchJob &IJ = A.jobs[ijob];
+        const DevMachine &IM = A.machs[IJ.mach];
+        const uint32_t in = IJ.n, iorig = IJ.orig;
+        const uint8_t *text = IJ.text;
+        const uint32_t *band = IM.band, *fin = band + IM.Q;
+        uint32_t base = v.y, pos = istart + static_cast<uint32_t>(IM.k) + L2_SYMS;
+        uint64_t mask = v.z | (static_cast<uint64_t>(v.w) << 32);
+        uint32_t g0 = 0, g1 = 0, left = 0;
+        on = on && pos < in;
+        while (__any_sync(FULLMASK, on)) {
+            if (on && left == 0) {
+                pack32_at(text, in, pos, g0, g1);
+                left = 32;
+            }
+            uint64_t next = 0, hits = 0;
+            if (on) {
+                const uint32_t c8 = (g0 & 3u) * 8;
+                for (uint64_t m = mask; m; m &= m - 1) {
+                    const uint32_t j = __ffsll(static_cast<long long>(m)) - 1;
+                    if (!PFSM_OK_IDX(base + j < static_cast<uint32_t>(IM.Q), A.status)) break;
+                    next |= static_cast<uint64_t>((__ldg(band + base + j) >> c8) & 0xFFu) << j;
+                }
+                on = next != 0;
+            }
+            if (on) {
+                const uint32_t sh = __ffsll(static_cast<long long>(next)) - 1;
+                mask = next >> sh;
+                base += 1 + sh;
+                // finality of states base .. base + 63 (words past the bitmap
+                // hold no state of the mask)
+                const uint32_t b = base >> 5, o = base & 31;
+                const uint32_t f0 = __ldg(fin + b), f1 = __ldg(fin + b + 1), f2 = __ldg(fin + b + 2);
+                hits = mask & (__funnelshift_r(f0, f1, o) | (static_cast<uint64_t>(__funnelshift_r(f1, f2, o)) << 32));
+            }
+            while (__any_sync(FULLMASK, hits != 0)) {
+                flat_emit(A, hits != 0, iorig, istart, pos, base + (hits ? __ffsll(static_cast<long long>(hits)) - 1 : 0), lane);
+                hits &= hits - 1;
+            }
+            ++pos;
+            on = on && pos < in;
+            g0 = __funnelshift_r(g0, g1, 2);
+            g1 >>= 2;
+            --left;
+        }
+    }
+    __syncwarp();
+}
+
+// The record of an NFA start (as sieve_levels finds it), or SIEVE_NO_RECORD.
+__device__ __forceinline__ uint32_t flat_record(const DevMachine &M, const BatchJob &J, uint32_t start, uint64_t pol_keep) {
+    const uint32_t rest = J.n - start, kk = static_cast<uint32_t>(M.k);
+    if (rest < M.min_match) return SIEVE_NO_RECORD;
+    uint32_t g0, g1;
+    pack32_at(J.text, J.n, start, g0, g1);
+    if (rest < 16) g0 &= (1u << (2 * rest)) - 1;
+    if (rest >= SIEVE_DEEP_M) {
+        const uint32_t d = g0 & ((1u << (2 * SIEVE_DEEP_M)) - 1);
+        if (!((ldg_u32_keep(M.surv2 + (d >> 5), pol_keep) >> (d & 31)) & 1u)) return SIEVE_NO_RECORD;
+    }
+    const uint32_t x = ldg_u16_keep(M.memox + (g0 & ((1u << (2 * kk)) - 1)), pol_keep);
+    if (x == L2_NONE) return SIEVE_NO_RECORD;
+    const uint32_t o2 = ldg_u16_keep(M.l2tab + x * L2_GRAMS + ((g0 >> (2 * kk)) & (L2_GRAMS - 1)), pol_keep);
+    return o2 == L2_EMPTY ? SIEVE_NO_RECORD : o2;
+}
+
+// Even CTAs run the DFA candidates, odd ones the NFA candidates. A list that
+// overflowed is replaced by every start of the texts of its kind.
+__global__ void __launch_bounds__(256) flat_finish(const __grid_constant__ FlatArgs A) {
+    __shared__ uint4 items_sm[8][32 * SIEVE_PARTS];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint64_t pol_keep = policy_evict_last();
+    const uint32_t kind = blockIdx.x & 1, ctas = gridDim.x / 2;
+    const uint32_t found = A.cand_n[kind];
+    const uint64_t warps = static_cast<uint64_t>(ctas) * 8, me = static_cast<uint64_t>(wid) * ctas + blockIdx.x / 2;
+    uint4 *items = items_sm[wid];
+    if (found <= A.cand_cap) {
+        const uint32_t per = static_cast<uint32_t>(min(static_cast<uint64_t>(32), (found + warps - 1) / warps));
+        for (uint64_t x0 = me * per; x0 < found; x0 += warps * per) {
+            const bool act = static_cast<uint32_t>(lane) < per && x0 + lane < found;
+            const uint4 c = act ? A.cand[kind][x0 + lane] : A.cand[kind][x0];
+            if (kind == 0) flat_dfa(A, act, c.x, c.y, lane, pol_keep);
+            else flat_nfa(A, act, c.x, c.y, c.z, items, lane);
+        }
+        return;
+    }
+    for (int c = 0; c < FLAT_WALK; ++c)
+        for (uint64_t j = A.job_lo[c] + me; j < A.job_hi[c]; j += warps) {
+            const BatchJob &J = A.jobs[j];
+            const DevMachine &M = A.machs[J.mach];
+            if (static_cast<uint32_t>(M.kind) != kind) continue;
+            for (uint64_t s0 = 0; s0 < J.n; s0 += 32) {
+                const uint32_t start = static_cast<uint32_t>(s0) + lane;
+                bool act = start < J.n;
+                uint32_t rec = SIEVE_NO_RECORD;
+                if (kind == 1 && act) {
+                    rec = flat_record(M, J, start, pol_keep);
+                    act = rec != SIEVE_NO_RECORD;
+                }
+                if (!__any_sync(FULLMASK, act)) continue;
+                if (kind == 0) flat_dfa(A, act, static_cast<uint32_t>(j), start, lane, pol_keep);
+                else flat_nfa(A, act, static_cast<uint32_t>(j), start, rec, items, lane);
+            }
+        }
+}
+
+// ------------------------------------------------------------ host helpers
+cudaError_t launch_flat(const FlatArgs &a, bool big, int nsm, std::atomic<uint32_t> &smem_set, cudaStream_t s) {
+    uint64_t steps = 0;
+    for (int c = 0; c < FLAT_CLASSES; ++c) steps += a.steps[c];
+    if (steps == 0) return cudaSuccess;
+    if (big) {
+        constexpr uint32_t smem = (1u << (2 * SIEVE_NEAR_M)) / 8 + 32 * kSieveList * 16;
+        static_assert(smem >= 32 * 2 * kFlatStage * 16, "the match buffers fit the sieve's regions");
+        if (!(smem_set.load(std::memory_order_relaxed) >> 9 & 1u)) {
+            const cudaError_t e = cudaFuncSetAttribute(flat_front<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (e != cudaSuccess) return e;
+            smem_set.fetch_or(1u << 9, std::memory_order_relaxed);
+        }
+        flat_front<true><<<nsm, 1024, smem, s>>>(a);
+    } else {
+        constexpr uint32_t smem = 4 * 2 * kFlatStage * 16;
+        static_assert(smem >= 4 * kSieveList * 16, "the lists fit the match buffers");
+        const int grid = static_cast<int>(std::min<uint64_t>((steps + 3) / 4, 8ull * nsm));
+        flat_front<false><<<grid, 128, smem, s>>>(a);
+    }
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    if (a.steps[FLAT_DNA] + a.steps[FLAT_BYTES] == 0) return cudaSuccess;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(big ? 8 * nsm : 2 * nsm));
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, flat_finish, a);
+}
+
+}  // namespace pfsm

@@ -618,6 +618,13 @@ static DevMachine dev_view(const Machine &m, uint8_t *base) {
     dm.chain = m.chain.empty() ? nullptr : reinterpret_cast<const uint4 *>(base + m.o_chain);
     dm.sv_strand = m.sv_strand.empty() ? nullptr : reinterpret_cast<const uint16_t *>(base + m.o_strand);
     dm.walk = m.walk_tab.empty() ? nullptr : base + m.o_walk;
+    dm.flat = -1;
+    dm.walk_words = m.walk_bitset() ? static_cast<int32_t>(walk_nfa_words(m.Q)) : 0;
+    for (int w = 0; w < 2; ++w) {
+        dm.walk_first[w] = m.walk_first[w];
+        dm.walk_finals[w] = m.walk_finals[w];
+    }
+    dm.min_match = m.min_match;
     dm.sv_l3 = m.sv_l3.empty() ? nullptr : reinterpret_cast<const uint32_t *>(base + m.o_l3);
     dm.sv_deep = m.sv_deep.empty() ? nullptr : reinterpret_cast<const uint32_t *>(base + m.o_deep);
     if (m.kind == 0) {
@@ -973,14 +980,18 @@ void collect_timing(pfsm_ctx *ctx, Slot *slot, int keep) {
 // (Positions within 256 of 2^32 would wrap.) A scan that is being captured
 // takes the tile kernel too: the counters of the other two belong to the
 // stream, and a graph may be replayed on others.
+bool default_params(const Machine &m) {
+    pfsm_params d{};
+    d.prefix_k = m.params.prefix_k;   // lowered at load where the records did not fit
+    fill_defaults(m, d);
+    return d.prefix_k >= 0 && memcmp(&d, &m.params, sizeof(d)) == 0;
+}
+
 enum Route { ROUTE_TILES, ROUTE_SIEVE, ROUTE_WALK };
 static Route route_of(const pfsm_ctx *ctx, const Machine &m, uint64_t n, cudaStream_t s) {
     const bool sieve = m.sv_kind && m.k > 0;
     if ((!sieve && !m.walks) || ctx->hold_tiles || n == 0 || n >= (1ull << 32) - 256) return ROUTE_TILES;
-    pfsm_params d{};
-    d.prefix_k = m.params.prefix_k;   // lowered at load where the records did not fit
-    fill_defaults(m, d);
-    if (d.prefix_k < 0 || memcmp(&d, &m.params, sizeof(d)) != 0) return ROUTE_TILES;
+    if (!default_params(m)) return ROUTE_TILES;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
         cudaGetLastError();
@@ -1025,7 +1036,7 @@ static int walk_enqueue(pfsm_ctx *ctx, const Machine &m, const uint8_t *text, ui
                        long_scratch_words(a.n, a.Q) <= static_cast<size_t>(kCandCap) * 2;
     return with_counters(slot, s, [&] {
         return (longs ? launch_long(a, reinterpret_cast<uint32_t *>(slot->cand), ctx->nsm, ctx->smem_set, s)
-                      : launch_walk(a, m.kind == 1 || m.lives ? 1 : 0, ctx->nsm, ctx->smem_set, s)) == cudaSuccess;
+                      : launch_walk(a, m.walk_bitset() ? 1 : 0, ctx->nsm, ctx->smem_set, s)) == cudaSuccess;
     });
 }
 

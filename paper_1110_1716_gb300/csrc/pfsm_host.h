@@ -53,11 +53,17 @@ struct Machine {
     // NFA with a sieve whose states but q0 all have band rows and none leads
     // back to q0: the weakly connected part (without q0) of every state
     std::vector<uint16_t> sv_strand;
+    // and whether a batch's kernels can take it: no match shorter than the
+    // prefix depth, every prefix with survivors leads to second-level records
+    // of at most SIEVE_PARTS strands, no strand wider than 64 states
+    bool sv_lean = false;
+    uint32_t min_match = 0;           //   symbols of the shortest match
     // direct scans (walk.cu): taken at all, the table, an NFA's sets
     // and whether its instances live long (the table is then an NFA's)
     bool walks = false, lives = false;
     std::vector<uint32_t> walk_tab;
     uint32_t walk_first[2] = {0, 0}, walk_finals[2] = {0, 0};
+    bool walk_bitset() const { return kind == 1 || lives; }
     pfsm_params params{};
     // residency: the device image is built once in pinned host memory and
     // copied in on the scan's stream whenever the machine becomes resident
@@ -182,6 +188,7 @@ void build_survival(Machine &m);
 void build_sieve(Machine &m);                                              // sieve_tables.cu
 void build_level3(Machine &m);
 void build_walk(Machine &m);
+bool default_params(const Machine &m);   // pfsm_api.cu: nothing but the prefix depth was set
 bool survival_bits_dna(const Machine &m, int mm, std::vector<uint32_t> &bits);
 size_t align256(size_t x);
 void release(pfsm_ctx *ctx, Machine &m);

@@ -96,6 +96,7 @@ constexpr int SIEVE_NONE = 0, SIEVE_DNA = 1, SIEVE_BYTES = 2;
 constexpr int SIEVE_NEAR_M = 10;     // 128 KB: what a CTA's shared memory holds
 constexpr int SIEVE_DEEP_M = 13;     // 8 MB in L2
 constexpr int SIEVE_HASH_BITS = 19;  // 64 KB: three CTAs per SM
+constexpr int SIEVE_PARTS = 3;       // strands of a record's set that a lane takes
 constexpr uint32_t SIEVE_NO_RECORD = 0xFFFFFFFFu;   // a candidate without a second-level record
 constexpr uint32_t SIEVE_HASH_MAX = 1u << (SIEVE_HASH_BITS - 4);   // most bits set
 // A sieved DFA's chains, one uint4 per state: where exactly one symbol leads
@@ -212,6 +213,8 @@ struct SieveArgs {
     const uint32_t *l3;            // NFA: third level (see L3_SYMS), or null
     const uint16_t *strand;        // NFA: strand of every state (see sv_strand), or null
     int32_t k;
+    uint32_t min_match;            // batch, NFA: symbols of the shortest match
+    uint32_t job;                  // batch: the job of the text
     uint2 *cand;                   // candidates, cand_cap of them: start and second-level
                                    // record (or SIEVE_NO_RECORD)
     uint32_t *cand_n;              // their number (past cand_cap: the list is incomplete)
@@ -236,6 +239,8 @@ struct WalkArgs {
     unsigned long long *status;      // the stream's own counters, zero between scans
     unsigned long long *status_out;  // where the scan's status goes
     uint32_t *done;                  // CTAs that ended, zero between scans
+    unsigned long long *job_counts;  // batch: matches per job
+    uint32_t orig;                   // batch: the caller's job index
     // long-lived instances (launch_long fills them): the set that each start
     // enters the segment after its own with; per segment and state the set
     // after the segment and the final states met at each of its positions
@@ -312,6 +317,12 @@ struct DevMachine {
     const uint4 *chain;
     const uint16_t *sv_strand;
     const void *walk;   // direct scan: the table (walk.cu), or null
+    // flat batches (flat_batch.cu)
+    int32_t flat;              // FLAT_* class, or -1
+    int32_t walk_words;        // direct scan: words of an NFA set (0: a DFA's table)
+    uint32_t walk_first[2], walk_finals[2];
+    uint32_t min_match;        // NFA: symbols of the shortest match
+    uint32_t flat_end;         // the step after the machine's last one in its class
     // batch: byte offsets of the tables copied into the CTA's shared-memory
     // table arena when this machine's tiles run (kNotStaged: read from
     // global memory; for the survival bitmap: not used)
@@ -336,6 +347,42 @@ struct BatchArgs {
     const DevMachine *machs;
     unsigned long long *job_counts;
 };
+
+// ---- flat batches (flat_batch.cu) -----------------------------------------
+// The texts of a batch whose machines the sieve or the direct scan takes are
+// cut into steps per class; BatchJob::unit_begin is a text's first step and
+// ntiles its number of steps.
+enum : int32_t { FLAT_DNA = 0, FLAT_BYTES = 1, FLAT_WALK = 2, FLAT_CLASSES = 3 };
+constexpr uint32_t kFlatCand = 1u << 21;   // candidates per list (DFA, NFA): 2 x 32 MB per stream
+constexpr int kFlatGroups = 32;
+struct FlatArgs {
+    const BatchJob *jobs;
+    const DevMachine *machs;
+    uint32_t job_lo[FLAT_CLASSES], job_hi[FLAT_CLASSES];
+    uint64_t steps[FLAT_CLASSES];
+    uint64_t group_end[kFlatGroups];   // ascending, in flat_cost units over the classes in turn
+    uint32_t groups;
+    uint32_t *out;
+    uint64_t cap;
+    unsigned long long *status, *job_counts;
+    uint4 *cand[2];            // DFA, NFA
+    uint32_t *cand_n;          // [2]
+    uint32_t cand_cap;
+};
+// bytes or starts per step
+__host__ __device__ constexpr uint32_t flat_step(int cls, bool big) {
+    return cls == FLAT_DNA ? 512u : cls == FLAT_BYTES ? 2048u : big ? 256u : 32u;
+}
+// Relative cost of one step: measured 0.49 ns of the whole chip per 512 bytes
+// of DNA, 0.42 ns per 2 KB of bytes and 2.4 ns per 256 starts of a dense DFA.
+__host__ __device__ constexpr uint32_t flat_cost(int cls, bool big) {
+    return cls == FLAT_DNA ? (big ? 6u : 3u) : cls == FLAT_BYTES ? (big ? 5u : 2u) : (big ? 30u : 2u);
+}
+// A text costs a warp this many steps more than it has: its arguments, its
+// first loads and its list's last entries are chains of dependent loads. Without
+// them a warp that is dealt a run of short texts keeps its CTA waiting.
+__host__ __device__ constexpr uint32_t flat_pad(bool big) { return big ? 3u : 0u; }
+cudaError_t launch_flat(const FlatArgs &a, bool big, int nsm, std::atomic<uint32_t> &smem_set, cudaStream_t s);
 
 // ---- launch helpers (scan_kernels.cu) ------------------------------------
 // Fill the smem offsets of `a` (kind_mask: 1 = DFA present, 2 = NFA present)

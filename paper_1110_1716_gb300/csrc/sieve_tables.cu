@@ -373,7 +373,8 @@ void build_sieve(Machine &m) {
     if (!dna && !bytes) return;
     if (dna) {
         uint64_t direct = 0;
-        for (uint32_t w : m.surv2) direct += static_cast<uint64_t>(__builtin_popcount(w));
+        for (uint32_t w : m.surv2)
+            if (w) direct += static_cast<uint64_t>(__builtin_popcount(w));   // (most are 0)
         if (direct * 8 > (1ull << (2 * SIEVE_DEEP_M))) return;
     }
     Delta d;
@@ -387,7 +388,8 @@ void build_sieve(Machine &m) {
             return;
         }
         for (std::vector<uint32_t> *v : {&m.sv_near, &m.sv_deep})
-            for (uint32_t &w : *v) w = top_down(w);
+            for (uint32_t &w : *v)
+                if (w) w = top_down(w);   // (most are 0)
         m.sv_kind = SIEVE_DNA;
         if (m.kind == 0) build_chains(m, d);
         else build_strands(m);
@@ -404,9 +406,56 @@ void build_sieve(Machine &m) {
     build_chains(m, d);
 }
 
+// Whether every start of a sieved NFA that can report has a second-level
+// record whose set a lane can run (see Machine::sv_lean); sets the length of
+// the shortest match.
+static bool lean(Machine &m, const Delta &d) {
+    if (m.sv_strand.empty() || m.memox.empty() || m.k + L2_SYMS > SIEVE_DEEP_M) return false;
+    std::vector<int> dist(m.Q, -1);
+    std::vector<uint16_t> cur = d.start;
+    for (uint16_t q : cur) dist[q] = 0;
+    m.min_match = 0;
+    for (uint32_t len = 1; !cur.empty() && !m.min_match; ++len) {
+        std::vector<uint16_t> nxt;
+        for (uint16_t q : cur)
+            for (uint32_t e = d.row[q]; e < d.row[q + 1]; ++e) {
+                if (d.tgt[e] & FINAL_BIT) m.min_match = len;
+                const uint16_t t = d.tgt[e] & 0x7FFF;
+                if (dist[t] >= 0) continue;
+                dist[t] = static_cast<int>(len);
+                nxt.push_back(t);
+            }
+        cur.swap(nxt);
+    }
+    if (m.min_match < static_cast<uint32_t>(m.k)) return false;   // (or nothing is ever reported)
+    for (size_t g = 0; g < m.memox.size(); ++g)
+        if (m.memo[g] != PT_SKIP && m.memox[g] == L2_NONE) return false;
+    std::vector<int> lo(m.Q, m.Q), hi(m.Q, -1);
+    for (int q = 0; q < m.Q; ++q) {
+        const int r = m.sv_strand[q];
+        if (q == m.q0) continue;
+        lo[r] = std::min(lo[r], q);
+        hi[r] = std::max(hi[r], q);
+        if (hi[r] - lo[r] >= 64) return false;
+    }
+    for (size_t at = 0; at < m.pool2.size();) {
+        const uint32_t nm = m.pool2[at] & 0xFFFFu, ns = m.pool2[at] >> 16;
+        int parts = 0, last = -1;
+        for (uint32_t x = 0; x < ns; ++x) {
+            const int r = m.sv_strand[m.pool2[at + 1 + nm + x]];
+            parts += r != last;
+            last = r;
+        }
+        if (parts > SIEVE_PARTS) return false;
+        at += 1 + nm + ns;
+    }
+    return true;
+}
+
 // The third level of a sieved NFA (see L3_SYMS); rebuilt with the records.
 void build_level3(Machine &m) {
     m.sv_l3.clear();
+    m.sv_lean = false;
     if (m.kind != 1 || m.sv_kind != SIEVE_DNA || m.l2tab.empty() || m.pool2.empty() ||
         m.pool2.size() > L3_MAX_ROWS)
         return;
@@ -427,6 +476,7 @@ void build_level3(Machine &m) {
         }
         at += 1 + nm + ns;
     }
+    m.sv_lean = lean(m, d);
 }
 
 // The bitset form of a machine of at most 64 states (see WalkArgs::tab).
@@ -487,7 +537,9 @@ static bool lives_long(const Machine &m, const Delta &d) {
 
 // Whether the machine's scans walk every start (walk.cu), and the tables for
 // it. DFAs: tables that L1 can hold, where the shallow survival bitmap would
-// pass at least 1 start in 8. NFAs: at most 64 states, tables of at most 64 KB.
+// pass at least 1 start in 256 (1 MiB, whole calls: 16384 states and 1 start
+// in 12 left, 22 us against the tiles' 30; 706 states and 1 in 21, 18 against
+// 25; 3000 states and 1 in 174, 29 against 29). NFAs: at most 64 states, tables of at most 64 KB.
 void build_walk(Machine &m) {
     m.walks = m.lives = false;
     m.walk_tab.clear();
@@ -496,7 +548,7 @@ void build_walk(Machine &m) {
         if (static_cast<size_t>(m.Q) * m.S * 2 > 160 * 1024) return;
         uint64_t ones = 0;
         for (uint32_t w : m.surv) ones += static_cast<uint64_t>(__builtin_popcount(w));
-        if (!m.surv.empty() && ones * 8 < (1ull << (m.sm_m * m.sbits))) return;
+        if (!m.surv.empty() && ones * 256 < (1ull << (m.sm_m * m.sbits))) return;
     } else if (m.Q > 64) {
         return;
     }

@@ -22,193 +22,15 @@
 #include <algorithm>
 #include <atomic>
 
-#include "scan_device.cuh"
+#include "walk.cuh"
 
 namespace pfsm {
 
 constexpr int kWalkThreads = 512;
-constexpr uint32_t kWalkStage = 192;       // staged matches per warp and half (two halves)
+constexpr uint32_t kWalkStage = 192;       // staged matches per warp and half
 constexpr uint32_t kWalkTabSmem = 32768;   // tables up to this size are copied to shared memory
-constexpr int kRound = 8;                  // symbols per round
-constexpr uint32_t kSegment = 64;          // symbols per segment (long_walk)
 
-// The eight text bytes from position pos (those past the end of the text are
-// unspecified).
-__device__ __forceinline__ uint64_t window8(uintptr_t text, uintptr_t end, uint32_t pos) {
-    const uintptr_t at = text + pos, lo = at & ~static_cast<uintptr_t>(7);
-    const uint32_t sh = static_cast<uint32_t>(at & 7) * 8;
-    const uint64_t a = __ldg(reinterpret_cast<const unsigned long long *>(lo));
-    const uint64_t b = lo + 8 < end ? __ldg(reinterpret_cast<const unsigned long long *>(lo + 8)) : 0ull;
-    return sh ? (a >> sh) | (b << (64 - sh)) : a;
-}
-
-// A warp's match buffer: one half fills while the place of the other's
-// matches in the output is being reserved, so that no round waits for the
-// atomic's round trip.
-struct WalkOut {
-    uint32_t *buf;              // two halves of kWalkStage matches
-    uint32_t half;              // the one that fills
-    uint32_t n;                 // its matches
-    uint32_t leaving;           // matches of the other half, not yet copied
-    unsigned long long base;    //   (lane 0) their place
-
-    // copies what is leaving
-    __device__ __forceinline__ void copy(const WalkArgs &a, int lane) {
-        if (leaving == 0) return;
-        const unsigned long long b = __shfl_sync(FULLMASK, base, 0);
-        const uint32_t words =
-            b >= a.cap ? 0u : 3 * static_cast<uint32_t>(min(static_cast<unsigned long long>(leaving), a.cap - b));
-        uint32_t *o = a.out + b * 3;
-        const uint32_t *from = buf + (half ^ 1) * (3 * kWalkStage);
-        __syncwarp();
-        for (uint32_t w = lane; w < words; w += 32) o[w] = from[w];
-        __syncwarp();
-        leaving = 0;
-    }
-    // the filling half leaves; the other must have been copied
-    __device__ __forceinline__ void turn(const WalkArgs &a, int lane) {
-        if (lane == 0) base = atomicAdd(&a.status[0], static_cast<unsigned long long>(n));
-        leaving = n;
-        n = 0;
-        half ^= 1;
-    }
-};
-
-// A DFA instance: its state; the table has the dead state as its last row.
-template <bool TAB_SMEM>
-struct WalkDfa {
-    uint32_t s;
-    uint32_t seen[kRound];   // the round's table entries
-    uint32_t hits;           // bit j: the j-th of them is final
-    __device__ __forceinline__ void begin(const WalkArgs &a) { s = a.q0; }
-    __device__ __forceinline__ void step(const WalkArgs &a, const uint8_t *tab, uint32_t c, int j) {
-        const uint32_t ix = s * a.S + c;
-        const uint32_t e = TAB_SMEM ? reinterpret_cast<const uint16_t *>(tab)[ix]
-                                    : __ldg(reinterpret_cast<const uint16_t *>(a.tab) + ix);
-        s = e & 0x7FFFu;
-        seen[j] = s;
-        if (j == 0) hits = 0;
-        hits |= (e >> 15) << j;
-    }
-    __device__ __forceinline__ bool alive(const WalkArgs &a) const { return s != static_cast<uint32_t>(a.Q); }
-    // matches of the round's first `lim` symbols
-    __device__ __forceinline__ uint32_t count(uint32_t lim) {
-        if (lim < kRound) hits &= (1u << lim) - 1;
-        return __popc(hits);
-    }
-    __device__ __forceinline__ void put_out(const WalkArgs &a, uint32_t start, uint32_t pos, unsigned long long at) const {
-#pragma unroll
-        for (int j = 0; j < kRound; ++j) {
-            if ((hits >> j) & 1u) {
-                if (at < a.cap) {
-                    uint32_t *o = a.out + at * 3;
-                    o[0] = start;
-                    o[1] = pos + j;
-                    o[2] = seen[j];
-                }
-                ++at;
-            }
-        }
-    }
-    __device__ __forceinline__ void put(const WalkArgs &a, uint32_t start, uint32_t pos, uint32_t *p) const {
-#pragma unroll
-        for (int j = 0; j < kRound; ++j) {
-            if ((hits >> j) & 1u) {
-                p[0] = start;
-                p[1] = pos + j;
-                p[2] = seen[j];
-                p += 3;
-            }
-        }
-    }
-};
-
-// An NFA instance: its states as a bitset of W words of 32. The table holds,
-// per eight states and symbol, the targets of each of their 256 subsets.
-template <int W>
-struct WalkNfa {
-    uint32_t s[W];
-    uint32_t seen[kRound][W];   // the round's final states
-    uint32_t sets[kRound][W];   // and sets
-    __device__ __forceinline__ void begin(const WalkArgs &a) {
-#pragma unroll
-        for (int w = 0; w < W; ++w) s[w] = a.first[w];
-    }
-    __device__ __forceinline__ void step(const WalkArgs &a, const uint8_t *tab, uint32_t c, int j) {
-        const uint32_t *t = reinterpret_cast<const uint32_t *>(tab) + c * (256 * W);
-        const uint32_t row = a.S * 256 * W;
-        uint32_t n[W];
-#pragma unroll
-        for (int w = 0; w < W; ++w) n[w] = 0;
-#pragma unroll
-        for (int g = 0; g < 4 * W; ++g) {
-            if (g * 8 < a.Q) {
-                const uint32_t *e = t + g * row + ((s[g >> 2] >> (8 * (g & 3))) & 0xFFu) * W;
-#pragma unroll
-                for (int w = 0; w < W; ++w) n[w] |= e[w];
-            }
-        }
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-            s[w] = n[w];
-            sets[j][w] = n[w];
-            seen[j][w] = n[w] & a.finals[w];
-        }
-    }
-    __device__ __forceinline__ bool alive(const WalkArgs &) const { return (s[0] | s[W - 1]) != 0; }
-    // the segment ended `lim` symbols into the round, or the instance died:
-    // the set it enters the next segment with (segments are whole rounds, but
-    // a start's first round is not aligned to them)
-    __device__ __forceinline__ void leave(const WalkArgs &a, uint32_t start, uint32_t lim) const {
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-            uint32_t v = s[w];
-#pragma unroll
-            for (int j = 0; j < kRound - 1; ++j) v = lim == static_cast<uint32_t>(j) + 1 ? sets[j][w] : v;
-            a.entry[static_cast<size_t>(start) * W + w] = v;
-        }
-    }
-    __device__ __forceinline__ uint32_t count(uint32_t lim) {
-        uint32_t c = 0;
-#pragma unroll
-        for (int j = 0; j < kRound; ++j)
-#pragma unroll
-            for (int w = 0; w < W; ++w) {
-                if (static_cast<uint32_t>(j) >= lim) seen[j][w] = 0;
-                c += __popc(seen[j][w]);
-            }
-        return c;
-    }
-    __device__ __forceinline__ void put_out(const WalkArgs &a, uint32_t start, uint32_t pos, unsigned long long at) const {
-#pragma unroll
-        for (int j = 0; j < kRound; ++j)
-#pragma unroll
-            for (int w = 0; w < W; ++w)
-                for (uint32_t f = seen[j][w]; f; f &= f - 1, ++at) {
-                    if (at >= a.cap) continue;
-                    uint32_t *o = a.out + at * 3;
-                    o[0] = start;
-                    o[1] = pos + j;
-                    o[2] = 32 * w + __ffs(f) - 1;
-                }
-    }
-    __device__ __forceinline__ void put(const WalkArgs &, uint32_t start, uint32_t pos, uint32_t *p) const {
-#pragma unroll
-        for (int j = 0; j < kRound; ++j)
-#pragma unroll
-            for (int w = 0; w < W; ++w)
-                for (uint32_t f = seen[j][w]; f; f &= f - 1) {
-                    p[0] = start;
-                    p[1] = pos + j;
-                    p[2] = 32 * w + __ffs(f) - 1;
-                    p += 3;
-                }
-    }
-};
-
-// Walks the warp's range of starts; with SEG (long_walk below) only to the end
-// of the start's own segment of the text, leaving the sets held there in
-// a.entry.
+// The CTA's part of a scan's starts: a warp takes a range of consecutive ones.
 template <class I, bool TAB_SMEM, bool SEG>
 __device__ __forceinline__ void walk_starts(const WalkArgs &a, uint8_t *smem) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
@@ -218,72 +40,14 @@ __device__ __forceinline__ void walk_starts(const WalkArgs &a, uint8_t *smem) {
         for (uint32_t i = tid; i < (a.tab_bytes + 15) / 16; i += blockDim.x) d[i] = __ldg(g + i);
         __syncthreads();
     }
-    WalkOut out{reinterpret_cast<uint32_t *>(smem + a.sm_stage) + wid * (2 * 3 * kWalkStage), 0u, 0u, 0u, 0ull};
-    const uint32_t n = a.n, S = a.S;
-    const uintptr_t text = reinterpret_cast<uintptr_t>(a.text), end = text + n;
+    WalkOut<3, kWalkStage> out{reinterpret_cast<uint32_t *>(smem + a.sm_stage) + wid * (2 * 3 * kWalkStage), 0u, 0u, 0u,
+                               0ull};
     const uint64_t lo = (static_cast<uint64_t>(blockIdx.x) * nw + wid) * a.range;
-    uint32_t head = lo < n ? static_cast<uint32_t>(lo) : n;              // the range's next start
-    const uint32_t stop = lo + a.range < n ? static_cast<uint32_t>(lo + a.range) : n;
-    bool bad = false, act = false;
-    I inst;
-    inst.begin(a);
-    uint32_t start = 0, pos = 0;
-    while (true) {
-        const uint32_t idle = __ballot_sync(FULLMASK, !act);
-        bool fresh = false;
-        if (idle && head < stop) {
-            const uint32_t mine = head + __popc(idle & lanemask_lt());
-            fresh = !act && mine < stop;
-            if (fresh) {
-                start = pos = mine;
-                inst.begin(a);
-                act = true;
-            }
-            head = min(stop, head + __popc(idle));
-        } else if (idle == FULLMASK) {
-            break;
-        }
-        const uint64_t w = act ? window8(text, end, pos) : 0ull;
-        // every symbol is some start's first; one out of range fails the scan,
-        // whatever is stepped in its place
-        bad |= fresh && (static_cast<uint32_t>(w) & 0xFFu) >= S;
-#pragma unroll
-        for (int j = 0; j < kRound; ++j) inst.step(a, smem, min(static_cast<uint32_t>(w >> (8 * j)) & 0xFFu, S - 1), j);
-        // symbols left (of the segment)
-        const uint32_t lim = !act ? 0u : SEG ? min(n, (start / kSegment + 1) * kSegment) - pos : n - pos;
-        const uint32_t c = inst.count(lim);
-        if (__any_sync(FULLMASK, c != 0)) {
-            uint32_t incl = c;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const uint32_t t = __shfl_up_sync(FULLMASK, incl, d);
-                if (lane >= d) incl += t;
-            }
-            const uint32_t total = __shfl_sync(FULLMASK, incl, 31);
-            if (out.n + total > kWalkStage) {
-                out.copy(a, lane);
-                out.turn(a, lane);
-            }
-            if (total <= kWalkStage) {
-                inst.put(a, start, pos, out.buf + out.half * (3 * kWalkStage) + 3 * (out.n + incl - c));
-                out.n += total;
-            } else {   // a round of very many matches: straight to the output
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(&a.status[0], static_cast<unsigned long long>(total));
-                base = __shfl_sync(FULLMASK, base, 0) + (incl - c);
-                inst.put_out(a, start, pos, base);
-            }
-        }
-        pos += kRound;
-        const bool on = act && lim > kRound && inst.alive(a);
-        if constexpr (SEG) {
-            if (act && !on) inst.leave(a, start, lim);
-        }
-        act = on;
-    }
-    out.copy(a, lane);
-    out.turn(a, lane);
-    out.copy(a, lane);
+    const uint32_t head = lo < a.n ? static_cast<uint32_t>(lo) : a.n;
+    const uint32_t stop = lo + a.range < a.n ? static_cast<uint32_t>(lo + a.range) : a.n;
+    bool bad = false;
+    walk_range<I, SEG>(a, smem, head, stop, out, bad, lane);
+    out.finish(a, lane);
     if (bad) atomicOr(&a.status[1], ERR_SYMBOL);
 }
 
@@ -349,7 +113,7 @@ __global__ void __launch_bounds__(256) long_finish(const WalkArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    WalkOut out{reinterpret_cast<uint32_t *>(smem) + wid * (2 * 3 * kWalkStage), 0u, 0u, 0u, 0ull};
+    WalkOut<3, kWalkStage> out{reinterpret_cast<uint32_t *>(smem) + wid * (2 * 3 * kWalkStage), 0u, 0u, 0u, 0ull};
     const uint32_t segs = (a.n + kSegment - 1) / kSegment, Q = a.Q;
     constexpr int PER = kSegment / 32;   // positions per lane
     for (uint32_t i = blockIdx.x * nw + wid; i < a.n; i += gridDim.x * nw) {
@@ -386,12 +150,9 @@ __global__ void __launch_bounds__(256) long_finish(const WalkArgs a) {
                     uint32_t m;
                     while ((m = __ballot_sync(FULLMASK, f != 0)) != 0) {
                         const uint32_t c = __popc(m);
-                        if (out.n + c > kWalkStage) {
-                            out.copy(a, lane);
-                            out.turn(a, lane);
-                        }
+                        out.room(a, c, lane);
                         if (f) {
-                            uint32_t *p = out.buf + out.half * (3 * kWalkStage) + 3 * (out.n + __popc(m & lanemask_lt()));
+                            uint32_t *p = out.row(__popc(m & lanemask_lt()));
                             p[0] = i;
                             p[1] = g * kSegment + 32 * x + lane;
                             p[2] = 32 * w + __ffs(f) - 1;
@@ -405,9 +166,7 @@ __global__ void __launch_bounds__(256) long_finish(const WalkArgs a) {
             for (int w = 0; w < W; ++w) any |= s[w] = to[w];
         }
     }
-    out.copy(a, lane);
-    out.turn(a, lane);
-    out.copy(a, lane);
+    out.finish(a, lane);
     scan_status_out(a.status, a.status_out, a.done, nullptr);
 }
 
