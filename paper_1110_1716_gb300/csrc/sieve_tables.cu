@@ -130,13 +130,14 @@ struct GramWalk {
     uint32_t *bits;
     uint64_t limit;      // give up past this many set bits
     int part;            // -1: the whole tree
+    uint32_t flip;       // 31: bits stored from the top of a word down
     uint64_t ones = 0;
     std::vector<uint32_t> mark;
     uint32_t stamp = 0;
     std::vector<std::vector<uint16_t>> lv;
 
-    GramWalk(const Delta &dd, const std::vector<uint8_t> &nx, int m, uint32_t *b, uint64_t lim, int p)
-        : d(dd), next(nx), mm(m), bits(b), limit(lim), part(p), mark(dd.Q, 0), lv(m + 1) {}
+    GramWalk(const Delta &dd, const std::vector<uint8_t> &nx, int m, uint32_t *b, uint64_t lim, int p, uint32_t f)
+        : d(dd), next(nx), mm(m), bits(b), limit(lim), part(p), flip(f), mark(dd.Q, 0), lv(m + 1) {}
 
     bool mine(int depth, uint32_t prefix) const {
         if (part < 0) return true;
@@ -149,7 +150,7 @@ struct GramWalk {
         for (uint32_t hw = 0; hw < (1u << rest); ++hw) {
             const uint32_t w = p | (hw << (2 * depth));
             if (depth < 6 && !mine(6, w)) continue;
-            bits[w >> 5] |= 1u << (w & 31);
+            bits[w >> 5] |= 1u << ((w & 31) ^ flip);
             ++ones;
         }
     }
@@ -162,7 +163,7 @@ struct GramWalk {
             for (int a = 0; a < 4; ++a)
                 if ((any >> a) & 1u) {
                     const uint32_t w = prefix | (static_cast<uint32_t>(a) << (2 * depth));
-                    bits[w >> 5] |= 1u << (w & 31);
+                    bits[w >> 5] |= 1u << ((w & 31) ^ flip);
                     ++ones;
                 }
             return;
@@ -201,8 +202,9 @@ std::vector<uint8_t> successor_symbols(const Delta &d) {
 }
 
 // The m-gram bitmap of instances that hold `from`; false (and no bitmap)
-// when more than `limit` grams are set.
-bool gram_bits(const Delta &d, const std::vector<uint16_t> &from, int mm, uint64_t limit,
+// when more than `limit` grams are set. `flip` 31: stored from the top of a
+// word down, as the sieve reads them.
+bool gram_bits(const Delta &d, const std::vector<uint16_t> &from, int mm, uint64_t limit, uint32_t flip,
                std::vector<uint32_t> &bits) {
     const std::vector<uint8_t> next = successor_symbols(d);
     bits.assign((size_t(1) << (2 * mm)) / 32, 0);
@@ -212,7 +214,7 @@ bool gram_bits(const Delta &d, const std::vector<uint16_t> &from, int mm, uint64
     const uint64_t part_limit = split ? limit / kParts * 4 : limit;
     std::vector<uint64_t> ones(parts, 0);
     auto work = [&](int p) {
-        GramWalk w(d, next, mm, bits.data(), part_limit, split ? p : -1);
+        GramWalk w(d, next, mm, bits.data(), part_limit, split ? p : -1, flip);
         w.lv[0] = from;
         w.run(0, 0);
         ones[p] = w.ones;
@@ -312,14 +314,6 @@ static void build_chains(Machine &m, const Delta &d) {
     }
 }
 
-// Bit x of a word to bit 31 - x.
-static uint32_t top_down(uint32_t w) {
-    w = ((w >> 1) & 0x55555555u) | ((w & 0x55555555u) << 1);
-    w = ((w >> 2) & 0x33333333u) | ((w & 0x33333333u) << 2);
-    w = ((w >> 4) & 0x0F0F0F0Fu) | ((w & 0x0F0F0F0Fu) << 4);
-    return __builtin_bswap32(w);
-}
-
 // The strands of a sieved NFA (see sv_strand): parts of the machine that no
 // edge joins once q0 is left.
 static void build_strands(Machine &m) {
@@ -373,8 +367,10 @@ void build_sieve(Machine &m) {
     if (!dna && !bytes) return;
     if (dna) {
         uint64_t direct = 0;
-        for (uint32_t w : m.surv2)
-            if (w) direct += static_cast<uint64_t>(__builtin_popcount(w));   // (most are 0)
+        for (size_t i = 0; i + 1 < m.surv2.size(); i += 2) {   // (most are 0)
+            const uint64_t w = m.surv2[i] | (static_cast<uint64_t>(m.surv2[i + 1]) << 32);
+            if (w) direct += static_cast<uint64_t>(__builtin_popcountll(w));
+        }
         if (direct * 8 > (1ull << (2 * SIEVE_DEEP_M))) return;
     }
     Delta d;
@@ -382,14 +378,11 @@ void build_sieve(Machine &m) {
     std::vector<uint16_t> u;
     if (!sampled_states(d, dna ? SIEVE_DNA_STEP : SIEVE_BYTE_STEP, u)) return;
     if (dna) {
-        if (!gram_bits(d, u, SIEVE_NEAR_M, (1ull << (2 * SIEVE_NEAR_M)) * 3 / 4, m.sv_near)) return;
-        if (!gram_bits(d, u, SIEVE_DEEP_M, (1ull << (2 * SIEVE_DEEP_M)) / 8, m.sv_deep)) {
+        if (!gram_bits(d, u, SIEVE_NEAR_M, (1ull << (2 * SIEVE_NEAR_M)) * 3 / 4, 31, m.sv_near)) return;
+        if (!gram_bits(d, u, SIEVE_DEEP_M, (1ull << (2 * SIEVE_DEEP_M)) / 8, 31, m.sv_deep)) {
             m.sv_near.clear();
             return;
         }
-        for (std::vector<uint32_t> *v : {&m.sv_near, &m.sv_deep})
-            for (uint32_t &w : *v)
-                if (w) w = top_down(w);   // (most are 0)
         m.sv_kind = SIEVE_DNA;
         if (m.kind == 0) build_chains(m, d);
         else build_strands(m);
@@ -463,7 +456,7 @@ void build_level3(Machine &m) {
     flatten(m, d);
     m.sv_l3.assign(m.pool2.size() * (L3_GRAMS / 32), 0u);
     const std::vector<uint8_t> next = successor_symbols(d);
-    GramWalk w(d, next, L3_SYMS, nullptr, ~0ull, -1);
+    GramWalk w(d, next, L3_SYMS, nullptr, ~0ull, -1, 0);
     for (size_t at = 0; at < m.pool2.size();) {
         const uint32_t nm = m.pool2[at] & 0xFFFFu, ns = m.pool2[at] >> 16;
         uint32_t *to = m.sv_l3.data() + at * (L3_GRAMS / 32);
@@ -579,7 +572,7 @@ void build_walk(Machine &m) {
 bool survival_bits_dna(const Machine &m, int mm, std::vector<uint32_t> &bits) {
     Delta d;
     flatten(m, d);
-    return gram_bits(d, d.start, mm, (1ull << (2 * mm)) / 2, bits);
+    return gram_bits(d, d.start, mm, (1ull << (2 * mm)) / 2, 0, bits);
 }
 
 }  // namespace pfsm
