@@ -1032,10 +1032,10 @@ static int walk_enqueue(pfsm_ctx *ctx, const Machine &m, const uint8_t *text, ui
     a.status_out = status;
     a.done = slot->sv_count + 1;
     // (the scratch of long-lived instances is the candidates' buffer)
-    const bool longs = m.lives && n >= kLongText &&
-                       long_scratch_words(a.n, a.Q) <= static_cast<size_t>(kCandCap) * 2;
+    const size_t words = 2 * static_cast<size_t>(ctx->test_carry_cap ? std::min(kCandCap, ctx->test_carry_cap) : kCandCap);
+    const bool longs = m.lives && n >= kLongText && long_fits(a.n, a.Q, words);
     return with_counters(slot, s, [&] {
-        return (longs ? launch_long(a, reinterpret_cast<uint32_t *>(slot->cand), ctx->nsm, ctx->smem_set, s)
+        return (longs ? launch_long(a, reinterpret_cast<uint32_t *>(slot->cand), words, ctx->nsm, ctx->smem_set, s)
                       : launch_walk(a, m.walk_bitset() ? 1 : 0, ctx->nsm, ctx->smem_set, s)) == cudaSuccess;
     });
 }

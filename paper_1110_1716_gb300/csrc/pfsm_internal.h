@@ -242,10 +242,13 @@ struct WalkArgs {
     unsigned long long *job_counts;  // batch: matches per job
     uint32_t orig;                   // batch: the caller's job index
     // long-lived instances (launch_long fills them): the set that each start
-    // enters the segment after its own with; per segment and state the set
-    // after the segment and the final states met at each of its positions
+    // enters the segment after its own with; per segment and row (long_rows)
+    // the set after the segment and the final states met at each of its
+    // positions
     uint32_t *entry, *exit, *met;
+    unsigned long long *hits;   // and the positions with any
     uint32_t start_ctas;        // CTAs of long_walk that walk starts
+    uint32_t seg_smem;          // long_finish: the segments' exits in shared memory
     // filled by the launch
     uint32_t range;             // starts per warp
     uint32_t sm_stage;          // shared-memory offset of the match buffers
@@ -419,8 +422,9 @@ cudaError_t launch_finish_nfa(const ScanArgs &a, const SieveArgs &sv, uint32_t s
 // the direct scan (walk.cu); words of an NFA set
 cudaError_t launch_walk(WalkArgs a, int kind, int nsm, std::atomic<uint32_t> &smem_set, cudaStream_t s);
 uint32_t walk_nfa_words(int Q);
-cudaError_t launch_long(WalkArgs a, uint32_t *scratch, int nsm, std::atomic<uint32_t> &smem_set, cudaStream_t s);
-size_t long_scratch_words(uint32_t n, int Q);
+cudaError_t launch_long(const WalkArgs &a, uint32_t *scratch, size_t words, int nsm, std::atomic<uint32_t> &smem_set,
+                        cudaStream_t s);
+bool long_fits(uint32_t n, int Q, size_t words);   // launch_long's scratch
 constexpr uint32_t kLongText = 512;   // symbols from which launch_long is taken
 
 // ---- batch launch helpers (batch_kernels.cu) -----------------------------
