@@ -134,7 +134,9 @@ def _check(status: int, what: str, required: Optional[int] = None):
 def _stream_ptr(stream) -> Optional[int]:
     if stream is None:
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        # the handle without a Stream object around it: 0.3 us instead of 3
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        return raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream
     return getattr(stream, "cuda_stream", stream)
 
 
