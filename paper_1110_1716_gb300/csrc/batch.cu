@@ -35,9 +35,13 @@ constexpr int kFlatCtr = 16;            // counter words holding the flat batche
 // machine it meets). 64 texts, 4 motif sets, whole calls: 4 MiB 64 us (62
 // without), 8 MiB 63 (74), 64 MiB 138 (197); bytes 50 us (50), 50 (50), 62 (75)
 constexpr uint64_t kFlatBig = 8ull << 20;
-// least cost of a group of machines, 25 us of the whole chip: every group
-// copies its bitmaps and starts its warps anew (5 us)
-constexpr uint64_t kFlatGroupCost = 306000;
+// least cost of a group of machines, 50 us of the whole chip: every group
+// copies its bitmaps and starts its warps anew, and only long groups lose
+// more than that to each other's deep bitmaps (flat_front, 8 motif sets of 48
+// over 8 MiB: 49 us as one group, 57 as two, 70 as four; 8 of 256 and 8
+// signature sets over 1.1 GB: 0.88 ms with this bound, 0.90 with a quarter of
+// it, 1.16 with one that puts two of the larger sets together)
+constexpr uint64_t kFlatGroupCost = 600000;
 
 struct BatchGraph {
     cudaGraphExec_t exec = nullptr;

@@ -136,7 +136,7 @@ __device__ __forceinline__ void flat_steps(const FlatArgs &A, FlatWarp &wa, uint
 // The CTAs share the steps group by group: the deep bitmaps of the machines
 // they test with at one time have to stay in L2 (8 MB each, read at random).
 // 10,000 texts over 8 motif and 8 signature sets: all machines at once 1.63 ms
-// for the kernel, 1.16 ms with two sets to a group, 0.90 ms with one.
+// for the kernel, 1.16 ms with two sets to a group, 0.88 ms with one.
 template <bool BIG>
 __global__ void __launch_bounds__(BIG ? 1024 : 128, 1) flat_front(const __grid_constant__ FlatArgs A) {
     __shared__ FlatWarp warps[BIG ? 32 : 4];
