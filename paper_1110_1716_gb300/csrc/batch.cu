@@ -35,13 +35,13 @@ constexpr int kFlatCtr = 16;            // counter words holding the flat batche
 // machine it meets). 64 texts, 4 motif sets, whole calls: 4 MiB 64 us (62
 // without), 8 MiB 63 (74), 64 MiB 138 (197); bytes 50 us (50), 50 (50), 62 (75)
 constexpr uint64_t kFlatBig = 8ull << 20;
-// least cost of a group of machines, 50 us of the whole chip: every group
-// copies its bitmaps and starts its warps anew, and only long groups lose
-// more than that to each other's deep bitmaps (flat_front, 8 motif sets of 48
-// over 8 MiB: 49 us as one group, 57 as two, 70 as four; 8 of 256 and 8
-// signature sets over 1.1 GB: 0.88 ms with this bound, 0.90 with a quarter of
-// it, 1.16 with one that puts two of the larger sets together)
-constexpr uint64_t kFlatGroupCost = 600000;
+// least cost of a group of machines, 25 us of the whole chip: every group
+// copies its bitmaps and starts its warps anew, and groups of several machines
+// lose to each other's deep bitmaps. flat_front with a third of this bound,
+// this one and twice it: 8 motif and 8 signature sets over 2000 texts 255, 247
+// and 285 us; 8 sets of 256 motifs over 8 MiB 95, 85 and 101; of 48 motifs 70,
+// 57 and 50.
+constexpr uint64_t kFlatGroupCost = 300000;
 
 struct BatchGraph {
     cudaGraphExec_t exec = nullptr;
@@ -319,8 +319,9 @@ static void plan_groups(const std::vector<uint32_t> &order, FlatPlan &pl) {
 }
 
 // Cuts the flat texts (jobs of machine slots with a class in flat_of) into
-// steps, sorted by class, machine and the caller's order.
-static int plan_flat(const pfsm_job *jobs, int32_t k, const std::vector<uint32_t> &job_slot,
+// steps, sorted by class, machine and the caller's order. False where a class
+// has too many steps to number: the class kernels then take the whole batch.
+static bool plan_flat(const pfsm_job *jobs, int32_t k, const std::vector<uint32_t> &job_slot,
                      const std::vector<int> &flat_of, const std::vector<Machine *> &machines, FlatPlan &pl) {
     uint64_t sieved = 0;
     std::vector<uint32_t> first(flat_of.size(), 0), order;
@@ -368,14 +369,14 @@ static int plan_flat(const pfsm_job *jobs, int32_t k, const std::vector<uint32_t
         for (uint32_t j = pl.job_lo[c]; j < pl.job_hi[c]; ++j) {
             BatchJob &b = pl.jobs[j];
             const uint64_t steps = b.ntiles ? static_cast<uint64_t>(b.ntiles) + flat_pad(pl.big) : 0u;
-            if (pl.steps[c] + steps >= (1ull << 31)) return PFSM_E_INVAL;
+            if (pl.steps[c] + steps >= (1ull << 31)) return false;
             b.unit_begin = static_cast<uint32_t>(pl.steps[c]);
             pl.steps[c] += steps;
             pl.machs[b.mach].flat_end = static_cast<uint32_t>(pl.steps[c]);
         }
     }
     plan_groups(order, pl);
-    return PFSM_OK;
+    return true;
 }
 
 // Validate the jobs, make their machines resident, classify them and cut
@@ -424,9 +425,10 @@ static int plan_batch(pfsm_ctx *ctx, const pfsm_job *jobs, int32_t k, BatchPlan 
         if (jobs[i].n >= (1ull << 32) - 256) flat_of[job_slot[i]] = -1;   // positions would wrap
     }
     for (int32_t i = 0; i < k; ++i) rest -= flat_of[job_slot[i]] >= 0;
-    if (rest < k) {
-        int fs = plan_flat(jobs, k, job_slot, flat_of, pl.used, pl.flat);
-        if (fs) return fs;
+    if (rest < k && !plan_flat(jobs, k, job_slot, flat_of, pl.used, pl.flat)) {
+        std::fill(flat_of.begin(), flat_of.end(), -1);
+        pl.flat = FlatPlan{};
+        rest = k;
     }
     if (rest == 0) return PFSM_OK;
     // the DFA classes share one shape (threads, arena), as do the NFA classes

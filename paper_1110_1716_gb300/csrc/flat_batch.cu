@@ -11,8 +11,8 @@
 // Measured, whole calls, against one tile kernel per class and shape plus the
 // carry kernel in a graph: 64 requests over 24 machines 450 -> 69 us, of which
 // flat_front takes 25 and flat_finish 12 (chains of dependent loads: a request
-// is a few steps long); 10,000 texts over 16 machines, 1.1 GB, 4.7 -> 1.28 ms;
-// 8 machines over 8 MiB each 350 -> 109 us. With full warps of steps flat_front
+// is a few steps long); 10,000 texts over 16 machines, 1.1 GB, 4.7 -> 1.25 ms;
+// 8 machines over 8 MiB each 350 -> 105 us. With full warps of steps flat_front
 // is bound like the single-text kernels: 64 MiB of DNA 72 us against 60,
 // 256 MiB of bytes 61 us against 50; the rest is the start of a share (its
 // job, arguments and first loads) and arguments read from shared memory
@@ -136,7 +136,7 @@ __device__ __forceinline__ void flat_steps(const FlatArgs &A, FlatWarp &wa, uint
 // The CTAs share the steps group by group: the deep bitmaps of the machines
 // they test with at one time have to stay in L2 (8 MB each, read at random).
 // 10,000 texts over 8 motif and 8 signature sets: all machines at once 1.63 ms
-// for the kernel, 1.16 ms with two sets to a group, 0.88 ms with one.
+// for the kernel, 1.16 ms with two sets to a group, 0.90 ms with one.
 template <bool BIG>
 __global__ void __launch_bounds__(BIG ? 1024 : 128, 1) flat_front(const __grid_constant__ FlatArgs A) {
     __shared__ FlatWarp warps[BIG ? 32 : 4];
