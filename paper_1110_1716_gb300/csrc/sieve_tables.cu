@@ -14,6 +14,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <thread>
 #include <vector>
 
@@ -365,8 +366,8 @@ void build_sieve(Machine &m) {
     const bool dna = m.sbits == 2 && m.sm_m2 == SIEVE_DEEP_M;
     const bool bytes = m.kind == 0 && m.sbits > 2;
     if (!dna && !bytes) return;
+    uint64_t direct = 0;
     if (dna) {
-        uint64_t direct = 0;
         for (size_t i = 0; i + 1 < m.surv2.size(); i += 2) {   // (most are 0)
             const uint64_t w = m.surv2[i] | (static_cast<uint64_t>(m.surv2[i + 1]) << 32);
             if (w) direct += static_cast<uint64_t>(__builtin_popcountll(w));
@@ -379,6 +380,21 @@ void build_sieve(Machine &m) {
     if (!sampled_states(d, dna ? SIEVE_DNA_STEP : SIEVE_BYTE_STEP, u)) return;
     if (dna) {
         if (!gram_bits(d, u, SIEVE_NEAR_M, (1ull << (2 * SIEVE_NEAR_M)) * 3 / 4, 31, m.sv_near)) return;
+        // What is left of the near grams three symbols on, by how the direct
+        // ones thin out from 9 symbols to 13: instances that live on as those
+        // of random DFAs do would fill the deep bitmap past its limit, and
+        // finding that out takes several times as long as the other tables.
+        auto share = [](const std::vector<uint32_t> &v) {
+            uint64_t n = 0;
+            for (uint32_t w : v) n += static_cast<uint64_t>(__builtin_popcount(w));
+            return static_cast<double>(n) / (32.0 * static_cast<double>(v.size()));
+        };
+        const double at9 = m.sm_m == 9 ? share(m.surv) : 0.0;
+        const double at13 = static_cast<double>(direct) / static_cast<double>(1ull << (2 * SIEVE_DEEP_M));
+        if (at9 > 0.0 && share(m.sv_near) * std::pow(at13 / at9, 0.75) > 1.25 / 8) {
+            m.sv_near.clear();
+            return;
+        }
         if (!gram_bits(d, u, SIEVE_DEEP_M, (1ull << (2 * SIEVE_DEEP_M)) / 8, 31, m.sv_deep)) {
             m.sv_near.clear();
             return;
