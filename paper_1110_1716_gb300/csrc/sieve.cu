@@ -14,7 +14,7 @@
 // (device time per scan): 1000-signature trie, 1 GiB: 752 -> 203 us (5.3
 // TB/s of text; bound by shared-memory wavefronts of the random bitmap reads,
 // 85 % of peak, and DRAM, 72 %); 4 MB: 40 -> 17 us; 256-motif NFA, 64 MiB:
-// 213 -> 72 us (bound by the random 32-byte reads of the bitmaps in L2, one
+// 213 -> 69 us (bound by the random 32-byte reads of the bitmaps in L2, one
 // request per cycle and SM at 70 % of peak); 100 KB: 18 -> 17 us.
 //
 // Should the candidates outgrow their list, the finishing kernel takes every
@@ -405,8 +405,12 @@ static cudaError_t launch_steps(K k, const SieveArgs &a, uint32_t span, int thre
 
 cudaError_t launch_sieve(const SieveArgs &a, int kind, int nsm, std::atomic<uint32_t> &smem_set, cudaStream_t s) {
     // the shared copy of the near bitmap (128 KB, or 2 x 64 KB per SM) pays
-    // once every warp has several steps to test with it
-    const bool near_sm = a.n >= (8u << 20);
+    // once the steps tested with it outweigh the copying (whole scans, with
+    // it and without: DNA 1 MiB 22.6 and 20.5 us, 2 MiB 22.2 and 21.8, 3 MiB
+    // 23.1 and 26.1, 8 MiB 26.8 and 39.8; bytes 1 MiB 12.3 and 12.3, 4 MiB
+    // 14.3 and 16.4, 8 MiB 14.4 and 18.6, though 16 files of 4 MB with their
+    // matches sorted took 337 and 329 us)
+    const bool near_sm = a.n >= (kind == SIEVE_DNA ? 3u : 8u) << 20;
     if (kind == SIEVE_DNA) {
         const uint32_t lists = kSieveList * 16;
         if (!near_sm) return launch_steps(sieve_dna<false, 1>, a, 512, 64, 16, 2 * lists, nsm, s);

@@ -1,5 +1,5 @@
 // Device building blocks of the sieve, shared by the single-text kernels
-// (sieve.cu) and the batch kernels (sieve_batch.cu).
+// (sieve.cu) and the batch kernels (flat_batch.cu).
 #pragma once
 
 #include "scan_device.cuh"
