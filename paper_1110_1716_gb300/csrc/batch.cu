@@ -319,15 +319,17 @@ static void plan_groups(const std::vector<uint32_t> &order, FlatPlan &pl) {
 }
 
 // Cuts the flat texts (jobs of machine slots with a class in flat_of) into
-// steps, sorted by class, machine and the caller's order. False where a class
-// has too many steps to number: the class kernels then take the whole batch.
+// steps, sorted by class, machine and the caller's order; texts without
+// symbols have no matches and are left out, so every text listed has a step.
+// False where a class has too many steps to number: the class kernels then
+// take the whole batch.
 static bool plan_flat(const pfsm_job *jobs, int32_t k, const std::vector<uint32_t> &job_slot,
                      const std::vector<int> &flat_of, const std::vector<Machine *> &machines, FlatPlan &pl) {
     uint64_t sieved = 0;
     std::vector<uint32_t> first(flat_of.size(), 0), order;
     for (int32_t i = 0; i < k; ++i) {
         const int c = flat_of[job_slot[i]];
-        if (c < 0) continue;
+        if (c < 0 || jobs[i].n == 0) continue;
         first[job_slot[i]]++;
         if (c != FLAT_WALK) sieved += jobs[i].n;
     }
@@ -349,7 +351,7 @@ static bool plan_flat(const pfsm_job *jobs, int32_t k, const std::vector<uint32_
     for (int32_t i = 0; i < k; ++i) {
         const uint32_t s = job_slot[i];
         const int c = flat_of[s];
-        if (c < 0) continue;
+        if (c < 0 || jobs[i].n == 0) continue;
         BatchJob &b = pl.jobs[first[s]++];
         b.text = jobs[i].text;
         b.n = static_cast<uint32_t>(jobs[i].n);
@@ -358,7 +360,7 @@ static bool plan_flat(const pfsm_job *jobs, int32_t k, const std::vector<uint32_
         const uint64_t step = flat_step(c, pl.big);
         // (the sieves' steps begin at 16-byte boundaries of the address space)
         const uint64_t shift = c == FLAT_WALK ? 0 : reinterpret_cast<uintptr_t>(b.text) & 15;
-        b.ntiles = b.n ? static_cast<uint32_t>((b.n + shift + step - 1) / step) : 0u;
+        b.ntiles = static_cast<uint32_t>((b.n + shift + step - 1) / step);
     }
     for (uint32_t s : order) {
         DevMachine &d = pl.machs[s];
@@ -368,7 +370,7 @@ static bool plan_flat(const pfsm_job *jobs, int32_t k, const std::vector<uint32_
     for (int c = 0; c < FLAT_CLASSES; ++c) {
         for (uint32_t j = pl.job_lo[c]; j < pl.job_hi[c]; ++j) {
             BatchJob &b = pl.jobs[j];
-            const uint64_t steps = b.ntiles ? static_cast<uint64_t>(b.ntiles) + flat_pad(pl.big) : 0u;
+            const uint64_t steps = static_cast<uint64_t>(b.ntiles) + flat_pad(pl.big);
             if (pl.steps[c] + steps >= (1ull << 31)) return false;
             b.unit_begin = static_cast<uint32_t>(pl.steps[c]);
             pl.steps[c] += steps;

@@ -66,9 +66,9 @@ __device__ __forceinline__ void flat_steps(const FlatArgs &A, FlatWarp &wa, uint
     for (uint32_t j = flat_job(A.jobs, A.job_lo[CLS], A.job_hi[CLS], s0, lane); s0 < s1; ++j) {
         const BatchJob &J = A.jobs[j];
         const DevMachine &M = A.machs[J.mach];
-        const uint32_t b0 = s0 - J.unit_begin, b1 = min(J.ntiles, b0 + (s1 - s0));
-        s0 = min(s1, J.unit_begin + J.ntiles + flat_pad(BIG));
-        if (b0 >= b1) continue;   // an empty text, or the padding after one
+        uint32_t b0, b1;
+        flat_take(J, BIG, s0, s1, b0, b1);
+        if (b0 >= b1) continue;   // the padding after a text
         __syncwarp();
         if (lane == 0) {
             if (CLS == FLAT_WALK) {

@@ -385,6 +385,17 @@ __host__ __device__ constexpr uint32_t flat_cost(int cls, bool big) {
 // first loads and its list's last entries are chains of dependent loads. Without
 // them a warp that is dealt a run of short texts keeps its CTA waiting.
 __host__ __device__ constexpr uint32_t flat_pad(bool big) { return big ? 3u : 0u; }
+// What a warp with the steps [s0, s1) of a class takes of the text J that s0
+// lies in (or in the padding after it): steps [b0, b1) of the text. s0 moves
+// on to the next text's first step: every text of a plan has steps, and the
+// padding after them (plan_flat).
+__host__ __device__ inline void flat_take(const BatchJob &J, bool big, uint32_t &s0, uint32_t s1, uint32_t &b0,
+                                          uint32_t &b1) {
+    b0 = s0 - J.unit_begin;
+    b1 = b0 + (s1 - s0) < J.ntiles ? b0 + (s1 - s0) : J.ntiles;
+    const uint32_t next = J.unit_begin + J.ntiles + flat_pad(big);
+    s0 = s1 < next ? s1 : next;
+}
 cudaError_t launch_flat(const FlatArgs &a, bool big, int nsm, std::atomic<uint32_t> &smem_set, cudaStream_t s);
 
 // ---- launch helpers (scan_kernels.cu) ------------------------------------

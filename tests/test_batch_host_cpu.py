@@ -1,0 +1,70 @@
+"""The host side of batches without a GPU (host_batch.cpp: csrc/batch.cu over
+stand-ins for the CUDA runtime, where launching the flat kernels replays how
+their warps take the steps of the texts)."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+DNA, BYTES, WALK = 0, 1, 2
+FIELDS = ("flat", "graph", "big", "groups", "steps", "missed", "bounds", "null_lists")
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("host") / "libhost_batch.so")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic",
+                    "-I" + os.path.join(cuda, "include"), "-I" + os.path.join(ROOT, "include"),
+                    "-I" + os.path.join(ROOT, "paper_1110_1716_gb300", "csrc"),
+                    os.path.join(HERE, "host_batch.cpp"), "-o", so, "-ldl"], check=True)
+    lib = ctypes.CDLL(so)
+    lib.hb_ctx.restype = ctypes.c_void_p
+    lib.hb_free.argtypes = [ctypes.c_void_p]
+    return lib
+
+
+class Host:
+    """A context over machines of the given flat classes."""
+
+    def __init__(self, lib, classes):
+        self.lib = lib
+        c = np.array(classes, dtype=np.int32)
+        self.ctx = ctypes.c_void_p(lib.hb_ctx(c.ctypes.data_as(ctypes.c_void_p), len(c)))
+
+    def scan(self, auts, lens, addrs=None):
+        a = np.array(auts, dtype=np.int32) + 1
+        n = np.array(lens, dtype=np.uint64)
+        t = np.array(addrs if addrs is not None else np.full(len(n), 1 << 20), dtype=np.uint64)
+        out = np.zeros(len(FIELDS), dtype=np.int64)
+        p = [x.ctypes.data_as(ctypes.c_void_p) for x in (a, t, n, out)]
+        st = self.lib.hb_scan(self.ctx, p[0], p[1], p[2], len(n), p[3])
+        return st, dict(zip(FIELDS, out.tolist()))
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *e):
+        self.lib.hb_free(self.ctx)
+
+
+@pytest.mark.parametrize("big", [False, True])
+@pytest.mark.parametrize("chunk", [1, 2, 5, 16, 1 << 20])
+def test_every_step_is_taken_once(lib, big, chunk):
+    """Texts of no, few and many steps in any order, whatever share of the
+    steps a warp is dealt."""
+    rng = np.random.default_rng(chunk + big)
+    lens = np.where(rng.random(600) < 0.4, 0, np.exp(rng.uniform(0, np.log(20_000), 600))).astype(np.int64)
+    auts = rng.integers(0, 9, 600)
+    if big:
+        lens = np.concatenate([lens, [5 << 20, 0, 4 << 20, 0]])
+        auts = np.concatenate([auts, [0, 0, 1, 1]])
+    lib.hb_chunk(chunk)
+    with Host(lib, [DNA, BYTES, WALK] * 3) as h:
+        st, got = h.scan(auts, lens, (1 << 20) + rng.integers(0, 64, len(lens)))
+    assert st == 0 and got["flat"] == 1 and got["graph"] == 0 and got["big"] == big
+    assert got["steps"] > 600 and got["missed"] == 0 and got["bounds"] == 0

@@ -146,3 +146,33 @@ def test_union_over_one_text(world):
     rows = out[:total].cpu().numpy().view(np.uint32)
     rows = rows[np.lexsort(rows.T[::-1])]
     assert np.array_equal(rows[:, 1:], np.concatenate(want))
+
+
+def late_start(m, n, seed):
+    """A text whose matches all begin in its first symbols (machines of plain
+    random tables: random symbols throughout)."""
+    aut, S, pats = m
+    if not pats:
+        return make_text(m, n, seed)
+    t = W.text_dna(n, seed) if S == 4 else np.random.default_rng(seed).integers(0, S, n).astype(np.uint8)
+    at, step = seed % 5, 512 if S == 4 else 2048
+    for i in range(3):
+        p = pats[(seed + i) % len(pats)]
+        t[at + i * step:at + i * step + len(p)] = p
+    return t
+
+
+def test_empty_texts_between_texts_of_a_large_batch(world):
+    """Past the size of the large form, an empty text before every text of
+    several steps, for machines of every class: matches in the first steps."""
+    pf, ms, auts, _, _, _ = world
+    jobs, texts, want = [], [], []
+    for i in range(1500):
+        j = (0, 3, 2, 5, 1, 4, 9)[i % 7]
+        t = late_start(ms[j], 5000 + 37 * (i % 211) + (8192 if ms[j][1] == 256 else 0), 3000 + i)
+        for u in (np.zeros(0, np.uint8), t):
+            jobs.append(j)
+            texts.append(u)
+            want.append(oracle.scan(ms[j][0], u))
+    assert sum(len(t) for j, t in zip(jobs, texts) if ms[j][2]) > 8 << 20
+    check(pf, auts, jobs, texts, want, ms)
