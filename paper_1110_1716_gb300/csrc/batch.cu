@@ -299,10 +299,12 @@ static int flat_class(const pfsm_ctx *ctx, const Machine &m) {
 }
 
 // Groups of machines (in `order`) that the whole chip scans one after the
-// other, in flat_cost units.
+// other, in flat_cost units. No batch has more than kFlatGroups: each group
+// but the last holds at least 1 / (kFlatGroups - 1) of the cost.
 static void plan_groups(const std::vector<uint32_t> &order, FlatPlan &pl) {
     uint64_t total = 0, base = 0;
     for (int c = 0; c < FLAT_CLASSES; ++c) total += pl.steps[c] * flat_cost(c, pl.big);
+    if (total == 0) return;   // only empty texts
     const uint64_t least = pl.big ? std::max<uint64_t>(kFlatGroupCost, total / (kFlatGroups - 1) + 1) : total;
     uint64_t from = 0;
     int last = FLAT_DNA;
@@ -310,7 +312,7 @@ static void plan_groups(const std::vector<uint32_t> &order, FlatPlan &pl) {
         const int c = pl.machs[s].flat;
         for (; last < c; ++last) base += pl.steps[last] * flat_cost(last, pl.big);
         const uint64_t end = base + pl.machs[s].flat_end * static_cast<uint64_t>(flat_cost(c, pl.big));
-        if (end - from >= least && total - end >= least) {
+        if (end - from >= least && total - end >= least && pl.groups + 1 < static_cast<uint32_t>(kFlatGroups)) {
             pl.group_end[pl.groups++] = end;
             from = end;
         }

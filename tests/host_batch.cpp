@@ -61,6 +61,7 @@ static struct Seen {
     int64_t steps, missed;    // flat steps of the texts; those not taken exactly once
     int64_t bounds;           // group bounds that do not ascend to the total
     int null_lists;           // a sieved flat launch without candidate lists
+    int64_t used;             // machines whose use was recorded
 } seen;
 static uint32_t chunk = 5;    // steps a warp takes
 
@@ -76,7 +77,7 @@ bool default_params(const Machine &) { return true; }
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 int ensure_words(uint32_t **, size_t *, size_t) { return PFSM_OK; }
 int make_resident(pfsm_ctx *, int, Machine &, cudaStream_t) { return PFSM_OK; }
-int mark_use(pfsm_ctx *, cudaStream_t, Machine *const *, size_t) { return PFSM_OK; }
+int mark_use(pfsm_ctx *, cudaStream_t, Machine *const *, size_t k) { return seen.used = static_cast<int64_t>(k), PFSM_OK; }
 Slot *get_slot(pfsm_ctx *, cudaStream_t) { return nullptr; }
 void collect_timing(pfsm_ctx *, Slot *, int) {}
 int finish_status(const unsigned long long *hs, uint64_t, uint64_t *n) { return *n = hs[0], PFSM_OK; }
@@ -154,7 +155,7 @@ int hb_scan(pfsm_ctx *c, const int32_t *aut, const uint64_t *text, const uint64_
     seen = Seen{};
     uint64_t total = 0;
     const int st = pfsm_scan_batch(c, jobs.data(), k, nullptr, 0, counts.data(), &total, nullptr);
-    const int64_t v[] = {seen.flat, seen.graph, seen.big, seen.groups, seen.steps, seen.missed, seen.bounds, seen.null_lists};
+    const int64_t v[] = {seen.flat, seen.graph, seen.big, seen.groups, seen.steps, seen.missed, seen.bounds, seen.null_lists, seen.used};
     memcpy(out, v, sizeof(v));
     return st;
 }

@@ -4,6 +4,7 @@ their warps take the steps of the texts)."""
 import ctypes
 import os
 import subprocess
+import traceback
 
 import numpy as np
 import pytest
@@ -11,14 +12,16 @@ import pytest
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 DNA, BYTES, WALK = 0, 1, 2
-FIELDS = ("flat", "graph", "big", "groups", "steps", "missed", "bounds", "null_lists")
+FIELDS = ("flat", "graph", "big", "groups", "steps", "missed", "bounds", "null_lists", "used")
 
 
 @pytest.fixture(scope="module")
 def lib(tmp_path_factory):
     so = str(tmp_path_factory.mktemp("host") / "libhost_batch.so")
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    # (an array index out of bounds traps)
     subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic",
+                    "-fsanitize=bounds", "-fsanitize-undefined-trap-on-error",
                     "-I" + os.path.join(cuda, "include"), "-I" + os.path.join(ROOT, "include"),
                     "-I" + os.path.join(ROOT, "paper_1110_1716_gb300", "csrc"),
                     os.path.join(HERE, "host_batch.cpp"), "-o", so, "-ldl"], check=True)
@@ -68,3 +71,32 @@ def test_every_step_is_taken_once(lib, big, chunk):
         st, got = h.scan(auts, lens, (1 << 20) + rng.integers(0, 64, len(lens)))
     assert st == 0 and got["flat"] == 1 and got["graph"] == 0 and got["big"] == big
     assert got["steps"] > 600 and got["missed"] == 0 and got["bounds"] == 0
+
+
+@pytest.mark.parametrize("machines", [1, 31, 32, 40, 200])
+@pytest.mark.parametrize("cls", [DNA, BYTES, WALK])
+def test_groups_of_machines_without_symbols(lib, machines, cls):
+    """More machines than groups, all or all but one of them with empty texts
+    only (in a child process: a trap ends it)."""
+    def run():
+        lib.hb_chunk(3)
+        with Host(lib, [cls] * machines) as h:
+            st, got = h.scan(list(range(machines)) * 2, [0] * (2 * machines))
+            assert st == 0 and got["flat"] == 0 and got["graph"] == 0 and got["used"] == machines
+            for n in (1, 777, 9 << 20):
+                st, got = h.scan(list(range(machines)) * 2, [0] * machines + [n] + [0] * (machines - 1))
+                assert st == 0 and got["flat"] == 1 and got["missed"] == 0 and got["bounds"] == 0
+                assert got["groups"] == 1
+            # as many bytes for every machine as the large form takes
+            st, got = h.scan(range(machines), [9 << 20] * machines)
+            assert st == 0 and got["missed"] == 0 and got["bounds"] == 0 and got["groups"] <= 32
+
+    pid = os.fork()
+    if pid == 0:
+        try:
+            run()
+            os._exit(0)
+        except BaseException:
+            traceback.print_exc()
+            os._exit(1)
+    assert os.waitpid(pid, 0)[1] == 0
