@@ -187,7 +187,8 @@ __global__ void __launch_bounds__(BIG ? 1024 : 128, 1) flat_front(const __grid_c
 
 // ------------------------------------------------------------ candidates
 // The match (start, end, st) of every lane with `has`, to the output and the
-// counts.
+// counts. (Rows are written word by word: the caller's buffer may begin at any
+// multiple of four bytes.)
 __device__ __forceinline__ void flat_emit(const FlatArgs &A, bool has, uint32_t orig, uint32_t start, uint32_t end,
                                           uint32_t st, int lane) {
     const uint32_t m = __ballot_sync(FULLMASK, has);
@@ -197,7 +198,13 @@ __device__ __forceinline__ void flat_emit(const FlatArgs &A, bool has, uint32_t 
     base = __shfl_sync(FULLMASK, base, 0) + __popc(m & lanemask_lt());
     if (has) {
         atomicAdd(&A.job_counts[orig], 1ull);
-        if (base < A.cap) reinterpret_cast<uint4 *>(A.out)[base] = make_uint4(orig, start, end, st);
+        if (base < A.cap) {
+            uint32_t *o = A.out + base * 4;
+            o[0] = orig;
+            o[1] = start;
+            o[2] = end;
+            o[3] = st;
+        }
     }
 }
 

@@ -176,3 +176,30 @@ def test_empty_texts_between_texts_of_a_large_batch(world):
             want.append(oracle.scan(ms[j][0], u))
     assert sum(len(t) for j, t in zip(jobs, texts) if ms[j][2]) > 8 << 20
     check(pf, auts, jobs, texts, want, ms)
+
+
+@pytest.mark.parametrize("words", [1, 2, 3])
+def test_rows_at_any_word(world, words):
+    """Output rows that begin 4, 8 and 12 bytes past a 16-byte boundary, for a
+    batch and for a union, with nothing written around them."""
+    pf, ms, auts, jobs, texts, want = world
+    data = [pf.to_device(t) for t in texts]
+    u = make_text(ms[1], 50_001, 5)
+    ud = pf.to_device(u)
+    picks = [0, 1, 2, 5]
+    parts = [oracle.scan(ms[j][0], u) for j in picks]
+    for rows in (want, parts):
+        total = sum(len(w) for w in rows)
+        buf = torch.full((4 * total + 8,), -7, dtype=torch.int32, device="cuda")
+        assert buf.data_ptr() % 16 == 0
+        out = buf[words:words + 4 * total].view(total, 4)
+        if rows is want:
+            st, counts, got = P.pfsm_scan_batch(pf.ctx, [(auts[j], d, d.numel()) for j, d in zip(jobs, data)], out)
+        else:
+            st, counts, got = P.pfsm_scan_union(pf.ctx, [auts[j] for j in picks], ud, None, out)
+        assert st == P.PFSM_OK and got == total and counts.tolist() == [len(w) for w in rows]
+        m = out.cpu().numpy().view(np.uint32)
+        m = m[np.lexsort(m.T[::-1])]
+        assert np.array_equal(m[:, 0], np.repeat(np.arange(len(rows)), [len(w) for w in rows]))
+        assert np.array_equal(m[:, 1:], np.concatenate(rows))
+        assert (buf[:words] == -7).all() and (buf[words + 4 * total:] == -7).all()
