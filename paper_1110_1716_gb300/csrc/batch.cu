@@ -104,7 +104,10 @@ void batch_free(pfsm_ctx *ctx) {
 
 static int state_reserve(pfsm_ctx *ctx, cudaStream_t s, size_t njobs, size_t nmachs,
                          BatchState **out) {
-    BatchState *&b = ctx->batch[s];
+    // (a state is entered when it is whole: after a failure the next call
+    // starts anew)
+    const auto it = ctx->batch.find(s);
+    BatchState *b = it == ctx->batch.end() ? nullptr : it->second;
     if (!b) {
         b = new BatchState();
         bool ok = cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking) == cudaSuccess &&
@@ -113,15 +116,15 @@ static int state_reserve(pfsm_ctx *ctx, cudaStream_t s, size_t njobs, size_t nma
         for (int c = 0; ok && c < kBatchClasses; ++c)
             ok = cudaStreamCreateWithFlags(&b->aux[c], cudaStreamNonBlocking) == cudaSuccess &&
                  cudaEventCreateWithFlags(&b->join[c], cudaEventDisableTiming) == cudaSuccess;
-        if (!ok) {
+        const int st = !ok ? PFSM_E_CUDA
+                       : cudaMalloc(&b->cand, 2ull * kFlatCand * sizeof(uint4)) != cudaSuccess ? PFSM_E_NOMEM
+                                                                                               : PFSM_OK;
+        if (st) {
             cudaGetLastError();
-            return PFSM_E_CUDA;
+            state_free(b);
+            return st;
         }
-        if (cudaMalloc(&b->cand, 2ull * kFlatCand * sizeof(uint4)) != cudaSuccess) {
-            cudaGetLastError();
-            b->cand = nullptr;
-            return PFSM_E_NOMEM;
-        }
+        ctx->batch[s] = b;
     }
     if (njobs <= b->cap_jobs && nmachs <= b->cap_machs) {
         *out = b;

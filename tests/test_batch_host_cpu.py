@@ -12,6 +12,7 @@ import pytest
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 DNA, BYTES, WALK = 0, 1, 2
+E_NOMEM = 2
 FIELDS = ("flat", "graph", "big", "groups", "steps", "missed", "bounds", "null_lists", "used")
 
 
@@ -100,3 +101,18 @@ def test_groups_of_machines_without_symbols(lib, machines, cls):
             traceback.print_exc()
             os._exit(1)
     assert os.waitpid(pid, 0)[1] == 0
+
+
+@pytest.mark.parametrize("nth", range(1, 9))
+@pytest.mark.parametrize("cls", [DNA, BYTES, WALK])
+def test_a_call_after_one_that_found_no_memory(lib, nth, cls):
+    """The nth device allocation of a batch fails, on a new stream and where
+    its buffers grow: the next call allocates what is missing."""
+    with Host(lib, [cls]) as h:
+        for jobs in (3, 700, 3000):
+            lib.hb_fail(nth)
+            st, got = h.scan([0] * jobs, [5000] * jobs)
+            lib.hb_fail(0)
+            assert st in (0, E_NOMEM) and got["flat"] == (st == 0) and got["null_lists"] == 0
+            st, got = h.scan([0] * jobs, [5000] * jobs)
+            assert st == 0 and got["flat"] == 1 and got["null_lists"] == 0 and got["missed"] == 0
