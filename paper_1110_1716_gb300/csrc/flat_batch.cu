@@ -418,24 +418,30 @@ __global__ void __launch_bounds__(256) flat_finish(const __grid_constant__ FlatA
         }
         return;
     }
-    for (int c = 0; c < FLAT_WALK; ++c)
-        for (uint64_t j = A.job_lo[c] + me; j < A.job_hi[c]; j += warps) {
+    // step by step, dealt out in turn: texts may be long, and what a start
+    // costs differs from place to place
+    for (int c = 0; c < FLAT_WALK; ++c) {
+        const uint64_t span = flat_step(c, false);   // (the same in both forms)
+        for (uint64_t x = me; x < A.steps[c]; x += warps) {
+            const uint32_t j = flat_job(A.jobs, A.job_lo[c], A.job_hi[c], static_cast<uint32_t>(x), lane);
             const BatchJob &J = A.jobs[j];
             const DevMachine &M = A.machs[J.mach];
+            const uint64_t from = (x - J.unit_begin) * span, to = min(static_cast<uint64_t>(J.n), from + span);
             if (static_cast<uint32_t>(M.kind) != kind) continue;
-            for (uint64_t s0 = 0; s0 < J.n; s0 += 32) {
+            for (uint64_t s0 = from; s0 < to; s0 += 32) {   // (none in the padding after a text)
                 const uint32_t start = static_cast<uint32_t>(s0) + lane;
-                bool act = start < J.n;
+                bool act = s0 + lane < to;
                 uint32_t rec = SIEVE_NO_RECORD;
                 if (kind == 1 && act) {
                     rec = flat_record(M, J, start, pol_keep);
                     act = rec != SIEVE_NO_RECORD;
                 }
                 if (!__any_sync(FULLMASK, act)) continue;
-                if (kind == 0) flat_dfa(A, act, static_cast<uint32_t>(j), start, lane, pol_keep);
-                else flat_nfa(A, act, static_cast<uint32_t>(j), start, rec, items, lane);
+                if (kind == 0) flat_dfa(A, act, j, start, lane, pol_keep);
+                else flat_nfa(A, act, j, start, rec, items, lane);
             }
         }
+    }
 }
 
 // ------------------------------------------------------------ host helpers

@@ -203,3 +203,21 @@ def test_rows_at_any_word(world, words):
         assert np.array_equal(m[:, 0], np.repeat(np.arange(len(rows)), [len(w) for w in rows]))
         assert np.array_equal(m[:, 1:], np.concatenate(rows))
         assert (buf[:words] == -7).all() and (buf[words + 4 * total:] == -7).all()
+
+
+@pytest.mark.parametrize("n", [300_001, 9_500_003])
+def test_candidate_lists_overflow_in_long_texts(world, n):
+    """Lists that overflow in texts of many steps, beside texts of few: every
+    start is run, step by step, in both forms of the front kernel."""
+    pf, ms, auts, jobs, texts, want = world
+    jobs, texts, want = list(jobs[:40]), list(texts[:40]), list(want[:40])
+    for k, (j, m) in enumerate([(1, n), (4, n - 7), (2, n // 3), (3, 4097), (0, 513)]):
+        t = make_text(ms[j], m, 91 + k)
+        jobs.insert(7 * k, j)
+        texts.insert(7 * k, t)
+        want.insert(7 * k, oracle.scan(ms[j][0], t))
+    P.pfsm_test_carry_cap(pf.ctx, 1000, 0)
+    try:
+        check(pf, auts, jobs, texts, want, ms)
+    finally:
+        P.pfsm_test_carry_cap(pf.ctx, 0, 0)
