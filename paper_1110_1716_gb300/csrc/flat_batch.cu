@@ -197,7 +197,9 @@ __device__ __forceinline__ void flat_emit(const FlatArgs &A, bool has, uint32_t 
     if (lane == 0) base = atomicAdd(&A.status[0], static_cast<unsigned long long>(__popc(m)));
     base = __shfl_sync(FULLMASK, base, 0) + __popc(m & lanemask_lt());
     if (has) {
-        atomicAdd(&A.job_counts[orig], 1ull);
+        // one atomic per text: neighbouring candidates mostly share theirs
+        const uint32_t peers = __match_any_sync(m, orig);
+        if (lane == __ffs(peers) - 1) atomicAdd(&A.job_counts[orig], static_cast<unsigned long long>(__popc(peers)));
         if (base < A.cap) {
             uint32_t *o = A.out + base * 4;
             o[0] = orig;
