@@ -382,27 +382,89 @@ __device__ __forceinline__ void flat_nfa(const FlatArgs &A, bool act, uint32_t j
     __syncwarp();
 }
 
-// The record of an NFA start (as sieve_levels finds it), or SIEVE_NO_RECORD.
-__device__ __forceinline__ uint32_t flat_record(const DevMachine &M, const BatchJob &J, uint32_t start, uint64_t pol_keep) {
-    const uint32_t rest = J.n - start, kk = static_cast<uint32_t>(M.k);
-    if (rest < M.min_match) return SIEVE_NO_RECORD;
-    uint32_t g0, g1;
-    pack32_at(J.text, J.n, start, g0, g1);
-    if (rest < 16) g0 &= (1u << (2 * rest)) - 1;
-    if (rest >= SIEVE_DEEP_M) {
-        const uint32_t d = g0 & ((1u << (2 * SIEVE_DEEP_M)) - 1);
-        if (!((ldg_u32_keep(M.surv2 + (d >> 5), pol_keep) >> (d & 31)) & 1u)) return SIEVE_NO_RECORD;
+// Candidates of the fallback, collected per warp: starts that pass the deep
+// bitmap, then those with a record.
+struct FlatEvery {
+    uint2 starts[64];      // {start, its first 16 symbols}
+    uint4 found[64];       // as the list of the front kernel has them
+    uint32_t n;            // entries of found
+};
+
+// Every start of one NFA's steps [b0, b1), as the front kernel and the list
+// would have brought them: four starts per lane through the bitmap of single
+// starts, then the records and the runs of full warps of what is left. (Runs
+// of the one start in twenty that has a record, 32 starts at a time, left the
+// other lanes idle: 64 MiB dense in motifs 8.3 ms.)
+static __device__ __noinline__ void flat_every_nfa(const FlatArgs &A, uint32_t j, uint32_t b0, uint32_t b1, FlatEvery &E,
+                                               uint4 *items, int lane, uint64_t pol_keep) {
+    const BatchJob &J = A.jobs[j];
+    const DevMachine &M = A.machs[J.mach];
+    constexpr uint32_t SPAN = flat_step(FLAT_DNA, false);
+    SieveArgs a{};
+    a.text = J.text;
+    a.n = J.n;
+    a.k = M.k;
+    a.min_match = M.min_match;
+    a.memox = M.memox;
+    a.l2tab = M.l2tab;
+    a.l3 = M.sv_l3;
+    a.job = j;
+    a.cand = reinterpret_cast<uint2 *>(E.found);
+    a.cand_n = &E.n;
+    a.cand_cap = 64;
+    const uint32_t *surv2 = M.surv2;
+    uint32_t cnt = 0;   // entries of E.starts
+    // runs the last entries of E.found, full warps of them (all at the end)
+    auto run = [&](bool all) {
+        __syncwarp();
+        uint32_t n = *static_cast<volatile uint32_t *>(&E.n);
+        while (n >= 32 || (all && n)) {
+            const uint32_t k = min(n, 32u);
+            n -= k;
+            const uint4 c = E.found[n + min(static_cast<uint32_t>(lane), k - 1)];
+            flat_nfa(A, static_cast<uint32_t>(lane) < k, c.x, c.y, c.z, items, lane);
+        }
+        if (lane == 0) E.n = n;
+        __syncwarp();
+    };
+    const uint64_t to = min(static_cast<uint64_t>(J.n), static_cast<uint64_t>(b1) * SPAN);
+    for (uint64_t s0 = static_cast<uint64_t>(b0) * SPAN; s0 < to; s0 += 128) {
+        const uint64_t first = s0 + 4 * lane;
+        uint32_t g0 = 0, g1 = 0, keep = 0;
+        if (first < to) {
+            pack32_at(a.text, a.n, static_cast<uint32_t>(first), g0, g1);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const uint32_t g = __funnelshift_r(g0, g1, 2 * r) & ((1u << (2 * SIEVE_DEEP_M)) - 1);
+                const uint32_t w = first + r + SIEVE_DEEP_M <= a.n ? ldg_u32_keep(surv2 + (g >> 5), pol_keep) >> (g & 31) : 1u;
+                keep |= (first + r < to ? w & 1u : 0u) << r;
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const uint32_t m = __ballot_sync(FULLMASK, (keep >> r) & 1u);
+            if ((keep >> r) & 1u)
+                E.starts[cnt + __popc(m & lanemask_lt())] =
+                    make_uint2(static_cast<uint32_t>(first) + r, __funnelshift_r(g0, g1, 2 * r));
+            cnt += __popc(m);
+            if (cnt >= 32) {
+                cnt -= 32;
+                __syncwarp();
+                sieve_levels<true>(a, E.starts + cnt, 32, lane, pol_keep);
+                run(false);
+            }
+        }
     }
-    const uint32_t x = ldg_u16_keep(M.memox + (g0 & ((1u << (2 * kk)) - 1)), pol_keep);
-    if (x == L2_NONE) return SIEVE_NO_RECORD;
-    const uint32_t o2 = ldg_u16_keep(M.l2tab + x * L2_GRAMS + ((g0 >> (2 * kk)) & (L2_GRAMS - 1)), pol_keep);
-    return o2 == L2_EMPTY ? SIEVE_NO_RECORD : o2;
+    __syncwarp();
+    if (cnt) sieve_levels<true>(a, E.starts, cnt, lane, pol_keep);
+    run(true);
 }
 
 // Even CTAs run the DFA candidates, odd ones the NFA candidates. A list that
 // overflowed is replaced by every start of the texts of its kind.
-__global__ void __launch_bounds__(256) flat_finish(const __grid_constant__ FlatArgs A) {
+__global__ void __launch_bounds__(256, 4) flat_finish(const __grid_constant__ FlatArgs A) {
     __shared__ uint4 items_sm[8][32 * SIEVE_PARTS];
+    __shared__ FlatEvery every_sm[8];
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint64_t pol_keep = policy_evict_last();
@@ -420,27 +482,27 @@ __global__ void __launch_bounds__(256) flat_finish(const __grid_constant__ FlatA
         }
         return;
     }
-    // step by step, dealt out in turn: texts may be long, and what a start
-    // costs differs from place to place
+    // a few steps at a time, dealt out in turn: texts may be long, and what a
+    // start costs differs from place to place
+    if (lane == 0) every_sm[wid].n = 0;
     for (int c = 0; c < FLAT_WALK; ++c) {
         const uint64_t span = flat_step(c, false);   // (the same in both forms)
-        for (uint64_t x = me; x < A.steps[c]; x += warps) {
-            const uint32_t j = flat_job(A.jobs, A.job_lo[c], A.job_hi[c], static_cast<uint32_t>(x), lane);
-            const BatchJob &J = A.jobs[j];
-            const DevMachine &M = A.machs[J.mach];
-            const uint64_t from = (x - J.unit_begin) * span, to = min(static_cast<uint64_t>(J.n), from + span);
-            if (static_cast<uint32_t>(M.kind) != kind) continue;
-            for (uint64_t s0 = from; s0 < to; s0 += 32) {   // (none in the padding after a text)
-                const uint32_t start = static_cast<uint32_t>(s0) + lane;
-                bool act = s0 + lane < to;
-                uint32_t rec = SIEVE_NO_RECORD;
-                if (kind == 1 && act) {
-                    rec = flat_record(M, J, start, pol_keep);
-                    act = rec != SIEVE_NO_RECORD;
+        const uint32_t steps = static_cast<uint32_t>(A.steps[c]), each = kind == 0 ? 1u : 8u;
+        for (uint64_t x = me * each; x < steps; x += warps * each) {
+            uint32_t s0 = static_cast<uint32_t>(x);
+            const uint32_t s1 = static_cast<uint32_t>(min(static_cast<uint64_t>(steps), x + each));
+            for (uint32_t j = flat_job(A.jobs, A.job_lo[c], A.job_hi[c], s0, lane); s0 < s1; ++j) {
+                const BatchJob &J = A.jobs[j];
+                const uint32_t b0 = s0 - J.unit_begin, b1 = min(J.ntiles, b0 + (s1 - s0));
+                s0 = j + 1 < A.job_hi[c] ? min(s1, A.jobs[j + 1].unit_begin) : s1;
+                if (b0 >= b1 || static_cast<uint32_t>(A.machs[J.mach].kind) != kind) continue;
+                if (kind == 1) {
+                    flat_every_nfa(A, j, b0, b1, every_sm[wid], items, lane, pol_keep);
+                    continue;
                 }
-                if (!__any_sync(FULLMASK, act)) continue;
-                if (kind == 0) flat_dfa(A, act, j, start, lane, pol_keep);
-                else flat_nfa(A, act, j, start, rec, items, lane);
+                const uint64_t to = min(static_cast<uint64_t>(J.n), b1 * span);
+                for (uint64_t at = b0 * span; at < to; at += 32)
+                    flat_dfa(A, at + lane < to, j, static_cast<uint32_t>(at) + lane, lane, pol_keep);
             }
         }
     }
