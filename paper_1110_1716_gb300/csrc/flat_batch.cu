@@ -27,8 +27,6 @@
 
 namespace pfsm {
 
-constexpr uint32_t kFlatStage = 96;   // direct scans: staged matches per warp and half
-
 // Last job of [lo, hi) whose first step is <= x (every lane calls it).
 __device__ __forceinline__ uint32_t flat_job(const BatchJob *jobs, uint32_t lo, uint32_t hi, uint32_t x, int lane) {
     while (hi - lo > 1) {
@@ -52,12 +50,8 @@ template <int CLS, bool BIG>
 __device__ __forceinline__ void flat_steps(const FlatArgs &A, FlatWarp &wa, uint32_t s0, uint32_t s1, int wid, int lane,
                                            uint64_t pol_keep) {
     if (s0 >= s1) return;
-    // the near bitmap at offset 0 of the shared memory, then the warps' lists;
-    // direct scans have their match buffers there instead
-    const uint8_t *near = pfsm_dyn_smem;
-    constexpr uint32_t lists = BIG && CLS != FLAT_WALK ? (1u << (2 * SIEVE_NEAR_M)) / 8 : 0u;
-    constexpr uint32_t each = CLS == FLAT_WALK ? 2 * kFlatStage * 16 : kSieveList * 16;
-    uint8_t *own = pfsm_dyn_smem + lists + wid * each;
+    const uint8_t *near = pfsm_dyn_smem;   // BIG: the near bitmap
+    uint8_t *own = pfsm_dyn_smem + flat_own(CLS, BIG, wid);
     uint32_t *list = reinterpret_cast<uint32_t *>(own);
     uint2 *list2 = reinterpret_cast<uint2 *>(list + kSieveList * 2);
     uint32_t cnt = 0, cnt2 = 0;
@@ -514,8 +508,8 @@ cudaError_t launch_flat(const FlatArgs &a, bool big, int nsm, std::atomic<uint32
     for (int c = 0; c < FLAT_CLASSES; ++c) steps += a.steps[c];
     if (steps == 0) return cudaSuccess;
     if (big) {
-        constexpr uint32_t smem = (1u << (2 * SIEVE_NEAR_M)) / 8 + 32 * kSieveList * 16;
-        static_assert(smem >= 32 * 2 * kFlatStage * 16, "the match buffers fit the sieve's regions");
+        constexpr uint32_t smem = flat_own(FLAT_DNA, true, 32);
+        static_assert(smem >= flat_own(FLAT_WALK, true, 32), "the match buffers fit the sieve's regions");
         if (!(smem_set.load(std::memory_order_relaxed) >> 9 & 1u)) {
             const cudaError_t e = cudaFuncSetAttribute(flat_front<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
             if (e != cudaSuccess) return e;
@@ -523,8 +517,7 @@ cudaError_t launch_flat(const FlatArgs &a, bool big, int nsm, std::atomic<uint32
         }
         flat_front<true><<<nsm, 1024, smem, s>>>(a);
     } else {
-        constexpr uint32_t smem = 4 * 2 * kFlatStage * 16;
-        static_assert(smem >= 4 * kSieveList * 16, "the lists fit the match buffers");
+        constexpr uint32_t smem = flat_own(FLAT_WALK, false, 4);
         const int grid = static_cast<int>(std::min<uint64_t>((steps + 3) / 4, 8ull * nsm));
         flat_front<false><<<grid, 128, smem, s>>>(a);
     }

@@ -96,6 +96,7 @@ constexpr int SIEVE_NONE = 0, SIEVE_DNA = 1, SIEVE_BYTES = 2;
 constexpr int SIEVE_NEAR_M = 10;     // 128 KB: what a CTA's shared memory holds
 constexpr int SIEVE_DEEP_M = 13;     // 8 MB in L2
 constexpr int SIEVE_HASH_BITS = 19;  // 64 KB: three CTAs per SM
+constexpr int kSieveList = 64;       // a warp's list: refined by 32, up to 32 more at a time
 constexpr int SIEVE_PARTS = 3;       // strands of a record's set that a lane takes
 constexpr uint32_t SIEVE_NO_RECORD = 0xFFFFFFFFu;   // a candidate without a second-level record
 constexpr uint32_t SIEVE_HASH_MAX = 1u << (SIEVE_HASH_BITS - 4);   // most bits set
@@ -385,6 +386,20 @@ __host__ __device__ constexpr uint32_t flat_cost(int cls, bool big) {
 // first loads and its list's last entries are chains of dependent loads. Without
 // them a warp that is dealt a run of short texts keeps its CTA waiting.
 __host__ __device__ constexpr uint32_t flat_pad(bool big) { return big ? 3u : 0u; }
+// Shared memory of flat_front: each warp's own region, its lists (sieves) or
+// its match buffers (direct scans). Small form: the warps of a CTA pass from
+// one class to the next on their own, so a warp's region is the same one for
+// every class. Large form: they meet where the class changes; the near bitmap
+// comes first and the lists lie behind it.
+constexpr uint32_t kFlatStage = 96;   // direct scans: staged matches per warp and half
+__host__ __device__ constexpr uint32_t flat_own_bytes(int cls) {
+    return cls == FLAT_WALK ? 2 * kFlatStage * 16 : kSieveList * 16;
+}
+__host__ __device__ constexpr uint32_t flat_own(int cls, bool big, uint32_t warp) {
+    return big && cls != FLAT_WALK ? (1u << (2 * SIEVE_NEAR_M)) / 8 + warp * flat_own_bytes(cls)
+                                   : warp * flat_own_bytes(FLAT_WALK);
+}
+static_assert(flat_own_bytes(FLAT_DNA) <= flat_own_bytes(FLAT_WALK), "a warp's lists fit its region");
 // What a warp with the steps [s0, s1) of a class takes of the text J that s0
 // lies in (or in the padding after it): steps [b0, b1) of the text. s0 moves
 // on to the next text's first step: every text of a plan has steps, and the

@@ -7,7 +7,6 @@
 namespace pfsm {
 
 constexpr uint32_t kSpan = 2048;   // bytes a warp tests per step: 4 x 16 per lane
-constexpr int kSieveList = 64;       // a warp's list: refined by 32, up to 32 more at a time
 
 __device__ __forceinline__ uint4 ldg_stream(const uint8_t *p) {
     uint4 v;

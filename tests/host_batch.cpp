@@ -145,6 +145,11 @@ void hb_free(pfsm_ctx *c) {
     batch_free(c);
     delete c;
 }
+// The shared memory of a warp of flat_front for class c: {from, to}.
+void hb_own(int32_t c, int32_t big, uint32_t warp, uint32_t *range) {
+    range[0] = flat_own(c, big != 0, warp);
+    range[1] = range[0] + flat_own_bytes(c);
+}
 void hb_fail(int n) { fail_in = n; }
 void hb_chunk(uint32_t n) { chunk = n; }
 // One batch of texts of n[i] symbols at address text[i] for machine aut[i].

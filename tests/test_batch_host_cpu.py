@@ -116,3 +116,31 @@ def test_a_call_after_one_that_found_no_memory(lib, nth, cls):
             assert st in (0, E_NOMEM) and got["flat"] == (st == 0) and got["null_lists"] == 0
             st, got = h.scan([0] * jobs, [5000] * jobs)
             assert st == 0 and got["flat"] == 1 and got["null_lists"] == 0 and got["missed"] == 0
+
+
+def own(lib, cls, big, warp):
+    r = np.zeros(2, dtype=np.uint32)
+    lib.hb_own(cls, int(big), warp, r.ctypes.data_as(ctypes.c_void_p))
+    return r
+
+
+def apart(x, y):
+    return x[1] <= y[0] or y[1] <= x[0]
+
+
+def test_warps_of_the_front_kernel_do_not_share_memory(lib):
+    """Small form: nothing keeps the warps of a CTA in the same class, so one
+    warp's region for any class lies apart from another's for any class. Large
+    form: the warps meet where the class changes; the sieves' lists lie past
+    the 128 KB of the near bitmap."""
+    classes = (DNA, BYTES, WALK)
+    for w in range(4):
+        for v in range(4):
+            for c in classes:
+                for d in classes:
+                    assert v == w or apart(own(lib, c, False, w), own(lib, d, False, v)), (w, c, v, d)
+    for c in classes:
+        regions = [own(lib, c, True, w) for w in range(32)]
+        assert all(apart(regions[w], regions[v]) for w in range(32) for v in range(w))
+        assert c == WALK or min(r[0] for r in regions) >= 128 << 10
+        assert max(r[1] for r in regions) <= (128 << 10) + 32 * 1024
