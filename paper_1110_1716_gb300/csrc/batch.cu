@@ -29,7 +29,7 @@ constexpr uint32_t kMinArena = 8192;     // smallest table arena worth a class s
 constexpr int kUnitTilesMax = 8;        // tiles per work unit, at most
 constexpr int kCarryCtr = 15;           // counter word holding the carry count
 constexpr uint32_t kAllClasses = (1u << kBatchClasses) - 1;
-constexpr int kFlatCtr = 16;            // counter words holding the flat batches' candidate counts
+constexpr int kFlatCtr = 16;            // counter words holding the flat batches' candidate counts (64 bits each)
 // symbols of a batch's sieved texts from which the kernel with the near
 // bitmaps in shared memory is taken (each of its CTAs copies 128 KB per
 // machine it meets). 64 texts, 4 motif sets, whole calls: 4 MiB 64 us (62
@@ -629,7 +629,7 @@ static int batch_enqueue(pfsm_ctx *ctx, const pfsm_job *jobs, int32_t k, pfsm_bm
         f.job_counts = b->status + 2;
         f.cand[0] = b->cand;
         f.cand[1] = b->cand + kFlatCand;
-        f.cand_n = b->ctr + kFlatCtr;
+        f.cand_n = reinterpret_cast<unsigned long long *>(b->ctr + kFlatCtr);
         f.cand_cap = ctx->test_carry_cap ? std::min(kFlatCand, ctx->test_carry_cap) : kFlatCand;
         return launch_flat(f, pl.flat.big, ctx->nsm, ctx->smem_set, s) == cudaSuccess ? PFSM_OK : PFSM_E_CUDA;
     };

@@ -97,7 +97,7 @@ __device__ __forceinline__ void flat_steps(const FlatArgs &A, FlatWarp &wa, uint
                 a.min_match = M.min_match;
                 a.job = j;
                 a.cand = reinterpret_cast<uint2 *>(A.cand[M.kind]);
-                a.cand_n = A.cand_n + M.kind;
+                a.cand_sum = A.cand_n + M.kind;
                 a.cand_cap = A.cand_cap;
             }
         }
@@ -400,7 +400,7 @@ __device__ __forceinline__ void flat_nfa(const FlatArgs &A, FlatOut &out, bool a
 struct FlatEvery {
     uint2 starts[64];      // {start, its first 16 symbols}
     uint4 found[64];       // as the list of the front kernel has them
-    uint32_t n;            // entries of found
+    unsigned long long n;  // entries of found
 };
 
 // Every start of one NFA's steps [b0, b1), as the front kernel and the list
@@ -423,14 +423,14 @@ static __device__ __noinline__ void flat_every_nfa(const FlatArgs &A, uint32_t j
     a.l3 = M.sv_l3;
     a.job = j;
     a.cand = reinterpret_cast<uint2 *>(E.found);
-    a.cand_n = &E.n;
+    a.cand_sum = &E.n;
     a.cand_cap = 64;
     const uint32_t *surv2 = M.surv2;
     uint32_t cnt = 0;   // entries of E.starts
     // runs the last entries of E.found, full warps of them (all at the end)
     auto run = [&](bool all) {
         __syncwarp();
-        uint32_t n = *static_cast<volatile uint32_t *>(&E.n);
+        uint32_t n = static_cast<uint32_t>(*static_cast<volatile unsigned long long *>(&E.n));
         while (n >= 32 || (all && n)) {
             const uint32_t k = min(n, 32u);
             n -= k;
@@ -483,12 +483,12 @@ __global__ void __launch_bounds__(256, 4) flat_finish(const __grid_constant__ Fl
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint64_t pol_keep = policy_evict_last();
     const uint32_t kind = blockIdx.x & 1, ctas = gridDim.x / 2;
-    const uint32_t found = A.cand_n[kind];
+    const unsigned long long found = A.cand_n[kind];
     const uint64_t warps = static_cast<uint64_t>(ctas) * 8, me = static_cast<uint64_t>(wid) * ctas + blockIdx.x / 2;
     uint4 *items = items_sm[wid];
     FlatOut out{rows_sm[wid], 0u};
     if (found <= A.cand_cap) {
-        const uint32_t per = static_cast<uint32_t>(min(static_cast<uint64_t>(32), (found + warps - 1) / warps));
+        const uint32_t per = static_cast<uint32_t>(min(32ull, (found + warps - 1) / warps));
         for (uint64_t x0 = me * per; x0 < found; x0 += warps * per) {
             const bool act = static_cast<uint32_t>(lane) < per && x0 + lane < found;
             const uint4 c = act ? A.cand[kind][x0 + lane] : A.cand[kind][x0];

@@ -219,6 +219,7 @@ struct SieveArgs {
     uint2 *cand;                   // candidates, cand_cap of them: start and second-level
                                    // record (or SIEVE_NO_RECORD)
     uint32_t *cand_n;              // their number (past cand_cap: the list is incomplete)
+    unsigned long long *cand_sum;  // batch: their number (the texts of a batch may have more than 2^32)
     uint32_t cand_cap;
     uint32_t *out;
     uint64_t cap;
@@ -370,7 +371,7 @@ struct FlatArgs {
     uint64_t cap;
     unsigned long long *status, *job_counts;
     uint4 *cand[2];            // DFA, NFA
-    uint32_t *cand_n;          // [2]
+    unsigned long long *cand_n;   // [2]
     uint32_t cand_cap;
 };
 // bytes or starts per step

@@ -64,7 +64,14 @@ __device__ __forceinline__ void sieve_append(const SieveArgs &a, uint32_t keep, 
     const uint32_t total = __shfl_sync(FULLMASK, incl, 31);
     if (total == 0) return;
     uint32_t at = 0;
-    if (lane == 0) at = atomicAdd(a.cand_n, total);
+    if (lane == 0) {
+        if (BATCH) {
+            const unsigned long long n = atomicAdd(a.cand_sum, static_cast<unsigned long long>(total));
+            at = n < a.cand_cap ? static_cast<uint32_t>(n) : a.cand_cap;   // (and at most 128 more)
+        } else {
+            at = atomicAdd(a.cand_n, total);
+        }
+    }
     at = __shfl_sync(FULLMASK, at, 0) + incl - __popc(keep);
     while (keep) {
         const uint32_t r = __ffs(keep) - 1;

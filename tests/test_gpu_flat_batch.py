@@ -221,3 +221,25 @@ def test_candidate_lists_overflow_in_long_texts(world, n):
         check(pf, auts, jobs, texts, want, ms)
     finally:
         P.pfsm_test_carry_cap(pf.ctx, 0, 0)
+
+
+def test_more_candidates_than_32_bits_count(world):
+    """Four texts of 1 GiB and one of 1 MiB whose starts are nearly all
+    candidates: more than 2^32 of them, a list's length more than a multiple of
+    it."""
+    pf = world[0]
+    trie, _ = W.trie_dfa([bytes(7) + b"\x01"])
+    a = pf.load(trie)
+    n, m = 1 << 30, 1 << 20
+    text = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    ends = np.array([7, 4099, 12_345_678, 500_000_003, n - 1])
+    text[torch.from_numpy(ends).cuda()] = 1
+    jobs = [(a, text, n)] * 4 + [(a, text[4096:4096 + m], m)]
+    want = [[(int(e) - 7, int(e)) for e in ends]] * 4 + [[]]   # (a match begins before the last text)
+    total = sum(len(w) for w in want)
+    out = torch.empty((total + 8, 4), dtype=torch.int32, device="cuda")
+    st, counts, got = P.pfsm_scan_batch(pf.ctx, jobs, out)
+    P.pfsm_unload(pf.ctx, a)
+    assert st == P.PFSM_OK and got == total and counts.tolist() == [len(w) for w in want]
+    rows = sorted(map(tuple, out[:total, :3].tolist()))
+    assert rows == [(i, s, e) for i, w in enumerate(want) for s, e in w]
