@@ -102,30 +102,48 @@ void batch_free(pfsm_ctx *ctx) {
     ctx->batch.clear();
 }
 
+// The batch state of stream `s`. A state is entered when it is whole: after a
+// failure the next call starts anew.
+static int state_of(pfsm_ctx *ctx, cudaStream_t s, BatchState **out) {
+    const auto it = ctx->batch.find(s);
+    if (it != ctx->batch.end()) {
+        *out = it->second;
+        return PFSM_OK;
+    }
+    BatchState *b = new BatchState();
+    bool ok = cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaEventCreateWithFlags(&b->staged, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess;
+    for (int c = 0; ok && c < kBatchClasses; ++c)
+        ok = cudaStreamCreateWithFlags(&b->aux[c], cudaStreamNonBlocking) == cudaSuccess &&
+             cudaEventCreateWithFlags(&b->join[c], cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) {
+        cudaGetLastError();
+        state_free(b);
+        return PFSM_E_CUDA;
+    }
+    *out = ctx->batch[s] = b;
+    return PFSM_OK;
+}
+
+// Whether stream `s` has the candidate lists of sieved texts (allocated when a
+// batch first needs them). Where there is no room for them the class kernels
+// take such texts.
+static bool have_lists(pfsm_ctx *ctx, cudaStream_t s) {
+    BatchState *b = nullptr;
+    if (state_of(ctx, s, &b)) return false;
+    if (!b->cand && cudaMalloc(&b->cand, 2ull * kFlatCand * sizeof(uint4)) != cudaSuccess) {
+        cudaGetLastError();
+        b->cand = nullptr;
+    }
+    return b->cand != nullptr;
+}
+
 static int state_reserve(pfsm_ctx *ctx, cudaStream_t s, size_t njobs, size_t nmachs,
                          BatchState **out) {
-    // (a state is entered when it is whole: after a failure the next call
-    // starts anew)
-    const auto it = ctx->batch.find(s);
-    BatchState *b = it == ctx->batch.end() ? nullptr : it->second;
-    if (!b) {
-        b = new BatchState();
-        bool ok = cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking) == cudaSuccess &&
-                  cudaEventCreateWithFlags(&b->staged, cudaEventDisableTiming) == cudaSuccess &&
-                  cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess;
-        for (int c = 0; ok && c < kBatchClasses; ++c)
-            ok = cudaStreamCreateWithFlags(&b->aux[c], cudaStreamNonBlocking) == cudaSuccess &&
-                 cudaEventCreateWithFlags(&b->join[c], cudaEventDisableTiming) == cudaSuccess;
-        const int st = !ok ? PFSM_E_CUDA
-                       : cudaMalloc(&b->cand, 2ull * kFlatCand * sizeof(uint4)) != cudaSuccess ? PFSM_E_NOMEM
-                                                                                               : PFSM_OK;
-        if (st) {
-            cudaGetLastError();
-            state_free(b);
-            return st;
-        }
-        ctx->batch[s] = b;
-    }
+    BatchState *b = nullptr;
+    const int st = state_of(ctx, s, &b);
+    if (st) return st;
     if (njobs <= b->cap_jobs && nmachs <= b->cap_machs) {
         *out = b;
         return PFSM_OK;
@@ -428,6 +446,8 @@ static int plan_batch(pfsm_ctx *ctx, const pfsm_job *jobs, int32_t k, BatchPlan 
         pl.used.push_back(&m);
         flat_of[i] = flat_class(ctx, m);
     }
+    for (int &c : flat_of)
+        if ((c == FLAT_DNA || c == FLAT_BYTES) && !have_lists(ctx, s)) c = -1;
     for (int32_t i = 0; i < k; ++i) {
         if (jobs[i].n >= (1ull << 32) - 256) flat_of[job_slot[i]] = -1;   // positions would wrap
     }

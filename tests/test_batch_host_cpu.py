@@ -113,7 +113,7 @@ def test_a_call_after_one_that_found_no_memory(lib, nth, cls):
             lib.hb_fail(nth)
             st, got = h.scan([0] * jobs, [5000] * jobs)
             lib.hb_fail(0)
-            assert st in (0, E_NOMEM) and got["flat"] == (st == 0) and got["null_lists"] == 0
+            assert st in (0, E_NOMEM) and got["flat"] + got["graph"] == (st == 0) and got["null_lists"] == 0
             st, got = h.scan([0] * jobs, [5000] * jobs)
             assert st == 0 and got["flat"] == 1 and got["null_lists"] == 0 and got["missed"] == 0
 
@@ -144,3 +144,18 @@ def test_warps_of_the_front_kernel_do_not_share_memory(lib):
         assert all(apart(regions[w], regions[v]) for w in range(32) for v in range(w))
         assert c == WALK or min(r[0] for r in regions) >= 128 << 10
         assert max(r[1] for r in regions) <= (128 << 10) + 32 * 1024
+
+
+@pytest.mark.parametrize("cls", [DNA, BYTES, WALK])
+def test_no_room_for_the_candidate_lists(lib, cls):
+    """The class kernels take sieved texts where the lists find no room; the
+    next call tries again."""
+    with Host(lib, [cls, WALK]) as h:
+        if cls != WALK:
+            lib.hb_fail(1)
+            st, got = h.scan([0, 1], [5000, 5000])
+            lib.hb_fail(0)
+            assert st == 0 and got["graph"] == 1 and got["flat"] == 1 and got["used"] == 2
+            assert got["null_lists"] == 0 and got["missed"] == 0
+        st, got = h.scan([0, 1], [5000, 5000])
+        assert st == 0 and got["graph"] == 0 and got["flat"] == 1 and got["missed"] == 0
