@@ -1040,6 +1040,34 @@ static int walk_enqueue(pfsm_ctx *ctx, const Machine &m, const uint8_t *text, ui
     });
 }
 
+// Warp-wide bitsets in global memory for a scan by the tile kernel.
+static int tile_coop(pfsm_ctx *ctx, const Machine &m, Slot *slot, Plan &pl) {
+    if (m.kind != 1 || pl.a.coop_smem) return PFSM_OK;
+    // one pair of bitsets per warp of the tile kernel and, when the scan
+    // is chained, of the carry kernel (nsm CTAs of up to 256 threads)
+    size_t warps = static_cast<size_t>(pl.grid) * (pl.threads / 32);
+    if (pl.a.carry_cap) warps = std::max(warps, static_cast<size_t>(ctx->nsm) * (std::min(pl.threads, 256) / 32));
+    const size_t need = warps * 2 * m.dm.Wq;
+    if (ensure_words(&slot->coop, &slot->coop_words, need)) return PFSM_E_NOMEM;
+    pl.a.coop_g = slot->coop;
+    return PFSM_OK;
+}
+
+// A captured scan takes the tile kernel and cannot allocate: the scans on the
+// stream before it, whatever kernels they take, leave the scratch that one of
+// their length needs. (Where there is no room for it, only a captured scan
+// fails.)
+static void reserve_coop(pfsm_ctx *ctx, const Machine &m, const uint8_t *text, uint64_t n, Slot *slot) {
+    auto &c = slot->coop_for[m.id & 7];
+    if (c.id == m.id && n <= c.n) return;
+    Plan pl;
+    if (plan_scan(ctx, m, text, n, pl)) return;
+    pl.a.carry_cap = 0;   // (an NFA's default: not chained)
+    if (tile_coop(ctx, m, slot, pl)) return;
+    c.id = m.id;
+    c.n = n;
+}
+
 // The launches of a sieved scan.
 static int sieve_enqueue(pfsm_ctx *ctx, const Machine &m, const uint8_t *text, uint64_t n, uint32_t *out,
                          uint64_t cap, unsigned long long *status, Slot *slot, cudaStream_t s) {
@@ -1077,6 +1105,7 @@ static int sieve_enqueue(pfsm_ctx *ctx, const Machine &m, const uint8_t *text, u
         });
     };
     if (m.kind == 0) return launch([&] { return launch_finish_dfa(a, ctx->nsm, s); });
+    reserve_coop(ctx, m, text, n, slot);
     // the finishing kernel, in half an SM's shared memory: band rows and
     // warp-wide bitsets as far as they fit
     ScanArgs f;
@@ -1159,16 +1188,8 @@ int scan_enqueue(pfsm_ctx *ctx, pfsm_aut aut, const uint8_t *text, uint64_t n, u
     pl.a.cpool_cap = m.kind == 1 ? 2 * kCarryCap : 0u;
     if (pl.a.carry_cap && ctx->test_carry_cap) pl.a.carry_cap = std::min(pl.a.carry_cap, ctx->test_carry_cap);
     if (pl.a.cpool_cap && ctx->test_cpool_cap) pl.a.cpool_cap = std::min(pl.a.cpool_cap, ctx->test_cpool_cap);
-    if (m.kind == 1 && !pl.a.coop_smem) {
-        // one pair of bitsets per warp of the tile kernel and, when the scan
-        // is chained, of the carry kernel (nsm CTAs of up to 256 threads)
-        size_t warps = static_cast<size_t>(pl.grid) * (pl.threads / 32);
-        if (pl.a.carry_cap)
-            warps = std::max(warps, static_cast<size_t>(ctx->nsm) * (std::min(pl.threads, 256) / 32));
-        const size_t need = warps * 2 * m.dm.Wq;
-        if (ensure_words(&slot->coop, &slot->coop_words, need)) return PFSM_E_NOMEM;
-        pl.a.coop_g = slot->coop;
-    }
+    st = tile_coop(ctx, m, slot, pl);
+    if (st) return st;
     if (pl.a.carry_cap && cudaMemsetAsync(slot->carry_n, 0, 8 * sizeof(uint32_t), s) != cudaSuccess)
         return PFSM_E_CUDA;
     time_begin();
@@ -1289,6 +1310,7 @@ static int finish_load(pfsm_ctx *ctx, Machine &&m, pfsm_aut *out_id) {
     const int id = ctx->next_id++;
     auto &slot = ctx->machines[id];
     slot = std::move(m);
+    slot.id = id;
     ctx->n_loads++;
     int st = make_resident(ctx, id, slot, nullptr);
     if (!st && cudaEventSynchronize(slot.ready) != cudaSuccess) st = PFSM_E_CUDA;

@@ -22,6 +22,7 @@ constexpr uint32_t kBatchSmemStatic = 2048;  // the batch class kernels' static 
 constexpr int kEventRing = 256;              // timed launches kept in flight per stream
 
 struct Machine {
+    int id = 0;    // the caller's pfsm_aut
     int kind = 0;  // 0 DFA, 1 NFA
     int Q = 0, S = 0, q0 = 0, dead = -1;
     std::vector<uint8_t> fin;
@@ -98,6 +99,9 @@ struct Slot {   // per-stream scratch
     unsigned long long *host_status = nullptr;   // pinned [2]
     uint32_t *coop = nullptr;               // warp-wide NFA bitsets
     size_t coop_words = 0;
+    // automata (by the low bits of their ids) and the text length that `coop`
+    // has been sized for (reserve_coop)
+    struct { int id; uint64_t n; } coop_for[8] = {};
     // ring of (start, end) events around timed tile-kernel launches
     cudaEvent_t ev[2 * kEventRing] = {};
     int ev_head = 0, ev_pending = 0;
