@@ -744,7 +744,7 @@ Slot *get_slot(pfsm_ctx *ctx, cudaStream_t s) {
     Slot sl;
     void *p = nullptr;
     constexpr size_t head = 128;   // status, carry counters, the sieve's counters
-    const size_t bytes = head + static_cast<size_t>(kCarryCap) * 16 + static_cast<size_t>(kCandCap) * sizeof(uint2);
+    const size_t bytes = head + static_cast<size_t>(kCarryCap) * 16;
     if (cudaMalloc(&p, bytes) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
@@ -754,7 +754,6 @@ Slot *get_slot(pfsm_ctx *ctx, cudaStream_t s) {
     sl.sv_status = reinterpret_cast<unsigned long long *>(static_cast<uint8_t *>(p) + 64);
     sl.sv_count = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(p) + 80);
     sl.carry = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(p) + head);
-    sl.cand = reinterpret_cast<uint2 *>(sl.carry + static_cast<size_t>(kCarryCap) * 4);
     if (cudaMallocHost(&sl.host_status, 2 * sizeof(unsigned long long)) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(p);
@@ -1000,6 +999,17 @@ static Route route_of(const pfsm_ctx *ctx, const Machine &m, uint64_t n, cudaStr
     return sieve ? ROUTE_SIEVE : ROUTE_WALK;
 }
 
+// Whether the stream has the sieve's candidate list (also the scratch of
+// long-lived scans), allocated by the first scan that needs it. Where there is
+// no room for it the tile kernel takes the scan.
+static bool have_cand(Slot *slot) {
+    if (!slot->cand && cudaMalloc(&slot->cand, static_cast<size_t>(kCandCap) * sizeof(uint2)) != cudaSuccess) {
+        cudaGetLastError();
+        slot->cand = nullptr;
+    }
+    return slot->cand != nullptr;
+}
+
 // Runs `launch` (a scan whose last kernel leaves the stream's counters zero)
 // with the counters zero: they are cleared before the stream's first such
 // scan and after one that was not wholly launched.
@@ -1155,7 +1165,9 @@ int scan_enqueue(pfsm_ctx *ctx, pfsm_aut aut, const uint8_t *text, uint64_t n, u
         slot->ev_head = (slot->ev_head + 1) % kEventRing;
         slot->ev_pending++;
     };
-    const Route route = route_of(ctx, m, n, s);
+    Route route = route_of(ctx, m, n, s);
+    const bool scratch = route == ROUTE_SIEVE || (route == ROUTE_WALK && m.lives && n >= kLongText);
+    if (scratch && !have_cand(slot)) route = ROUTE_TILES;
     if (route != ROUTE_TILES) {
         time_begin();
         // a scan that is waited for gets its status written to host memory
@@ -1279,6 +1291,7 @@ int pfsm_ctx_destroy(pfsm_ctx *ctx) {
     for (auto &kv : ctx->slots) {
         cudaFree(kv.second.coop);
         cudaFree(kv.second.status);
+        cudaFree(kv.second.cand);
         cudaFreeHost(kv.second.host_status);
         for (int i = 0; i < 2 * kEventRing; ++i) cudaEventDestroy(kv.second.ev[i]);
     }

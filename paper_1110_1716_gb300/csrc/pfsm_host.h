@@ -90,7 +90,7 @@ struct Slot {   // per-stream scratch
     unsigned long long *status = nullptr;   // device [2]
     uint32_t *carry_n = nullptr;
     uint32_t *carry = nullptr;              // kCarryCap entries of 4 words
-    uint2 *cand = nullptr;                  // kCandCap candidates of the sieve
+    uint2 *cand = nullptr;                  // kCandCap candidates of the sieve, when a scan has needed them
     // the sieve's counters, zero between scans: {matches, error bits} and
     // {candidates, CTAs done}
     unsigned long long *sv_status = nullptr;

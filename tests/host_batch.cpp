@@ -1,58 +1,13 @@
 // The host side of batches (csrc/batch.cu) without a GPU: the CUDA runtime and
-// the rest of the library are replaced by the stand-ins below, device memory
-// is host memory, and the launch of a flat batch is replayed step by step as
-// its warps take them. Compiled by g++ (test_batch_host_cpu.py).
-#include <stdlib.h>
-
+// the rest of the library are replaced by stand-ins (host_cuda.h and below),
+// and the launch of a flat batch is replayed step by step as its warps take
+// them. Compiled by g++ (test_batch_host_cpu.py).
 #include <mutex>
 
 #include "batch.cu"
+#include "host_cuda.h"
 
 using namespace pfsm;
-
-// ------------------------------------------------------------ stand-ins
-static int fail_in = 0;   // the fail_in-th device allocation from now fails (0: none)
-static int dummy;
-
-extern "C" {
-cudaError_t cudaMalloc(void **p, size_t n) {
-    *p = nullptr;
-    if (fail_in && --fail_in == 0) return cudaErrorMemoryAllocation;
-    *p = calloc(n, 1);
-    return cudaSuccess;
-}
-cudaError_t cudaFree(void *p) { return free(p), cudaSuccess; }
-cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { return *p = calloc(n, 1), cudaSuccess; }
-cudaError_t cudaFreeHost(void *p) { return free(p), cudaSuccess; }
-cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t) {
-    return memcpy(d, s, n), cudaSuccess;
-}
-cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t) { return memset(d, v, n), cudaSuccess; }
-cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) {
-    return *e = reinterpret_cast<cudaEvent_t>(&dummy), cudaSuccess;
-}
-cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaGetDevice(int *d) { return *d = 0, cudaSuccess; }
-cudaError_t cudaSetDevice(int) { return cudaSuccess; }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
-cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
-cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
-cudaError_t cudaGraphInstantiate(cudaGraphExec_t *e, cudaGraph_t, unsigned long long) {
-    return *e = reinterpret_cast<cudaGraphExec_t>(&dummy), cudaSuccess;
-}
-cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaSuccess; }
-cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) {
-    return *s = reinterpret_cast<cudaStream_t>(&dummy), cudaSuccess;
-}
-cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *g) {
-    return *g = reinterpret_cast<cudaGraph_t>(&dummy), cudaSuccess;
-}
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
-}
 
 // What the launches of the last call did.
 static struct Seen {
@@ -65,7 +20,7 @@ static struct Seen {
 } seen;
 static uint32_t chunk = 5;    // steps a warp takes
 
-extern "C" cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return ++seen.graph, cudaSuccess; }
+void host_graph_launched() { seen.graph++; }
 
 namespace pfsm {
 uint32_t layout_smem(ScanArgs &, int, int, const SmemNeed &) { return 4096; }
@@ -150,7 +105,7 @@ void hb_own(int32_t c, int32_t big, uint32_t warp, uint32_t *range) {
     range[0] = flat_own(c, big != 0, warp);
     range[1] = range[0] + flat_own_bytes(c);
 }
-void hb_fail(int n) { fail_in = n; }
+void hb_fail(int n) { host_fail_in = n; }
 void hb_chunk(uint32_t n) { chunk = n; }
 // One batch of texts of n[i] symbols at address text[i] for machine aut[i].
 int hb_scan(pfsm_ctx *c, const int32_t *aut, const uint64_t *text, const uint64_t *n, int32_t k, int64_t *out) {
