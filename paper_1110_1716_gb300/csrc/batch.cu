@@ -314,6 +314,7 @@ struct BatchPlan {
 // the class kernels, which then run).
 static int flat_class(const pfsm_ctx *ctx, const Machine &m) {
     if (ctx->batch_threads || ctx->batch_ctas || ctx->batch_tile != kBatchTile || !default_params(m)) return -1;
+    if (!m.full) return -1;   // the core of its image only
     if (m.sv_kind == SIEVE_DNA && m.k > 0 && (m.kind == 0 || m.sv_lean)) return FLAT_DNA;
     if (m.sv_kind == SIEVE_BYTES && m.k > 0) return FLAT_BYTES;
     return m.walks ? FLAT_WALK : -1;
@@ -434,10 +435,22 @@ static int plan_batch(pfsm_ctx *ctx, const pfsm_job *jobs, int32_t k, BatchPlan 
         job_slot[i] = last_slot;
     }
     if (ids.size() >= (1u << 24)) return PFSM_E_INVAL;
-    for (int id : ids) {
-        int st = make_resident(ctx, id, ctx->machines[id], s);
-        if (st) return st;
+    // whole images, or, where they do not fit the budget together, their cores
+    // (first of those that are resident, which makes room)
+    int fit = PFSM_OK;
+    auto all = [&](bool core, bool resident) {
+        for (int id : ids) {
+            Machine &m = ctx->machines[id];
+            if (!fit && (!resident || m.dev)) fit = make_resident(ctx, id, m, s, core);
+        }
+    };
+    all(false, false);
+    if (fit == PFSM_E_NOMEM) {
+        fit = PFSM_OK;
+        all(true, true);
+        all(true, false);
     }
+    if (fit) return fit;
     // machines whose texts run flat, and the texts that keep to the classes
     std::vector<int> flat_of(ids.size());
     int32_t rest = k;

@@ -436,12 +436,11 @@ void build_survival(Machine &m) {
 // ---- residency --------------------------------------------------------------
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-size_t device_bytes(const Machine &m) {
+// Bytes of the tables that the tile and class kernels read: all that a machine
+// holds where the budget has no room for the others.
+static size_t core_bytes(const Machine &m) {
     size_t b = align256(m.memo.size() * 2 + 4) + align256(m.surv.size() * 4 + 4) +
-               align256(m.surv2.size() * 4 + 4) + align256(m.tail.size() * 2 + 4) +
-               align256(m.sv_near.size() * 4) + align256(m.sv_deep.size() * 4) + align256(m.sv_l3.size() * 4) +
-               align256(m.chain.size() * 4) + align256(m.sv_strand.size() * 2 + 4) +
-               align256(m.walk_tab.size() * 4);
+               align256(m.surv2.size() * 4 + 4) + align256(m.tail.size() * 2 + 4);
     if (m.kind == 0) {
         b += align256(m.dtab.size() * 2 + 4) + align256(m.pool.size() * 4);
     } else {
@@ -452,6 +451,13 @@ size_t device_bytes(const Machine &m) {
              align256(m.memox.size() * 2 + 4);
     }
     return b;
+}
+
+// With the tables of the sieve and of direct scans.
+size_t device_bytes(const Machine &m) {
+    return core_bytes(m) + align256(m.sv_near.size() * 4) + align256(m.sv_deep.size() * 4) +
+           align256(m.sv_l3.size() * 4) + align256(m.chain.size() * 4) + align256(m.sv_strand.size() * 2) +
+           align256(m.walk_tab.size() * 4);
 }
 
 // Frees a machine's device image once nothing can still read it: the host
@@ -543,8 +549,9 @@ int evict_lru(pfsm_ctx *ctx, uint64_t need, int keep_id, cudaStream_t s) {
 }
 
 // The device image of `m`, built once in pinned host memory: 256-byte
-// aligned sections (prefix table, short-gram table, survival bitmaps, then
-// the DFA table or the NFA CSR, records and band image).
+// aligned sections (prefix table, short-gram table, survival bitmaps, the DFA
+// table or the NFA CSR, records and band image, then the tables of the sieve
+// and of direct scans).
 static int build_host_image(Machine &m) {
     if (m.host_img) return PFSM_OK;
     const size_t bytes = device_bytes(m);
@@ -566,12 +573,6 @@ static int build_host_image(Machine &m) {
     m.o_tail = put(m.tail.data(), m.tail.size() * 2, 4);
     m.o_surv = put(m.surv.data(), m.surv.size() * 4, 4);
     m.o_surv2 = put(m.surv2.data(), m.surv2.size() * 4, 4);
-    m.o_near = put(m.sv_near.data(), m.sv_near.size() * 4, 0);
-    m.o_deep = put(m.sv_deep.data(), m.sv_deep.size() * 4, 0);
-    m.o_l3 = put(m.sv_l3.data(), m.sv_l3.size() * 4, 0);
-    m.o_chain = put(m.chain.data(), m.chain.size() * 4, 0);
-    m.o_strand = put(m.sv_strand.data(), m.sv_strand.size() * 2, 4);
-    m.o_walk = put(m.walk_tab.data(), m.walk_tab.size() * 4, 0);
     if (m.kind == 0) {
         m.o_tab = put(m.dtab.data(), m.dtab.size() * 2, 4);
         m.o_pool = put(m.pool.data(), m.pool.size() * 4, 0);
@@ -587,6 +588,13 @@ static int build_host_image(Machine &m) {
         m.o_pool2 = put(m.pool2.data(), m.pool2.size() * 4, 16);
         m.o_memox = put(m.memox.data(), m.memox.size() * 2, 4);
     }
+    m.core_bytes = o;
+    m.o_near = put(m.sv_near.data(), m.sv_near.size() * 4, 0);
+    m.o_deep = put(m.sv_deep.data(), m.sv_deep.size() * 4, 0);
+    m.o_l3 = put(m.sv_l3.data(), m.sv_l3.size() * 4, 0);
+    m.o_chain = put(m.chain.data(), m.chain.size() * 4, 0);
+    m.o_strand = put(m.sv_strand.data(), m.sv_strand.size() * 2, 0);
+    m.o_walk = put(m.walk_tab.data(), m.walk_tab.size() * 4, 0);
     if (o > bytes) {   // layout and size disagree: a bug, fail loudly
         cudaFreeHost(h);
         return PFSM_E_INVAL;
@@ -596,8 +604,9 @@ static int build_host_image(Machine &m) {
     return PFSM_OK;
 }
 
-// The kernels' view of a machine whose image starts at `base`.
-static DevMachine dev_view(const Machine &m, uint8_t *base) {
+// The kernels' view of a machine whose image, or (not `full`) the core of it,
+// starts at `base`.
+static DevMachine dev_view(const Machine &m, uint8_t *base, bool full) {
     DevMachine dm{};
     dm.kind = m.kind;
     dm.Q = m.Q;
@@ -614,10 +623,14 @@ static DevMachine dev_view(const Machine &m, uint8_t *base) {
     dm.surv_words = static_cast<uint32_t>(m.surv.size());
     dm.surv2 = m.surv2.empty() ? nullptr : reinterpret_cast<const uint32_t *>(base + m.o_surv2);
     dm.surv2_m = m.sm_m2;
-    dm.sv_near = m.sv_kind ? reinterpret_cast<const uint32_t *>(base + m.o_near) : nullptr;
-    dm.chain = m.chain.empty() ? nullptr : reinterpret_cast<const uint4 *>(base + m.o_chain);
-    dm.sv_strand = m.sv_strand.empty() ? nullptr : reinterpret_cast<const uint16_t *>(base + m.o_strand);
-    dm.walk = m.walk_tab.empty() ? nullptr : base + m.o_walk;
+    if (full) {
+        dm.sv_near = m.sv_kind ? reinterpret_cast<const uint32_t *>(base + m.o_near) : nullptr;
+        dm.sv_deep = m.sv_deep.empty() ? nullptr : reinterpret_cast<const uint32_t *>(base + m.o_deep);
+        dm.sv_l3 = m.sv_l3.empty() ? nullptr : reinterpret_cast<const uint32_t *>(base + m.o_l3);
+        dm.chain = m.chain.empty() ? nullptr : reinterpret_cast<const uint4 *>(base + m.o_chain);
+        dm.sv_strand = m.sv_strand.empty() ? nullptr : reinterpret_cast<const uint16_t *>(base + m.o_strand);
+        dm.walk = m.walk_tab.empty() ? nullptr : base + m.o_walk;
+    }
     dm.flat = -1;
     dm.walk_words = m.walk_bitset() ? static_cast<int32_t>(walk_nfa_words(m.Q)) : 0;
     for (int w = 0; w < 2; ++w) {
@@ -625,8 +638,6 @@ static DevMachine dev_view(const Machine &m, uint8_t *base) {
         dm.walk_finals[w] = m.walk_finals[w];
     }
     dm.min_match = m.min_match;
-    dm.sv_l3 = m.sv_l3.empty() ? nullptr : reinterpret_cast<const uint32_t *>(base + m.o_l3);
-    dm.sv_deep = m.sv_deep.empty() ? nullptr : reinterpret_cast<const uint32_t *>(base + m.o_deep);
     if (m.kind == 0) {
         dm.dtab = reinterpret_cast<const uint16_t *>(base + m.o_tab);
         dm.pool = reinterpret_cast<const uint32_t *>(base + m.o_pool);
@@ -649,13 +660,24 @@ static DevMachine dev_view(const Machine &m, uint8_t *base) {
 // Makes `m` resident for work enqueued on `s`: a resident machine only makes
 // `s` wait for its upload (when that has not finished yet); otherwise the
 // least recently used machines are evicted in stream order, an image is
-// taken from the pool and the pinned host image is copied in on `s`.
-int make_resident(pfsm_ctx *ctx, int id, Machine &m, cudaStream_t s) {
+// taken from the pool and the pinned host image is copied in on `s`. Where the
+// whole image finds no room its core is taken alone (`core`: from the start,
+// for batches whose machines do not fit the budget together otherwise), which
+// the tile and class kernels do with; a machine so held gets the rest by a
+// later call that finds the room for it without an eviction.
+int make_resident(pfsm_ctx *ctx, int id, Machine &m, cudaStream_t s, bool core) {
     NvtxRange nr("pfsm make_resident");
     m.last_use = ++ctx->clock;
     if (!m.ready && cudaEventCreateWithFlags(&m.ready, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         return PFSM_E_CUDA;
+    }
+    if (m.dev && m.full && core && m.core_bytes < m.img_bytes) {
+        release_async(ctx, m, s);
+    } else if (m.dev && !m.full && !core && ctx->resident_bytes - m.dev_bytes + m.img_bytes <= ctx->budget) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) release_async(ctx, m, s);
+        else cudaGetLastError();
     }
     if (m.dev) {
         if (!m.uploaded) {
@@ -670,13 +692,19 @@ int make_resident(pfsm_ctx *ctx, int id, Machine &m, cudaStream_t s) {
     }
     int st = build_host_image(m);
     if (st) return st;
-    const size_t bytes = m.img_bytes;
-    st = evict_lru(ctx, bytes, id, s);
-    if (st) return st;
     void *p = nullptr;
-    if (cudaMallocFromPoolAsync(&p, bytes, ctx->pool, s) != cudaSuccess) {
-        cudaGetLastError();
-        return PFSM_E_NOMEM;
+    bool full = !core || m.core_bytes == m.img_bytes;
+    size_t bytes = 0;
+    while (true) {
+        bytes = full ? m.img_bytes : m.core_bytes;
+        st = evict_lru(ctx, bytes, id, s);
+        if (!st && cudaMallocFromPoolAsync(&p, bytes, ctx->pool, s) != cudaSuccess) {
+            cudaGetLastError();
+            st = PFSM_E_NOMEM;
+        }
+        if (!st) break;
+        if (!full || m.core_bytes == m.img_bytes) return st;
+        full = false;
     }
     if (cudaMemcpyAsync(p, m.host_img, bytes, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaEventRecord(m.ready, s) != cudaSuccess) {
@@ -686,8 +714,9 @@ int make_resident(pfsm_ctx *ctx, int id, Machine &m, cudaStream_t s) {
     }
     m.dev = p;
     m.uploaded = false;
+    m.full = full;
     m.dev_bytes = bytes;
-    m.dm = dev_view(m, static_cast<uint8_t *>(p));
+    m.dm = dev_view(m, static_cast<uint8_t *>(p), full);
     ctx->resident_bytes += bytes;
     if (m.was_resident) ctx->n_reload++;
     m.was_resident = true;
@@ -974,8 +1003,8 @@ void collect_timing(pfsm_ctx *ctx, Slot *slot, int keep) {
 }
 
 // A machine's scans take the sieve (sieve.cu) or the direct scan (walk.cu)
-// when it has the tables for one of them and all its parameters are the
-// defaults: any other setting shapes the tile kernel, which then runs.
+// when it has the tables for one of them on the device and all its parameters
+// are the defaults: any other setting shapes the tile kernel, which then runs.
 // (Positions within 256 of 2^32 would wrap.) A scan that is being captured
 // takes the tile kernel too: the counters of the other two belong to the
 // stream, and a graph may be replayed on others.
@@ -989,7 +1018,7 @@ bool default_params(const Machine &m) {
 enum Route { ROUTE_TILES, ROUTE_SIEVE, ROUTE_WALK };
 static Route route_of(const pfsm_ctx *ctx, const Machine &m, uint64_t n, cudaStream_t s) {
     const bool sieve = m.sv_kind && m.k > 0;
-    if ((!sieve && !m.walks) || ctx->hold_tiles || n == 0 || n >= (1ull << 32) - 256) return ROUTE_TILES;
+    if ((!sieve && !m.walks) || !m.full || ctx->hold_tiles || n == 0 || n >= (1ull << 32) - 256) return ROUTE_TILES;
     if (!default_params(m)) return ROUTE_TILES;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {

@@ -72,6 +72,8 @@ struct Machine {
     size_t dev_bytes = 0;
     uint8_t *host_img = nullptr;      // pinned copy of the device image
     size_t img_bytes = 0;
+    size_t core_bytes = 0;            // of it: what the tile and class kernels read
+    bool full = false;                // all of it is on the device, not the core alone
     size_t o_memo = 0, o_tail = 0, o_surv = 0, o_surv2 = 0, o_tab = 0, o_off = 0,
            o_tgt = 0, o_pool = 0, o_band = 0, o_eoff = 0, o_etgt = 0, o_l2tab = 0,
            o_pool2 = 0, o_memox = 0, o_near = 0, o_deep = 0, o_l3 = 0, o_chain = 0, o_strand = 0, o_walk = 0;   // section offsets
@@ -198,7 +200,7 @@ size_t align256(size_t x);
 void release(pfsm_ctx *ctx, Machine &m);
 void drop_host_image(Machine &m);
 void sweep_retired(pfsm_ctx *ctx);
-int make_resident(pfsm_ctx *ctx, int id, Machine &m, cudaStream_t s);
+int make_resident(pfsm_ctx *ctx, int id, Machine &m, cudaStream_t s, bool core = false);
 int mark_use(pfsm_ctx *ctx, cudaStream_t s, Machine *const *ms, size_t k);
 Slot *get_slot(pfsm_ctx *ctx, cudaStream_t s);
 int ensure_words(uint32_t **buf, size_t *have, size_t need);

@@ -31,7 +31,7 @@ cudaError_t launch_carry_batch(const BatchArgs *, int, cudaStream_t) { return cu
 bool default_params(const Machine &) { return true; }
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 int ensure_words(uint32_t **, size_t *, size_t) { return PFSM_OK; }
-int make_resident(pfsm_ctx *, int, Machine &, cudaStream_t) { return PFSM_OK; }
+int make_resident(pfsm_ctx *, int, Machine &m, cudaStream_t, bool) { return m.full = true, PFSM_OK; }
 int mark_use(pfsm_ctx *, cudaStream_t, Machine *const *, size_t k) { return seen.used = static_cast<int64_t>(k), PFSM_OK; }
 Slot *get_slot(pfsm_ctx *, cudaStream_t) { return nullptr; }
 void collect_timing(pfsm_ctx *, Slot *, int) {}

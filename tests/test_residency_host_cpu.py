@@ -86,3 +86,85 @@ def test_no_room_for_the_scratch_of_the_newer_kernels(lib, name):
         finally:
             lib.hl_largest(0)
         assert h.scan(a) == (OK, [route])
+
+
+def stats(h):
+    v = np.zeros(6, dtype=np.uint64)   # resident_bytes, budget_bytes, loads, evictions, reloads, (counts)
+    h.lib.pfsm_get_stats(h.ctx, P(v.ctypes.data))
+    return int(v[0])
+
+
+def aut_bytes(h, a):
+    n = ctypes.c_uint64()
+    assert h.lib.pfsm_aut_bytes(h.ctx, a, ctypes.byref(n), None) == OK
+    return n.value
+
+
+def batch(h, auts, n=3000):
+    text = np.zeros(n, dtype=np.uint8)
+    jobs = np.zeros(len(auts), dtype=[("aut", "<i4"), ("reserved", "<u4"), ("text", "<u8"), ("n", "<u8")])
+    jobs["aut"], jobs["text"], jobs["n"] = auts, text.ctypes.data, n
+    total = ctypes.c_uint64()
+    st = h.lib.pfsm_scan_batch(h.ctx, P(jobs.ctypes.data), len(auts), P(), ctypes.c_uint64(0), P(), ctypes.byref(total), P())
+    return st, h.launched()
+
+
+# bytes of the tables that the tile kernel reads (what an automaton held before
+# there were tables of the sieve and of direct scans)
+def core(lib, make):
+    with Host(lib) as h:
+        st, a = h.load(make())
+        whole = aut_bytes(h, a)
+        lo, hi = 0, whole
+    while hi - lo > 256:      # the smallest budget that loads it
+        mid = (lo + hi) // 2 // 256 * 256
+        with Host(lib, mid) as h:
+            st, a = h.load(make())
+            lo, hi = (lo, mid) if st == OK else (mid, hi)
+    return hi, whole
+
+
+@pytest.mark.parametrize("name", ["trie", "motifs", "dense_dfa"])
+def test_budgets_that_hold_the_core_alone(lib, name):
+    make, route = MACHINES[name]
+    small, whole = core(lib, make)
+    assert small < whole
+    if name == "motifs":      # 8 MB of deep bitmap and the third level in the rest
+        assert small < 0.6 * whole
+    with Host(lib, whole - 256) as h:
+        st, a = h.load(make())
+        assert st == OK and h.scan(a) == (OK, ["tiles"]) and batch(h, [a, a]) == (OK, ["classes"])
+        assert stats(h) == small <= whole - 256
+    with Host(lib, whole) as h:
+        st, a = h.load(make())
+        assert st == OK and h.scan(a) == (OK, [route]) and batch(h, [a]) == (OK, ["flat"])
+    # two automata: both cores, and one whole image beside a core
+    for budget, want in ((2 * small, ["classes"]), (small + whole, ["classes", "flat"]), (2 * whole, ["flat"])):
+        with Host(lib, budget) as h:
+            a, b = h.load(make())[1], h.load(make())[1]
+            for _ in range(3):
+                assert batch(h, [a, b]) == (OK, want), budget
+                assert stats(h) <= budget
+            # each alone: the other makes room for the whole image, or leaves the core in place
+            for x in (a, b, a):
+                st, got = h.scan(x)
+                assert st == OK and got in ([route], ["tiles"])
+                assert stats(h) <= budget
+    # one whole image is never the last: with room again, a core is completed
+    with Host(lib, 2 * small) as h:
+        a, b = h.load(make())[1], h.load(make())[1]
+        assert batch(h, [a, b]) == (OK, ["classes"])
+        h.lib.pfsm_unload(h.ctx, b)
+        if 2 * small >= whole:
+            assert h.scan(a) == (OK, [route]) and stats(h) == whole
+    with Host(lib, small - 256) as h:
+        assert h.load(make())[0] == E_NOMEM
+
+
+def test_a_batch_that_does_not_fit_is_still_refused(lib):
+    make, _ = MACHINES["motifs"]
+    small, whole = core(lib, make)
+    with Host(lib, 2 * small - 256) as h:
+        a, b = h.load(make())[1], h.load(make())[1]
+        assert batch(h, [a, b])[0] == E_NOMEM
+        assert h.scan(a)[0] == OK and h.scan(b)[0] == OK and batch(h, [a])[0] == OK
