@@ -12,8 +12,10 @@
 
 #include <algorithm>
 #include <functional>
+#include <future>
 #include <map>
 #include <mutex>
+#include <system_error>
 #include <vector>
 
 #include "pfsm_host.h"
@@ -344,7 +346,7 @@ bool build_memo(Machine &m) {
 // Built depth-first; a subtree is settled as soon as the set empties (all
 // clear) or a final state is met (all set). Returns false (and no bitmap)
 // when fewer than half of the m-grams are clear.
-static bool survival_bits(const Machine &m, int mm, std::vector<uint32_t> &bits) {
+static bool survival_bits(const Machine &m, int mm, std::vector<uint32_t> &bits, uint64_t &grams) {
     const uint32_t nbits = 1u << (mm * m.sbits);
     bits.assign((nbits + 31) / 32, 0);
     uint64_t ones = 0;
@@ -405,6 +407,7 @@ static bool survival_bits(const Machine &m, int mm, std::vector<uint32_t> &bits)
         lv[0] = nfa_initial(m);
         dfs(0, 0);
     }
+    grams = ones;
     if (ones * 2 > nbits) {
         bits.clear();
         return false;
@@ -422,14 +425,15 @@ void build_survival(Machine &m) {
     m.sm_m = 0;
     m.sm_m2 = 0;
     const int m1 = std::min(9, 18 / m.sbits);
-    auto bits = [&](int mm, std::vector<uint32_t> &to) {
-        return m.kind == 1 && m.sbits == 2 ? survival_bits_dna(m, mm, to) : survival_bits(m, mm, to);
+    auto bits = [&](int mm, std::vector<uint32_t> &to, uint64_t &grams) {
+        return m.kind == 1 && m.sbits == 2 ? survival_bits_dna(m, mm, to, grams) : survival_bits(m, mm, to, grams);
     };
-    if (m1 >= 1 && bits(m1, m.surv)) m.sm_m = m1;
+    m.sm_ones = 0;
+    if (m1 >= 1 && bits(m1, m.surv, m.sm_ones)) m.sm_m = m1;
     const int m2 = std::min(13, 26 / m.sbits);
-    if (m2 > m1 && bits(m2, m.surv2)) m.sm_m2 = m2;
+    m.sm_ones2 = m.sm_ones;
+    if (m2 > m1 && bits(m2, m.surv2, m.sm_ones2)) m.sm_m2 = m2;
     build_sieve(m);
-    build_level3(m);
     build_walk(m);
 }
 
@@ -561,12 +565,12 @@ static int build_host_image(Machine &m) {
         return PFSM_E_NOMEM;
     }
     uint8_t *img = static_cast<uint8_t *>(h);
-    memset(img, 0, bytes);
     size_t o = 0;
     auto put = [&](const void *src, size_t n, size_t pad) {
-        const size_t at = o;
-        if (n) memcpy(img + o, src, n);
-        o += align256(n + pad);
+        const size_t at = o, end = at + align256(n + pad);
+        if (n) memcpy(img + at, src, n);
+        if (end <= bytes) memset(img + at + n, 0, end - at - n);   // (up to the next section)
+        o = end;
         return at;
     };
     m.o_memo = put(m.memo.data(), m.memo.size() * 2, 4);
@@ -1338,16 +1342,33 @@ static int finish_load(pfsm_ctx *ctx, Machine &&m, pfsm_aut *out_id) {
     m.k = m.params.prefix_k < 0 ? 0 : m.params.prefix_k;
     if (m.k * m.sbits > 16) m.k = 16 / m.sbits;
     if (!m.ecl_off.empty() && m.k < 1) m.k = 1;   // epsilon edges: no start steps from a bare q0
-    while (!build_memo(m)) {
-        if (--m.k <= 0) {
-            if (!m.ecl_off.empty()) return PFSM_E_INVAL;
-            m.k = 0;
-            build_memo(m);
-            break;
+    // the prefix table and its records beside the bitmaps: neither reads what
+    // the other writes
+    auto records = [&m]() {
+        while (!build_memo(m)) {
+            if (--m.k <= 0) {
+                if (!m.ecl_off.empty()) return false;
+                m.k = 0;
+                build_memo(m);
+                break;
+            }
         }
+        return true;
+    };
+    if (m.kind == 1) {
+        std::future<bool> beside;
+        try {
+            beside = std::async(std::launch::async, records);
+        } catch (const std::system_error &) {   // no more threads
+        }
+        build_survival(m);
+        if (!(beside.valid() ? beside.get() : records())) return PFSM_E_INVAL;
+    } else {
+        records();   // (a DFA's always builds)
+        build_survival(m);
     }
     m.params.prefix_k = m.k > 0 ? m.k : -1;
-    build_survival(m);
+    build_level3(m);
     DeviceGuard g(ctx->device);
     const int id = ctx->next_id++;
     auto &slot = ctx->machines[id];

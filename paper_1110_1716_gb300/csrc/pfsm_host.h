@@ -46,6 +46,7 @@ struct Machine {
     std::vector<uint32_t> band;   // NFA band image (S <= 4) or empty
     // survival bitmap over m-grams (m = 0: none)
     int sm_m = 0, sm_m2 = 0;
+    uint64_t sm_ones = 0, sm_ones2 = 0;   // grams set in them
     std::vector<uint32_t> surv, surv2;   // shallow (shared memory) and deep (global) bitmaps
     // sieve tables (see SIEVE_DNA_STEP): kind, near and deep bitmaps
     int sv_kind = 0;
@@ -195,7 +196,7 @@ void build_sieve(Machine &m);                                              // si
 void build_level3(Machine &m);
 void build_walk(Machine &m);
 bool default_params(const Machine &m);   // pfsm_api.cu: nothing but the prefix depth was set
-bool survival_bits_dna(const Machine &m, int mm, std::vector<uint32_t> &bits);
+bool survival_bits_dna(const Machine &m, int mm, std::vector<uint32_t> &bits, uint64_t &grams);
 size_t align256(size_t x);
 void release(pfsm_ctx *ctx, Machine &m);
 void drop_host_image(Machine &m);
