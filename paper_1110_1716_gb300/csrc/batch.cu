@@ -459,8 +459,13 @@ static int plan_batch(pfsm_ctx *ctx, const pfsm_job *jobs, int32_t k, BatchPlan 
         pl.used.push_back(&m);
         flat_of[i] = flat_class(ctx, m);
     }
-    for (int &c : flat_of)
+    std::vector<uint64_t> symbols(ids.size(), 0);
+    for (int32_t i = 0; i < k; ++i) symbols[job_slot[i]] += jobs[i].n;
+    for (size_t i = 0; i < ids.size(); ++i) {
+        int &c = flat_of[i];
         if ((c == FLAT_DNA || c == FLAT_BYTES) && !have_lists(ctx, s)) c = -1;
+        if (c == FLAT_WALK && !walk_takes_batch(*pl.used[i], symbols[i])) c = -1;
+    }
     for (int32_t i = 0; i < k; ++i) {
         if (jobs[i].n >= (1ull << 32) - 256) flat_of[job_slot[i]] = -1;   // positions would wrap
     }

@@ -1022,7 +1022,7 @@ bool default_params(const Machine &m) {
 enum Route { ROUTE_TILES, ROUTE_SIEVE, ROUTE_WALK };
 static Route route_of(const pfsm_ctx *ctx, const Machine &m, uint64_t n, cudaStream_t s) {
     const bool sieve = m.sv_kind && m.k > 0;
-    if ((!sieve && !m.walks) || !m.full || ctx->hold_tiles || n == 0 || n >= (1ull << 32) - 256) return ROUTE_TILES;
+    if ((!sieve && !(m.walks && n < m.walk_limit)) || !m.full || ctx->hold_tiles || n == 0 || n >= (1ull << 32) - 256) return ROUTE_TILES;
     if (!default_params(m)) return ROUTE_TILES;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {

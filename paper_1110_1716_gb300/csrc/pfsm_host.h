@@ -65,6 +65,10 @@ struct Machine {
     bool walks = false, lives = false;
     std::vector<uint32_t> walk_tab;
     uint32_t walk_first[2] = {0, 0}, walk_finals[2] = {0, 0};
+    // NFA: states that an instance holds, summed over its life (the mean of
+    // uniform texts; past 3: not counted further)
+    double walk_states = 0;
+    uint64_t walk_limit = 0;   // symbols of a text from which the tile kernel is the faster one
     bool walk_bitset() const { return kind == 1 || lives; }
     pfsm_params params{};
     // residency: the device image is built once in pinned host memory and
@@ -196,6 +200,7 @@ void build_sieve(Machine &m);                                              // si
 void build_level3(Machine &m);
 void build_walk(Machine &m);
 bool default_params(const Machine &m);   // pfsm_api.cu: nothing but the prefix depth was set
+bool walk_takes_batch(const Machine &m, uint64_t n);   // whether texts of n symbols in all run flat
 bool survival_bits_dna(const Machine &m, int mm, std::vector<uint32_t> &bits, uint64_t &grams);
 size_t align256(size_t x);
 void release(pfsm_ctx *ctx, Machine &m);

@@ -523,28 +523,89 @@ static bool bitset_table(Machine &m, const Delta &d) {
     return true;
 }
 
+// Instances of a machine of at most 64 states on uniform symbols.
+namespace {
+struct Tries {
+    int S;
+    std::vector<uint64_t> to;   // per state and symbol
+    uint64_t first = 0, x = 0x9E3779B97F4A7C15ull;
+    Tries(const Machine &m, const Delta &d) : S(m.S), to(static_cast<size_t>(m.Q) * m.S, 0) {
+        for (int q = 0; q < m.Q; ++q)
+            for (uint32_t e = d.row[q]; e < d.row[q + 1]; ++e)
+                to[static_cast<size_t>(q) * S + d.sym[e]] |= 1ull << (d.tgt[e] & 0x7FFF);
+        for (uint16_t q : d.start) first |= 1ull << q;
+    }
+    uint64_t step(uint64_t s) {
+        x = x * 6364136223846793005ull + 1442695040888963407ull;
+        const uint32_t a = static_cast<uint32_t>(((x >> 32) * static_cast<uint64_t>(S)) >> 32);
+        uint64_t n = 0;
+        for (; s; s &= s - 1) n |= to[static_cast<size_t>(__builtin_ctzll(s)) * S + a];
+        return n;
+    }
+};
+}  // namespace
+
 // Whether 1 in 16 or more of the instances live for 256 uniform symbols
 // (tried on 256 fixed texts).
 static bool lives_long(const Machine &m, const Delta &d) {
-    std::vector<uint64_t> to(static_cast<size_t>(m.Q) * m.S, 0);
-    for (int q = 0; q < m.Q; ++q)
-        for (uint32_t e = d.row[q]; e < d.row[q + 1]; ++e)
-            to[static_cast<size_t>(q) * m.S + d.sym[e]] |= 1ull << (d.tgt[e] & 0x7FFF);
-    uint64_t first = 0, x = 0x9E3779B97F4A7C15ull;
-    for (uint16_t q : d.start) first |= 1ull << q;
+    Tries t(m, d);
     int alive = 0;
-    for (int t = 0; t < 256; ++t) {
-        uint64_t s = first;
-        for (int j = 0; j < 256 && s; ++j) {
-            x = x * 6364136223846793005ull + 1442695040888963407ull;
-            const uint32_t a = static_cast<uint32_t>(((x >> 32) * static_cast<uint64_t>(m.S)) >> 32);
-            uint64_t n = 0;
-            for (; s; s &= s - 1) n |= to[static_cast<size_t>(__builtin_ctzll(s)) * m.S + a];
-            s = n;
-        }
+    for (int i = 0; i < 256; ++i) {
+        uint64_t s = t.first;
+        for (int j = 0; j < 256 && s; ++j) s = t.step(s);
         alive += s != 0;
     }
     return alive >= 16;
+}
+
+// Machine::walk_states (of 2048 instances).
+static double states_held(const Machine &m, const Delta &d) {
+    Tries t(m, d);
+    constexpr int runs = 2048;
+    uint64_t sum = 0;
+    for (int i = 0; i < runs && sum <= 3 * runs; ++i)
+        for (uint64_t s = t.step(t.first); s && sum <= 3 * runs; s = t.step(s))
+            sum += static_cast<uint64_t>(__builtin_popcountll(s));
+    return static_cast<double>(sum) / runs;
+}
+
+// From how many symbols on the tile kernel, which drops most starts by the
+// shallow bitmap before it steps them, beats the direct scan, which steps every
+// one. It costs more to begin with (10 - 40 us a scan) and less per symbol
+// where few starts are left. us per 2^20 symbols, of long texts:
+//   DFAs: the direct scan 7, the tile kernel by the share of starts left and
+//   the width of a symbol: 0.04 - 0.07 of DNA 5 - 6, 0.13 9; bytes 0.02 1.7,
+//   0.16 6.5, 0.27 11; 0.09 of 20 symbols 12
+//   NFAs: the direct scan by the words read per symbol, 8.5 + 2.4 per eight
+//   states of a one-word set, 8 per eight of a two-word set; the tile kernel
+//   5 where few starts are left, and where a quarter is, 8 and 8 more for every
+//   state that a start holds over its life (32 states 12 and 15, 64 states
+//   11 - 44; sets that grow 600)
+// Whole scans, direct and tiles: 64-state DNA DFA 4 MiB 42, 56, 8 MiB 71, 60,
+// 64 MiB 501, 410; 64 states over bytes 2 MiB 26, 28, 4 MiB 41, 29, 64 MiB
+// 461, 116; NFAs of 64 states 1 MiB 87, 37 and 104, 137, 2 MiB 150, 47 and
+// 177, 153; of 32, 4 MiB 88, 122, 8 MiB 161, 129.
+static uint64_t walk_limit(const Machine &m) {
+    constexpr uint64_t MiB = 1ull << 20, none = ~0ull;
+    if (m.sm_m == 0 || m.lives) return none;
+    const double left = static_cast<double>(m.sm_ones) / static_cast<double>(1ull << (m.sm_m * m.sbits));
+    if (m.kind == 0) {
+        if (m.sbits == 8) return left <= 1 / 32.0 ? 4 * MiB : left <= 1 / 6.0 ? 8 * MiB : none;
+        return left <= (m.sbits == 2 ? 1 / 8.0 : m.sbits == 7 ? 1 / 16.0 : 1 / 24.0) ? 8 * MiB : none;
+    }
+    if (m.sbits > 3 || m.walk_states > 2.5) return none;
+    const int words = (m.Q + 7) / 8;
+    const double walk = m.Q > 32 ? 8.0 * words : 8.5 + 2.4 * words;
+    const double gain = walk - (5 + (3 + 8 * m.walk_states) * std::min(1.0, 4 * left));
+    return gain < 1.5 ? none : std::max(MiB / 2, static_cast<uint64_t>(20 / gain * MiB));
+}
+
+// In a batch the class kernels come with a graph launch (one machine's texts,
+// direct and class kernels: 64 states over bytes, 64 of 64 KiB 66, 56, 16 of
+// 1 MiB 187, 81; 64-state DNA DFA, 16 of 1 MiB 228, 269, 64 of 1 MiB 912, 858;
+// NFA of 32 states, 64 of 64 KiB 121, 139, 16 of 1 MiB 411, 337).
+bool walk_takes_batch(const Machine &m, uint64_t n) {
+    return m.walks && (m.walk_limit == ~0ull || n < (m.kind == 1 ? 2 : m.sbits == 8 ? 1 : 8) * m.walk_limit);
 }
 
 // Whether the machine's scans walk every start (walk.cu), and the tables for
@@ -555,6 +616,7 @@ static bool lives_long(const Machine &m, const Delta &d) {
 void build_walk(Machine &m) {
     m.walks = m.lives = false;
     m.walk_tab.clear();
+    m.walk_limit = ~0ull;
     if (m.sv_kind != SIEVE_NONE) return;
     if (m.kind == 0) {
         if (static_cast<size_t>(m.Q) * m.S * 2 > 160 * 1024) return;
@@ -570,6 +632,8 @@ void build_walk(Machine &m) {
         m.lives = lives_long(m, d);
         if ((m.kind == 1 || m.lives) && bitset_table(m, d)) {
             m.walks = true;
+            if (!m.lives) m.walk_states = states_held(m, d);
+            m.walk_limit = walk_limit(m);
             return;
         }
         m.lives = false;
@@ -583,6 +647,7 @@ void build_walk(Machine &m) {
     m.walk_tab.assign((cells + m.S + 1) / 2, 0u);
     memcpy(m.walk_tab.data(), t.data(), m.walk_tab.size() * 4);
     m.walks = true;
+    m.walk_limit = walk_limit(m);
 }
 
 // The survival bitmap of an NFA over 2-bit symbols (bit set: an instance

@@ -29,6 +29,7 @@ int batch_class(int kind, int, int, bool) { return kind ? 6 : 0; }
 cudaError_t launch_units(int, const BatchArgs *, int, int, uint32_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_carry_batch(const BatchArgs *, int, cudaStream_t) { return cudaSuccess; }
 bool default_params(const Machine &) { return true; }
+bool walk_takes_batch(const Machine &, uint64_t) { return true; }
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 int ensure_words(uint32_t **, size_t *, size_t) { return PFSM_OK; }
 int make_resident(pfsm_ctx *, int, Machine &m, cudaStream_t, bool) { return m.full = true, PFSM_OK; }

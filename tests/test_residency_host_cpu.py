@@ -168,3 +168,38 @@ def test_a_batch_that_does_not_fit_is_still_refused(lib):
         a, b = h.load(make())[1], h.load(make())[1]
         assert batch(h, [a, b])[0] == E_NOMEM
         assert h.scan(a)[0] == OK and h.scan(b)[0] == OK and batch(h, [a])[0] == OK
+
+
+def random_nfa(Q, S, seed, p):
+    rng = np.random.default_rng(seed)
+    edges = [(q, x, t) for q in range(Q) for x in range(S) for t in range(Q) if rng.random() < p / Q]
+    return W.nfa_from_edges(Q, S, 0, edges, [q for q in range(Q) if rng.random() < 0.2] or [Q - 1])
+
+
+MIB = 1 << 20
+
+
+@pytest.mark.parametrize("make,below,above", [
+    (lambda: W.dfa_random(11), 8 * MIB - 1, 8 * MIB),                        # 0.07 of the starts left by the bitmap
+    (lambda: W.dfa_random(1), 99 * MIB, None),                               # 0.75
+    (lambda: W.dfa_random(12, Q=64, S=256, p_dead=0.9), 4 * MIB - 1, 4 * MIB),   # 0.02
+    (lambda: W.dfa_random(12, Q=64, S=256, p_dead=0.3), 99 * MIB, None),
+    (lambda: random_nfa(64, 4, 3, 0.5), MIB // 2 - 1, MIB // 2),             # 0.8 states held
+    (lambda: random_nfa(64, 4, 64, 0.9), 99 * MIB, None),                    # 6.6
+    (lambda: random_nfa(32, 4, 32, 0.9), 99 * MIB, None),                    # no bitmap
+    (lambda: random_nfa(8, 4, 8, 0.3), 99 * MIB, None),
+    (lambda: random_nfa(32, 4, 32, 0.3), 4 * MIB, 9 * MIB),
+    (lambda: random_nfa(40, 2, 47, 0.6), MIB // 2 - 1, MIB),                 # hardly any start left
+])
+def test_texts_too_long_for_the_direct_scan(lib, make, below, above):
+    with Host(lib) as h:
+        st, a = h.load(make())
+        assert h.scan(a, below) == (OK, ["walk"])
+        if above:
+            assert h.scan(a, above) == (OK, ["tiles"])
+
+
+def test_long_lived_instances_keep_to_their_segments(lib):
+    with Host(lib) as h:
+        st, a = h.load(W.live_core_nfa(5, 7))
+        assert h.scan(a, 99 * MIB) == (OK, ["long"])
