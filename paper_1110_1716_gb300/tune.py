@@ -6,8 +6,9 @@ round, filtering threads, tile length, persistent CTAs per SM, DFA table
 placement, NFA settling cap). Starting from the library's defaults, each
 axis in turn tries its values with the others fixed at the best found so
 far, timed with CUDA events around the scan on one stream; two sweeps. The
-result is cached in a JSON file keyed by (kind, |Q|, |Sigma|, GPU name), so a
-machine of the same shape is tuned once per GPU model.
+result is cached in a JSON file keyed by (version of the kernels, kind, |Q|,
+|Sigma|, GPU name), so a machine of the same shape is tuned once per GPU model,
+and again when the kernels that the parameters choose from have changed.
 
 Batch (``tune_batch``): the launch shape of the batch class kernels (threads
 and CTAs per SM, tile length), then per machine the DFA table placement
@@ -38,8 +39,14 @@ CACHE_PATH = os.environ.get("PFSM_TUNE_CACHE") or _default_cache_path()
 _lock = threading.Lock()
 
 
+# Raised when a choice stored by an older library may no longer be the best:
+# 2: machines with default parameters take the sieve or the direct scan, which
+# parameters off their defaults keep them from.
+CACHE_VERSION = 2
+
+
 def _key(kind: str, Q: int, S: int, gpu: str) -> str:
-    return "%s/Q%d/S%d/%s" % (kind, Q, S, gpu)
+    return "v%d/%s/Q%d/S%d/%s" % (CACHE_VERSION, kind, Q, S, gpu)
 
 
 def _load_cache() -> Dict[str, dict]:

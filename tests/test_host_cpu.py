@@ -190,3 +190,24 @@ def test_bench_compact_configs_keep_every_config():
     assert out["f2_long_lived_nfa_16kib"] == {"lazy_ms": 860.0, "chained_ms": 100.0, "matches": 6}
     assert out["c4_serving"]["max_pass_ms_by_load"]["0.25"] == [9.0, 8.5]
     assert out["c3_batch_10k_texts"]["params_source"] == "autotuner"
+
+
+def test_choices_of_an_older_library_are_not_taken(tmp_path, monkeypatch):
+    """An entry of the cache without the version, as libraries before the
+    direct scan and the sieve stored them, is searched anew; the new choice is
+    then taken as it was stored."""
+    import pytest
+    torch = pytest.importorskip("torch")
+    from paper_1110_1716_gb300 import tune
+    path = tmp_path / "cache.json"
+    path.write_text(json.dumps({"dfa/Q64/S4/gpu": {"params": {"settle": 16}, "ms": 1.0}}))
+    monkeypatch.setattr(tune, "CACHE_PATH", str(path))
+    state, searches = {"params": {"prefix_k": 6, "settle": 8}}, []
+    monkeypatch.setattr(tune, "pfsm_set_params", lambda ctx, aut, p: state.update(params=dict(p)))
+    monkeypatch.setattr(tune, "pfsm_get_params", lambda ctx, aut: dict(state["params"]))
+    monkeypatch.setattr(tune, "pfsm_scan", lambda *a: (0, 0))
+    monkeypatch.setattr(tune, "_descend", lambda start, *a, **k: (searches.append(1) or dict(start), 1.0, 1))
+    text, machine = torch.zeros(8, dtype=torch.uint8), W.dfa_random(1)
+    for _ in range(2):
+        assert tune.tune(0, 1, machine, text, gpu_name="gpu")["settle"] == 8
+    assert len(searches) == 1
