@@ -22,7 +22,7 @@
 #include <algorithm>
 #include <atomic>
 
-#include "sieve.cuh"
+#include "finish.cuh"
 #include "walk.cuh"
 
 namespace pfsm {
@@ -180,111 +180,13 @@ __global__ void __launch_bounds__(BIG ? 1024 : 128, 1) flat_front(const __grid_c
 }
 
 // ------------------------------------------------------------ candidates
-// A warp's matches on their way out: rows in shared memory that leave with one
-// atomic per few dozen and one per text among them. (With one atomic on the
-// batch's count per row of lanes, texts dense in matches waited for it: one
-// text of 64 MiB and 1.08 M matches 694 us, now 326; 4 MiB and 0.23 M 283 us,
-// now 186.) Rows are written word by word: the caller's buffer may begin at
-// any multiple of four bytes.
-constexpr uint32_t kFlatRows = 64;
-struct FlatOut {
-    uint4 *rows;
-    uint32_t n;
-};
-__device__ __forceinline__ void flat_flush(const FlatArgs &A, FlatOut &out, int lane) {
-    if (out.n == 0) return;
-    __syncwarp();
-    unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(&A.status[0], static_cast<unsigned long long>(out.n));
-    base = __shfl_sync(FULLMASK, base, 0);
-    for (uint32_t r = lane; r < (out.n + 31) / 32 * 32; r += 32) {
-        const uint32_t m = __ballot_sync(FULLMASK, r < out.n);
-        if (r < out.n) {
-            const uint32_t orig = out.rows[r].x, peers = __match_any_sync(m, orig);
-            if (lane == __ffs(peers) - 1) atomicAdd(&A.job_counts[orig], static_cast<unsigned long long>(__popc(peers)));
-        }
-    }
-    const uint32_t words =
-        base >= A.cap ? 0u : 4 * static_cast<uint32_t>(min(static_cast<unsigned long long>(out.n), A.cap - base));
-    uint32_t *o = A.out + base * 4;
-    const uint32_t *from = reinterpret_cast<const uint32_t *>(out.rows);
-    for (uint32_t w = lane; w < words; w += 32) o[w] = from[w];
-    __syncwarp();
-    out.n = 0;
-}
+using FlatOut = RowOut<4, FlatArgs>;
 
-// The match (start, end, st) of every lane with `has`.
-__device__ __forceinline__ void flat_emit(const FlatArgs &A, FlatOut &out, bool has, uint32_t orig, uint32_t start,
-                                          uint32_t end, uint32_t st, int lane) {
-    const uint32_t m = __ballot_sync(FULLMASK, has);
-    if (m == 0) return;
-    if (out.n + __popc(m) > kFlatRows) flat_flush(A, out, lane);
-    if (has) out.rows[out.n + __popc(m & lanemask_lt())] = make_uint4(orig, start, end, st);
-    out.n += __popc(m);
-}
-
-// One DFA candidate per lane (see finish_dfa).
+// One DFA candidate per lane, each with its own text and machine.
 __device__ __forceinline__ void flat_dfa(const FlatArgs &A, FlatOut &out, bool act, uint32_t job, uint32_t start, int lane,
                                          uint64_t pol_keep) {
     const BatchJob &J = A.jobs[job];
-    const DevMachine &M = A.machs[J.mach];
-    const uint32_t n = J.n, S = M.S, orig = J.orig;
-    const uintptr_t text = reinterpret_cast<uintptr_t>(J.text), end = text + n;
-    const uint4 *chain = M.chain;
-    const uint16_t *dtab = M.dtab;
-    uint32_t pos = start, s = M.q0;
-    const uint32_t kk = static_cast<uint32_t>(M.k);
-    if (act && n - start >= kk) {
-        const uint64_t w = bytes8_at(text, end, pos);
-        uint32_t gi = 0;
-        bool in = true;
-        for (uint32_t j = 0; j < kk; ++j) {
-            const uint32_t c = static_cast<uint32_t>(w >> (8 * j)) & 0xFFu;
-            in &= c < S;
-            gi |= c << (j * M.sbits);
-        }
-        if (in) {
-            const uint32_t e = ldg_u16_keep(M.memo + gi, pol_keep);
-            if (e == PT_SKIP) {
-                act = false;
-            } else if (!(e & PT_REC)) {   // a state; records and walks step from q0
-                s = e;
-                pos += kk;
-                if (pos >= n) act = false;
-            }
-        }
-    }
-    while (__any_sync(FULLMASK, act)) {
-        bool hit = false;
-        if (act) {
-            if (!PFSM_OK_IDX(s < static_cast<uint32_t>(M.Q), A.status)) s = 0;
-            const uint4 ch = __ldg(chain + s);
-            const uint64_t w = bytes8_at(text, end, pos);
-            const uint32_t len = ch.z & 0xFFu;
-            if (len) {
-                const uint64_t want = ch.x | (static_cast<uint64_t>(ch.y) << 32);
-                if (n - pos < len || ((w ^ want) << (64 - 8 * len)) != 0) {
-                    act = false;
-                } else {
-                    s = ch.w;
-                    pos += len;
-                    hit = (ch.z >> 8) & 1u;
-                }
-            } else {
-                const uint32_t c = static_cast<uint32_t>(w) & 0xFFu;
-                const uint32_t e = c < S ? ldg_u16_keep(dtab + s * S + c, pol_keep) : DEAD16;
-                if (e == DEAD16) {
-                    act = false;
-                } else {
-                    s = e & 0x7FFFu;
-                    hit = (e & FINAL_BIT) != 0;
-                    ++pos;
-                }
-            }
-            if (pos >= n) act = false;
-        }
-        flat_emit(A, out, hit, orig, start, pos - 1, s, lane);
-    }
+    run_dfa(J, A.machs[J.mach], J.orig, act, start, out, lane, pol_keep);
 }
 
 // One NFA candidate per lane with its second-level record: the record's
@@ -328,7 +230,7 @@ __device__ __forceinline__ void flat_nfa(const FlatArgs &A, FlatOut &out, bool a
     for (uint32_t x = 0; __any_sync(FULLMASK, x < matches); ++x) {
         const uint32_t w = x < matches ? __ldg(r + 1 + x) : 0u;
         const uint32_t step = w >> 16;
-        flat_emit(A, out, x < matches && step < n - start, orig, start, start + step, w & 0xFFFFu, lane);
+        out.emit(x < matches && step < n - start, orig, start, start + step, w & 0xFFFFu, lane);
     }
     uint32_t incl = parts;
 #pragma unroll
@@ -382,7 +284,7 @@ __device__ __forceinline__ void flat_nfa(const FlatArgs &A, FlatOut &out, bool a
                 hits = mask & (__funnelshift_r(f0, f1, o) | (static_cast<uint64_t>(__funnelshift_r(f1, f2, o)) << 32));
             }
             while (__any_sync(FULLMASK, hits != 0)) {
-                flat_emit(A, out, hits != 0, iorig, istart, pos, base + (hits ? __ffsll(static_cast<long long>(hits)) - 1 : 0), lane);
+                out.emit(hits != 0, iorig, istart, pos, base + (hits ? __ffsll(static_cast<long long>(hits)) - 1 : 0), lane);
                 hits &= hits - 1;
             }
             ++pos;
@@ -395,24 +297,21 @@ __device__ __forceinline__ void flat_nfa(const FlatArgs &A, FlatOut &out, bool a
     __syncwarp();
 }
 
-// Candidates of the fallback, collected per warp: starts that pass the deep
-// bitmap, then those with a record.
+// Candidates of the fallback, collected per warp: starts that the bitmap of
+// single starts leaves, then (NFA) those with a record.
 struct FlatEvery {
     uint2 starts[64];      // {start, its first 16 symbols}
     uint4 found[64];       // as the list of the front kernel has them
     unsigned long long n;  // entries of found
 };
 
-// Every start of one NFA's steps [b0, b1), as the front kernel and the list
-// would have brought them: four starts per lane through the bitmap of single
-// starts, then the records and the runs of full warps of what is left. (Runs
-// of the one start in twenty that has a record, 32 starts at a time, left the
-// other lanes idle: 64 MiB dense in motifs 8.3 ms.)
-static __device__ __noinline__ void flat_every_nfa(const FlatArgs &A, uint32_t j, uint32_t b0, uint32_t b1, FlatEvery &E,
+// The starts [from, to) of one NFA's text, as the front kernel and the list
+// would have brought them: four starts per lane through the bitmap, then the
+// records and the runs of full warps of what is left.
+__device__ __forceinline__ void flat_every_nfa(const FlatArgs &A, uint32_t j, uint64_t from, uint64_t to, FlatEvery &E,
                                                uint4 *items, FlatOut &out, int lane, uint64_t pol_keep) {
     const BatchJob &J = A.jobs[j];
     const DevMachine &M = A.machs[J.mach];
-    constexpr uint32_t SPAN = flat_step(FLAT_DNA, false);
     SieveArgs a{};
     a.text = J.text;
     a.n = J.n;
@@ -440,19 +339,11 @@ static __device__ __noinline__ void flat_every_nfa(const FlatArgs &A, uint32_t j
         if (lane == 0) E.n = n;
         __syncwarp();
     };
-    const uint64_t to = min(static_cast<uint64_t>(J.n), static_cast<uint64_t>(b1) * SPAN);
-    for (uint64_t s0 = static_cast<uint64_t>(b0) * SPAN; s0 < to; s0 += 128) {
-        const uint64_t first = s0 + 4 * lane;
-        uint32_t g0 = 0, g1 = 0, keep = 0;
-        if (first < to) {
-            pack32_at(a.text, a.n, static_cast<uint32_t>(first), g0, g1);
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const uint32_t g = __funnelshift_r(g0, g1, 2 * r) & ((1u << (2 * SIEVE_DEEP_M)) - 1);
-                const uint32_t w = first + r + SIEVE_DEEP_M <= a.n ? ldg_u32_keep(surv2 + (g >> 5), pol_keep) >> (g & 31) : 1u;
-                keep |= (first + r < to ? w & 1u : 0u) << r;
-            }
-        }
+    for (; from < to; from += 128) {
+        const uint64_t first = from + 4 * lane;
+        const uint32_t keep = starts_left(a.text, a.n, first, to, surv2, SIEVE_DEEP_M, 2, pol_keep);
+        uint32_t g0 = 0, g1 = 0;
+        if (keep) pack32_at(a.text, a.n, static_cast<uint32_t>(first), g0, g1);
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const uint32_t m = __ballot_sync(FULLMASK, (keep >> r) & 1u);
@@ -473,37 +364,45 @@ static __device__ __noinline__ void flat_every_nfa(const FlatArgs &A, uint32_t j
     run(true);
 }
 
-// Even CTAs run the DFA candidates, odd ones the NFA candidates. A list that
-// overflowed is replaced by every start of the texts of its kind.
-__global__ void __launch_bounds__(256, 4) flat_finish(const __grid_constant__ FlatArgs A) {
-    __shared__ uint4 items_sm[8][32 * SIEVE_PARTS];
-    __shared__ FlatEvery every_sm[8];
-    __shared__ uint4 rows_sm[8][kFlatRows];
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint64_t pol_keep = policy_evict_last();
-    const uint32_t kind = blockIdx.x & 1, ctas = gridDim.x / 2;
-    const unsigned long long found = A.cand_n[kind];
-    const uint64_t warps = static_cast<uint64_t>(ctas) * 8, me = static_cast<uint64_t>(wid) * ctas + blockIdx.x / 2;
-    uint4 *items = items_sm[wid];
-    FlatOut out{rows_sm[wid], 0u};
-    if (found <= A.cand_cap) {
-        const uint32_t per = static_cast<uint32_t>(min(32ull, (found + warps - 1) / warps));
-        for (uint64_t x0 = me * per; x0 < found; x0 += warps * per) {
-            const bool act = static_cast<uint32_t>(lane) < per && x0 + lane < found;
-            const uint4 c = act ? A.cand[kind][x0 + lane] : A.cand[kind][x0];
-            if (kind == 0) flat_dfa(A, out, act, c.x, c.y, lane, pol_keep);
-            else flat_nfa(A, out, act, c.x, c.y, c.z, items, lane);
+// The same for a DFA.
+__device__ __forceinline__ void flat_every_dfa(const FlatArgs &A, uint32_t j, uint64_t from, uint64_t to, FlatEvery &E,
+                                               FlatOut &out, int lane, uint64_t pol_keep) {
+    const BatchJob &J = A.jobs[j];
+    const DevMachine &M = A.machs[J.mach];
+    uint32_t *left = reinterpret_cast<uint32_t *>(E.found), cnt = 0;   // (160 of its 256 words)
+    while (from < to || cnt) {
+        for (; cnt < 32 && from < to; from += 128) {
+            const uint64_t first = from + 4 * lane;
+            const uint32_t keep = starts_left(J.text, J.n, first, to, M.surv2, M.surv2 ? M.surv2_m : 0, M.sbits, pol_keep);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const uint32_t m = __ballot_sync(FULLMASK, (keep >> r) & 1u);
+                if ((keep >> r) & 1u) left[cnt + __popc(m & lanemask_lt())] = static_cast<uint32_t>(first) + r;
+                cnt += __popc(m);
+            }
         }
-        flat_flush(A, out, lane);
-        return;
+        const uint32_t k = min(cnt, 32u);
+        cnt -= k;
+        __syncwarp();
+        const bool act = static_cast<uint32_t>(lane) < k;
+        const uint32_t start = act ? left[cnt + lane] : 0u;
+        __syncwarp();
+        if (k) flat_dfa(A, out, act, j, start, lane, pol_keep);
     }
-    // a few steps at a time, dealt out in turn: texts may be long, and what a
-    // start costs differs from place to place
-    if (lane == 0) every_sm[wid].n = 0;
+}
+
+// Every start of the texts of one kind, a few steps at a time, dealt out in
+// turn to `warps` warps (this one is the me-th): texts may be long, and what a
+// start costs differs from place to place. A function of its own, so that the
+// kernel needs no more registers than the candidates do.
+static __device__ __noinline__ void flat_every(const FlatArgs &A, uint32_t kind, uint64_t me, uint64_t warps, FlatEvery &E,
+                                               uint4 *items, uint32_t *rows, int lane) {
+    const uint64_t pol_keep = policy_evict_last();
+    if (lane == 0) E.n = 0;
+    FlatOut out{A, rows, 0u};
     for (int c = 0; c < FLAT_WALK; ++c) {
         const uint64_t span = flat_step(c, false);   // (the same in both forms)
-        const uint32_t steps = static_cast<uint32_t>(A.steps[c]), each = kind == 0 ? 1u : 8u;
+        const uint32_t steps = static_cast<uint32_t>(A.steps[c]), each = c == FLAT_DNA ? 8u : 2u;
         for (uint64_t x = me * each; x < steps; x += warps * each) {
             uint32_t s0 = static_cast<uint32_t>(x);
             const uint32_t s1 = static_cast<uint32_t>(min(static_cast<uint64_t>(steps), x + each));
@@ -512,17 +411,41 @@ __global__ void __launch_bounds__(256, 4) flat_finish(const __grid_constant__ Fl
                 const uint32_t b0 = s0 - J.unit_begin, b1 = min(J.ntiles, b0 + (s1 - s0));
                 s0 = j + 1 < A.job_hi[c] ? min(s1, A.jobs[j + 1].unit_begin) : s1;
                 if (b0 >= b1 || static_cast<uint32_t>(A.machs[J.mach].kind) != kind) continue;
-                if (kind == 1) {
-                    flat_every_nfa(A, j, b0, b1, every_sm[wid], items, out, lane, pol_keep);
-                    continue;
-                }
                 const uint64_t to = min(static_cast<uint64_t>(J.n), b1 * span);
-                for (uint64_t at = b0 * span; at < to; at += 32)
-                    flat_dfa(A, out, at + lane < to, j, static_cast<uint32_t>(at) + lane, lane, pol_keep);
+                if (kind == 1) flat_every_nfa(A, j, b0 * span, to, E, items, out, lane, pol_keep);
+                else flat_every_dfa(A, j, b0 * span, to, E, out, lane, pol_keep);
             }
         }
     }
-    flat_flush(A, out, lane);
+    out.flush(lane);
+}
+
+// Even CTAs run the DFA candidates, odd ones the NFA candidates. A list that
+// overflowed is replaced by every start of the texts of its kind.
+__global__ void __launch_bounds__(256, 4) flat_finish(const __grid_constant__ FlatArgs A) {
+    __shared__ uint4 items_sm[8][32 * SIEVE_PARTS];
+    __shared__ FlatEvery every_sm[8];
+    __shared__ uint32_t rows_sm[8][kOutRows * 4];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint64_t pol_keep = policy_evict_last();
+    const uint32_t kind = blockIdx.x & 1, ctas = gridDim.x / 2;
+    const unsigned long long found = A.cand_n[kind];
+    const uint64_t warps = static_cast<uint64_t>(ctas) * 8, me = static_cast<uint64_t>(wid) * ctas + blockIdx.x / 2;
+    uint4 *items = items_sm[wid];
+    if (found > A.cand_cap) {
+        flat_every(A, kind, me, warps, every_sm[wid], items, rows_sm[wid], lane);
+        return;
+    }
+    FlatOut out{A, rows_sm[wid], 0u};
+    const uint32_t per = static_cast<uint32_t>(min(32ull, (found + warps - 1) / warps));
+    for (uint64_t x0 = me * per; x0 < found; x0 += warps * per) {
+        const bool act = static_cast<uint32_t>(lane) < per && x0 + lane < found;
+        const uint4 c = act ? A.cand[kind][x0 + lane] : A.cand[kind][x0];
+        if (kind == 0) flat_dfa(A, out, act, c.x, c.y, lane, pol_keep);
+        else flat_nfa(A, out, act, c.x, c.y, c.z, items, lane);
+    }
+    out.flush(lane);
 }
 
 // ------------------------------------------------------------ host helpers

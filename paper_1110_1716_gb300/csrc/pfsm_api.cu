@@ -1124,6 +1124,8 @@ static int sieve_enqueue(pfsm_ctx *ctx, const Machine &m, const uint8_t *text, u
     a.deep = m.dm.sv_deep;
     // (bytes: single starts are tested by their 3-gram)
     a.surv2 = m.sv_kind == SIEVE_DNA || (m.sbits == 8 && m.sm_m2 == 3) ? m.dm.surv2 : nullptr;
+    a.all2 = m.dm.surv2;
+    a.all_m = m.sm_m2;
     a.dtab = m.dm.dtab;
     a.memo = m.dm.memo;
     a.chain = m.dm.chain;

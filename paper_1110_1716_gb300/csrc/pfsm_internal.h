@@ -207,6 +207,8 @@ struct SieveArgs {
     int32_t Q, S, q0;
     const uint32_t *near, *deep;   // sampled bitmaps (see SIEVE_DNA_STEP)
     const uint32_t *surv2;         // deep survival bitmap of single starts, or null (bytes)
+    const uint32_t *all2;          // deep survival bitmap of single starts, of all_m-grams (0: none), and
+    int32_t all_m;                 //   where the candidate list overflows, whatever the alphabet
     const uint16_t *dtab, *memo;   // DFA: table, prefix table (k symbols of sbits)
     const uint4 *chain;            // DFA: chains (see "A sieved DFA's chains")
     int32_t sbits;

@@ -21,7 +21,7 @@
 // start of the text instead (the list is then ignored): slower, same result.
 #include <atomic>
 
-#include "sieve.cuh"
+#include "finish.cuh"
 
 namespace pfsm {
 
@@ -76,95 +76,53 @@ __device__ __forceinline__ void finish_status_out(const SieveArgs &a) {
 }
 
 // ------------------------------------------------------------ candidates: DFA
-// One thread per candidate, over the text in global memory: the first k
-// symbols by the prefix table, then by chains (the only way on from
-// a state, up to eight symbols, compared at once) and single steps where the
-// automaton branches. What bounds a candidate is its chain of dependent
-// reads; a planted 32-byte signature takes some six instead of 32.
+// One thread per candidate (run_dfa), over the text in global memory.
+// Neighbouring candidates go to different CTAs, so that few of them still use
+// every SM. Where the list is incomplete, every start is looked at, 128 of a
+// warp at a time, and those left are run when a warp is full of them.
 __global__ void __launch_bounds__(256) finish_dfa(const SieveArgs a) {
+    __shared__ uint32_t rows_sm[8][kOutRows * 3];
+    __shared__ uint32_t left_sm[8][160];
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const uint32_t found = *a.cand_n;
-    const bool every = found > a.cand_cap;   // the list is incomplete: every start
-    const uint32_t total = every ? a.n : found;
+    const bool every = found > a.cand_cap;
+    const uint32_t total = every ? a.n : found, each = every ? 128u : 32u;
     const uint64_t pol_keep = policy_evict_last();
-    const int lane = threadIdx.x & 31;
-    const uint32_t n = a.n, S = a.S, kk = static_cast<uint32_t>(a.k);
-    const uintptr_t text = reinterpret_cast<uintptr_t>(a.text), end = text + n;
-    // neighbouring candidates go to different CTAs, so that few of them still
-    // use every SM
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint64_t warps = static_cast<uint64_t>(gridDim.x) * (blockDim.x >> 5);
-    const uint64_t gw = static_cast<uint64_t>(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-    for (uint64_t x0 = gw * 32; x0 < total; x0 += warps * 32) {
-        const uint64_t x = x0 + lane;
-        bool act = x < total;
-        const uint32_t start = !act ? 0u : every ? static_cast<uint32_t>(x) : a.cand[x].x;
-        uint32_t pos = start, s = a.q0;
-        if (act && kk && n - start >= kk) {
-            const uint64_t w = bytes8_at(text, end, pos);
-            uint32_t gi = 0;
-            bool in = true;
-            for (uint32_t j = 0; j < kk; ++j) {
-                const uint32_t c = static_cast<uint32_t>(w >> (8 * j)) & 0xFFu;
-                in &= c < S;
-                gi |= c << (j * a.sbits);
-            }
-            if (in) {
-                const uint32_t e = ldg_u16_keep(a.memo + gi, pol_keep);
-                if (e == PT_SKIP) {
-                    act = false;
-                } else if (!(e & PT_REC)) {   // a state; records and walks step from q0
-                    s = e;
-                    pos += kk;
-                    if (pos >= n) act = false;
+    RowOut<3, SieveArgs> out{a, rows_sm[wid], 0u};
+    uint32_t *left = left_sm[wid], cnt = 0;   // every: starts to run
+    uint64_t x0 = (static_cast<uint64_t>(wid) * gridDim.x + blockIdx.x) * each;
+    while (true) {
+        bool act;
+        uint32_t start = 0;
+        if (!every) {
+            if (x0 >= total) break;
+            act = x0 + lane < total;
+            if (act) start = a.cand[x0 + lane].x;
+            x0 += warps * each;
+        } else {
+            for (; cnt < 32 && x0 < total; x0 += warps * each) {
+                const uint64_t first = x0 + 4 * lane;
+                const uint32_t keep = starts_left(a.text, a.n, first, total, a.all2, a.all_m, a.sbits, pol_keep);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const uint32_t m = __ballot_sync(FULLMASK, (keep >> r) & 1u);
+                    if ((keep >> r) & 1u) left[cnt + __popc(m & lanemask_lt())] = static_cast<uint32_t>(first) + r;
+                    cnt += __popc(m);
                 }
             }
+            if (cnt == 0) break;
+            const uint32_t k = min(cnt, 32u);
+            cnt -= k;
+            __syncwarp();
+            act = static_cast<uint32_t>(lane) < k;
+            if (act) start = left[cnt + lane];
+            __syncwarp();
         }
-        while (__any_sync(FULLMASK, act)) {
-            bool hit = false;
-            if (act) {
-                if (!PFSM_OK_IDX(s < static_cast<uint32_t>(a.Q), a.status)) s = a.q0;
-                const uint4 ch = __ldg(a.chain + s);
-                const uint64_t w = bytes8_at(text, end, pos);
-                const uint32_t len = ch.z & 0xFFu;
-                if (len) {
-                    const uint64_t want = ch.x | (static_cast<uint64_t>(ch.y) << 32);
-                    // (no final state before the end of a chain: one that
-                    // passes the end of the text reports nothing)
-                    if (n - pos < len || ((w ^ want) << (64 - 8 * len)) != 0) {
-                        act = false;
-                    } else {
-                        s = ch.w;
-                        pos += len;
-                        hit = (ch.z >> 8) & 1u;
-                    }
-                } else {
-                    const uint32_t c = static_cast<uint32_t>(w) & 0xFFu;
-                    const uint32_t e = c < S ? ldg_u16_keep(a.dtab + s * S + c, pol_keep) : DEAD16;
-                    if (e == DEAD16) {
-                        act = false;
-                    } else {
-                        s = e & 0x7FFFu;
-                        hit = (e & FINAL_BIT) != 0;
-                        ++pos;
-                    }
-                }
-                if (pos >= n) act = false;
-            }
-            // the lanes that report on this symbol: one atomic
-            const uint32_t m = __ballot_sync(FULLMASK, hit);
-            if (m) {
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(&a.status[0], static_cast<unsigned long long>(__popc(m)));
-                base = __shfl_sync(FULLMASK, base, 0) + __popc(m & lanemask_lt());
-                if (hit && base < a.cap) {
-                    uint32_t *o = a.out + base * 3;
-                    o[0] = start;
-                    o[1] = pos - 1;
-                    o[2] = s;
-                }
-            }
-        }
+        run_dfa(a, a, 0u, act, start, out, lane, pol_keep);
     }
+    out.flush(lane);
     finish_status_out(a);
 }
 
@@ -448,7 +406,8 @@ static int finish_grid(uint32_t n, uint32_t symbols, int most) {
 }
 
 cudaError_t launch_finish_dfa(const SieveArgs &a, int nsm, cudaStream_t s) {
-    return launch_dependent(finish_dfa, finish_grid(a.n, 8192, 4 * nsm), 256, 0u, s, a);
+    // (eight CTAs fit an SM; four do but for long texts dense in candidates)
+    return launch_dependent(finish_dfa, finish_grid(a.n, 8192, (a.n >= 64u << 20 ? 8 : 4) * nsm), 256, 0u, s, a);
 }
 
 uint32_t layout_finish_nfa(ScanArgs &a, uint32_t band_bytes, uint32_t coop_bytes) {

@@ -244,16 +244,6 @@ static __device__ __noinline__ bool bad_step(const uint8_t *text, uint32_t n, ui
     return bad;
 }
 
-// The eight text bytes from position pos (those past the end of the text are
-// unspecified).
-__device__ __forceinline__ uint64_t bytes8_at(uintptr_t text, uintptr_t end, uint32_t pos) {
-    const uintptr_t at = text + pos, lo = at & ~static_cast<uintptr_t>(7);
-    const uint32_t sh = static_cast<uint32_t>(at & 7) * 8;
-    uint64_t w = __ldg(reinterpret_cast<const unsigned long long *>(lo)) >> sh;
-    if (sh && lo + 8 < end) w |= __ldg(reinterpret_cast<const unsigned long long *>(lo + 8)) << (64 - sh);
-    return w;
-}
-
 // One warp takes steps of 2 KB, from 16-byte boundaries of the address space
 // so that no text needs realigning; the four loads of a lane are in flight
 // together. A step wholly inside the text needs no bounds.
