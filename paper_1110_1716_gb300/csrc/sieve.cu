@@ -204,7 +204,13 @@ static __device__ __forceinline__ void run_items(const OView &ov, const MView &m
 // The candidates of an NFA, a warp's 32 at a time: those that come with a
 // second-level record report its matches and run on from its set, split into
 // strands (run_items); the others (near the end of the text, machines without
-// such tables, records of many states) take the general exact path.
+// such tables, records of many states) take the general exact path. Where the
+// list is incomplete, each warp uses a part of its place for starts that the
+// bitmap leaves (kEveryLeft) and those with a record (kEveryFound), and takes
+// its candidates from there.
+constexpr uint32_t kEveryLeft = 160, kEveryFound = 64;
+constexpr uint32_t kQueueBytes = WARP_QUEUE * 6 + WARP_QUEUE / 8;   // of a warp (smem_regions)
+static_assert(kQueueBytes % 4 == 0, "the counters behind the queues are aligned");
 __global__ void __launch_bounds__(kFinishThreads, 2) finish_nfa(const ScanArgs a, const SieveArgs sv) {
     extern __shared__ __align__(128) uint8_t smem[];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
@@ -233,11 +239,67 @@ __global__ void __launch_bounds__(kFinishThreads, 2) finish_nfa(const ScanArgs a
     const uint32_t mask = (1u << (2 * kk)) - 1;
     uint2 *items = reinterpret_cast<uint2 *>(smem + a.sm_list) + wid * kRunItems;   // {lane << 16 | base, mask}
     uint32_t sn = 0, wq_n = 0;
-    for (uint64_t x0 = (static_cast<uint64_t>(wid) * gridDim.x + blockIdx.x) * per; x0 < total;) {
-        const uint64_t x = x0 + lane;
-        bool have = static_cast<uint32_t>(lane) < per && x < total;
-        uint2 c = make_uint2(static_cast<uint32_t>(x), SIEVE_NO_RECORD);
-        if (have && !every) c = sv.cand[x];
+    const uint32_t each = every ? 128u : per;
+    const uint64_t warp = static_cast<uint64_t>(wid) * gridDim.x + blockIdx.x;
+    // (every) the warp's part of the list's place, and the entries of both lists
+    uint2 *left = sv.cand + warp * (kEveryLeft + kEveryFound);
+    uint32_t *found_sm = reinterpret_cast<uint32_t *>(smem + a.sm_queue + nw * kQueueBytes);
+    uint32_t cnt = 0, ready = 0;
+    SieveArgs lv = sv;
+    lv.cand = left + kEveryLeft;
+    lv.cand_n = found_sm + wid;
+    lv.cand_cap = kEveryFound;
+    if (every && lane == 0) found_sm[wid] = 0;
+    bool done = false;
+    for (uint64_t x0 = warp * each; !done && (every || x0 < total);) {
+        bool have;
+        uint2 c = make_uint2(0u, SIEVE_NO_RECORD);
+        if (!every) {
+            have = static_cast<uint32_t>(lane) < per && x0 + lane < total;
+            if (have) c = sv.cand[x0 + lane];
+            x0 += warps * each;
+            done = x0 >= total;
+        } else {
+            while (ready < 32 && (cnt || x0 < total)) {
+                if (cnt < 32 && x0 < total) {
+                    const uint64_t first = x0 + 4 * lane;
+                    const uint32_t keep = starts_left(a.text, n, first, total, sv.surv2, SIEVE_DEEP_M, 2, pol_keep);
+                    uint32_t g0 = 0, g1 = 0;
+                    if (keep) pack32_at(a.text, n, static_cast<uint32_t>(first), g0, g1);
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const uint32_t m = __ballot_sync(FULLMASK, (keep >> r) & 1u);
+                        if ((keep >> r) & 1u)
+                            left[cnt + __popc(m & lanemask_lt())] =
+                                make_uint2(static_cast<uint32_t>(first) + r, __funnelshift_r(g0, g1, 2 * r));
+                        cnt += __popc(m);
+                    }
+                    x0 += warps * each;
+                    continue;
+                }
+                const uint32_t k = min(cnt, 32u);
+                cnt -= k;
+                __syncwarp();
+                if (sv.l3) {
+                    sieve_levels<false>(lv, left + cnt, k, lane, pol_keep);
+                    __syncwarp();
+                    ready = *static_cast<volatile uint32_t *>(found_sm + wid);
+                } else {
+                    if (static_cast<uint32_t>(lane) < k)
+                        lv.cand[ready + lane] = make_uint2(left[cnt + lane].x, SIEVE_NO_RECORD);
+                    ready += k;
+                }
+                __syncwarp();
+            }
+            const uint32_t k = min(ready, 32u);
+            ready -= k;
+            have = static_cast<uint32_t>(lane) < k;
+            if (have) c = lv.cand[ready + lane];
+            __syncwarp();
+            if (lane == 0) found_sm[wid] = ready;
+            __syncwarp();
+            done = ready == 0 && cnt == 0 && x0 >= total;
+        }
         uint32_t e = PT_SKIP;      // entry for the exact path
         bool from_l2 = false;
         uint32_t parts = 0, matches = 0;
@@ -279,19 +341,13 @@ __global__ void __launch_bounds__(kFinishThreads, 2) finish_nfa(const ScanArgs a
         } else if (have) {
             uint32_t g0, g1;
             pack32_at(a.text, n, c.x, g0, g1);
-            if (every && n - c.x >= SIEVE_DEEP_M) {
-                const uint32_t d = g0 & ((1u << (2 * SIEVE_DEEP_M)) - 1);
-                have = (ldg_u32_keep(sv.surv2 + (d >> 5), pol_keep) >> (d & 31)) & 1u;
-            }
-            if (have) {
-                if (n - c.x >= kk) {
-                    e = a.memo[g0 & mask];
-                } else if (a.tail) {
-                    const int jl = static_cast<int>(n - c.x);
-                    e = __ldg(a.tail + tail_base(jl, 2) + (g0 & ((1u << (2 * jl)) - 1)));
-                } else {
-                    e = PT_WALK;
-                }
+            if (n - c.x >= kk) {
+                e = a.memo[g0 & mask];
+            } else if (a.tail) {
+                const int jl = static_cast<int>(n - c.x);
+                e = __ldg(a.tail + tail_base(jl, 2) + (g0 & ((1u << (2 * jl)) - 1)));
+            } else {
+                e = PT_WALK;
             }
         }
         const uint32_t qm = __ballot_sync(FULLMASK, e != PT_SKIP);
@@ -328,9 +384,8 @@ __global__ void __launch_bounds__(kFinishThreads, 2) finish_nfa(const ScanArgs a
             run_items(ov, mv, tv, sm, act, it, sn, lane, pol_keep);
         }
         __syncwarp();
-        x0 += warps * per;
         // the queue is drained when another 32 would not fit and at the end
-        if (wq_n && (wq_n + 32 > static_cast<uint32_t>(WARP_QUEUE) || x0 >= total)) {
+        if (wq_n && (wq_n + 32 > static_cast<uint32_t>(WARP_QUEUE) || done)) {
             drain_nfa<3>(ov, mv, tv, sm, wq_n, sn, lane, pol_keep);
             wq_n = 0;
             __syncwarp();
@@ -422,7 +477,7 @@ uint32_t layout_finish_nfa(ScanArgs &a, uint32_t band_bytes, uint32_t coop_bytes
     a.sm_band = take(band_bytes);
     a.band_smem = band_bytes > 0;
     a.sm_list = take(nw * kRunItems * sizeof(uint2));
-    a.sm_queue = take(nw * WARP_QUEUE * 6 + nw * (WARP_QUEUE / 8));
+    a.sm_queue = take(nw * (kQueueBytes + 4));   // the warps' queues, then their counters (found_sm)
     a.sm_stage = take(nw * a.stage_n * 16);
     a.sm_slots = take(nw * 2 * NFA_SLOT * 32 * 2);
     a.sm_coop = take(coop_bytes);
