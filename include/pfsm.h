@@ -220,7 +220,12 @@ int pfsm_scan(pfsm_ctx *ctx, pfsm_aut aut, const uint8_t *text_dev, uint64_t n,
  * On completion, status_dev (device, 2 x uint64) holds { |M|, error bits }
  * where error bit 0 = a symbol >= S, bit 1 = a device wait timed out.
  * Capturable in a CUDA graph once the automaton is resident (a scan
- * of a non-resident automaton reloads it, which is a host-synchronous copy).
+ * of a non-resident automaton reloads it, which is a host-synchronous copy)
+ * and a scan of it, as long or longer, has run on the stream. The graph reads
+ * the automaton's device copy as it was captured: until its last replay has
+ * finished the caller keeps the automaton loaded, resident and its parameters
+ * as they are, and issues no other scan that overlaps a replay on this stream's
+ * scratch.
  * Errors detected on the host are returned directly. */
 int pfsm_scan_async(pfsm_ctx *ctx, pfsm_aut aut, const uint8_t *text_dev, uint64_t n,
                     pfsm_match *out_dev, uint64_t cap, uint64_t *status_dev, void *stream);

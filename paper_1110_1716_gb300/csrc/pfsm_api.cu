@@ -1252,12 +1252,13 @@ int scan_enqueue(pfsm_ctx *ctx, pfsm_aut aut, const uint8_t *text, uint64_t n, u
         e = launch_carry_nfa(pl.a, ctx->nsm, std::min(pl.threads, 256), s);
         if (e != cudaSuccess) return PFSM_E_CUDA;
     }
-    {
-        Machine *mp = &m;
-        st = mark_use(ctx, s, &mp, 1);
-        if (st) return st;
-    }
-    return PFSM_OK;
+    // an event recorded under capture becomes the graph's and says nothing
+    // about its replays: those are the caller's to wait for
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
+    if (capture != cudaStreamCaptureStatusNone) return PFSM_OK;
+    Machine *mp = &m;
+    return mark_use(ctx, s, &mp, 1);
 }
 
 int finish_status(const unsigned long long *hs, uint64_t cap, uint64_t *n_matches) {

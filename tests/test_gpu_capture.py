@@ -59,6 +59,13 @@ def test_captured_scans(name, n):
         s.synchronize()
         assert status.tolist() == [len(want[1]), 0]
         del g
+        P.pfsm_evict(pf.ctx, a)
+        assert P.pfsm_scan(pf.ctx, a, text, n, out)[0] == P.PFSM_OK
+        P.pfsm_unload(pf.ctx, a)
+    # nothing of the capture is left for the next context's calls
+    with P.Pfsm(0) as pf:
+        got = oracle.sort_matches(pf.scan_numpy(pf.load(m), texts[0]))
+        assert np.array_equal(got, want[0])
 
 
 @pytest.mark.parametrize("n_motifs", [256, 450, 700])
