@@ -343,8 +343,8 @@ def run_ours(args, rank, world, local_rank):
             step_ms = float(t.item())
         kernel_ms = kms / max(1, klaunch)
         algo_bytes = n + 12 * int(cnt)
-        kind = 0 if hasattr(aut, "delta") else 1
-        launches_per_step = 2 if kind == 0 else 1
+        # the sieve and the kernel that finishes its candidates, or one direct scan
+        launches_per_step = 1 if name == "dna_dfa_1mib" else 2
         params = P.pfsm_get_params(pf.ctx, aid)
         res = {
             "workload": name, "desc": WORKLOADS[name], "bytes": n, "matches": int(cnt),

@@ -131,7 +131,13 @@ typedef struct {
 /* Create a context on CUDA device `device`. `budget_bytes` bounds the device
  * memory held by resident automata (0 = 8 GiB); scans reload evicted
  * automata and evict the least recently used ones to stay inside it (the
- * device form of the paper's treatment of insomnia, Sec. I-II). Errors:
+ * device form of the paper's treatment of insomnia, Sec. I-II). Where an
+ * automaton finds no room for all its tables, or a batch's automata do not fit
+ * together, their core tables are made resident alone and the general kernels
+ * take their scans. Outside the budget every stream that scans holds 16 MB of
+ * scratch, 32 MB more once a scan by the sieve or of long-lived instances has
+ * run on it, and 64 MB more once a batch with texts for the sieve has; where
+ * there is no room for those the general kernels take the call. Errors:
  * E_INVAL (bad device), E_CUDA, E_NOMEM. */
 int pfsm_ctx_create(int device, uint64_t budget_bytes, pfsm_ctx **out);
 
@@ -201,7 +207,10 @@ int pfsm_get_params(pfsm_ctx *ctx, pfsm_aut aut, pfsm_params *out);
 
 /* ------------------------------------------------------------------ scanning */
 /* Report every match of `aut` in the text (Sec. III.B; the result is the set
- * M above, in unspecified order).
+ * M above, in unspecified order). With default parameters, pattern sets take the
+ * sieve, machines whose starts mostly live the direct scan (up to a length
+ * where few of them do), and instances that never die are run segment by
+ * segment; every other scan takes the tile kernel that pfsm_params shapes.
  *   text_dev   device, n bytes, every byte < S (a byte >= S fails with
  *              E_INVAL after the scan; the output is then unspecified)
  *   out_dev    device, room for `cap` pfsm_match entries
@@ -231,10 +240,13 @@ int pfsm_scan_async(pfsm_ctx *ctx, pfsm_aut aut, const uint8_t *text_dev, uint64
                     pfsm_match *out_dev, uint64_t cap, uint64_t *status_dev, void *stream);
 
 /* Scan k texts, each with its own automaton, in one batch (the regex and
- * data partitioning of Sec. III.D combined). The automata are grouped into
- * classes (DFA or NFA, prefix-symbol width, DFA table in shared memory); each
- * class runs one persistent kernel over work units of a few consecutive tiles
- * of one text, and the class kernels of a batch run concurrently.
+ * data partitioning of Sec. III.D combined). Texts whose automata have the
+ * tables of the sieve or of the direct scan, and default parameters, run in two
+ * launches for all of them. The other automata are grouped into classes (DFA or
+ * NFA, prefix-symbol width, DFA table in shared memory); each class runs one
+ * persistent kernel over work units of a few consecutive tiles of one text, and
+ * the class kernels of a batch run concurrently.
+ * out_dev may begin at any multiple of four bytes.
  *   jobs     host, k entries; texts are device pointers
  *   out_dev  device, room for `cap` pfsm_bmatch entries (text = job index)
  *   counts   host, k entries; receives |M| per job (may be NULL)
@@ -315,8 +327,10 @@ int pfsm_scan_dfa_noalloc(const int16_t *delta_dev, int32_t Q, int32_t S, int32_
 /* ------------------------------------------------------------------ misc */
 int pfsm_get_stats(pfsm_ctx *ctx, pfsm_stats *out);
 
-/* Device bytes that automaton `aut` holds while resident (its encoded
- * tables; every automaton of one batch must fit the budget together), and
+/* Device bytes that automaton `aut` holds while resident with all its tables
+ * (a batch whose automata fit the budget together at these sizes reloads
+ * nothing; the core tables, which every automaton of a batch must have room
+ * for, are a good half of them for motif sets and nearly all for others), and
  * in *resident whether it is resident now (either pointer may be NULL).
  * The paper has no counterpart: this is a query for callers that pack
  * batches under a residency budget. Errors: E_INVAL, E_NOENT. */
@@ -343,7 +357,8 @@ int pfsm_test_hold_tiles(pfsm_ctx *ctx, int32_t enable);
 int pfsm_test_carry_cap(pfsm_ctx *ctx, uint32_t entries, uint32_t pool_states);
 
 /* Kernel timing: when enabled, every scan records CUDA events around its
- * tile kernel (a batch: around its graph) on the scan's stream;
+ * kernels (of a scan by the tile kernel: around that; a batch: around its graph
+ * and its flat kernels) on the scan's stream;
  * pfsm_kernel_time returns the summed milliseconds and launch count since
  * timing was last enabled. */
 int pfsm_set_timing(pfsm_ctx *ctx, int enable);

@@ -95,7 +95,7 @@ constexpr int SIEVE_DNA_STEP = 2, SIEVE_BYTE_STEP = 4;
 constexpr int SIEVE_NONE = 0, SIEVE_DNA = 1, SIEVE_BYTES = 2;
 constexpr int SIEVE_NEAR_M = 10;     // 128 KB: what a CTA's shared memory holds
 constexpr int SIEVE_DEEP_M = 13;     // 8 MB in L2
-constexpr int SIEVE_HASH_BITS = 19;  // 64 KB: three CTAs per SM
+constexpr int SIEVE_HASH_BITS = 19;  // 64 KB: two CTAs of 16 warps per SM
 constexpr int kSieveList = 64;       // a warp's list: refined by 32, up to 32 more at a time
 constexpr int SIEVE_PARTS = 3;       // strands of a record's set that a lane takes
 constexpr uint32_t SIEVE_NO_RECORD = 0xFFFFFFFFu;   // a candidate without a second-level record
@@ -380,8 +380,10 @@ struct FlatArgs {
 __host__ __device__ constexpr uint32_t flat_step(int cls, bool big) {
     return cls == FLAT_DNA ? 512u : cls == FLAT_BYTES ? 2048u : big ? 256u : 32u;
 }
-// Relative cost of one step: measured 0.49 ns of the whole chip per 512 bytes
-// of DNA, 0.42 ns per 2 KB of bytes and 2.4 ns per 256 starts of a dense DFA.
+// Relative cost of one step. Large form: measured 0.49 ns of the whole chip per
+// 512 bytes of DNA, 0.42 ns per 2 KB of bytes and 2.4 ns per 256 starts of a
+// dense DFA. Small form: chosen, not measured (a step there is a chain of
+// dependent loads, a little longer where there are more levels).
 __host__ __device__ constexpr uint32_t flat_cost(int cls, bool big) {
     return cls == FLAT_DNA ? (big ? 6u : 3u) : cls == FLAT_BYTES ? (big ? 5u : 2u) : (big ? 30u : 2u);
 }

@@ -5,10 +5,12 @@
 // (16 bytes per lane, the next loads in flight), and tests one gram per
 // SIEVE_BYTE_STEP starts. Where the bit is set, the starts are tested one by one
 // against the deep survival bitmap, and those that pass are appended to a
-// list of candidates. It holds no instance and reports no match, so it needs
-// few registers and runs at full occupancy; `finish_dfa` / `finish_nfa` then
-// run the few candidates (1 in 100 for the 256-motif NFA, 1 in 10,000 for
-// the 1000-signature trie), spread evenly over the SMs.
+// list of candidates. It holds no instance and reports no match: in its form for
+// long texts 61 - 63 registers and 32 warps per SM, as many as fit beside the
+// bitmap; for short ones 72 (DNA) and 104 (bytes) in CTAs of two warps.
+// `finish_dfa` / `finish_nfa` then run the few candidates (1 in 100 for the
+// 256-motif NFA, 1 in 10,000 for the 1000-signature trie), spread evenly over
+// the SMs.
 //
 // Measured on GB300 against the tile kernel that such scans took before
 // (device time per scan): 1000-signature trie, 1 GiB: 752 -> 203 us (5.3
@@ -17,8 +19,9 @@
 // 213 -> 69 us (bound by the random 32-byte reads of the bitmaps in L2, one
 // request per cycle and SM at 70 % of peak); 100 KB: 18 -> 17 us.
 //
-// Should the candidates outgrow their list, the finishing kernel takes every
-// start of the text instead (the list is then ignored): slower, same result.
+// Should the candidates outgrow their list (4 M), the finishing kernel takes
+// every start of the text that the bitmap of single starts leaves instead: same
+// result, in 0.4 - 0.7 of the tile kernel's time (finish.cuh).
 #include <atomic>
 
 #include "finish.cuh"
@@ -421,8 +424,9 @@ cudaError_t launch_sieve(const SieveArgs &a, int kind, int nsm, std::atomic<uint
     // once the steps tested with it outweigh the copying (whole scans, with
     // it and without: DNA 1 MiB 22.6 and 20.5 us, 2 MiB 22.2 and 21.8, 3 MiB
     // 23.1 and 26.1, 8 MiB 26.8 and 39.8; bytes 1 MiB 12.3 and 12.3, 4 MiB
-    // 14.3 and 16.4, 8 MiB 14.4 and 18.6, though 16 files of 4 MB with their
-    // matches sorted took 337 and 329 us)
+    // 14.3 and 16.4, 8 MiB 14.4 and 18.6; between 2 and 8 MiB both are right: 16
+    // files of 4 MB with their matches sorted took 337 and 329 us, which is
+    // within what runs differ by)
     const bool near_sm = a.n >= (kind == SIEVE_DNA ? 3u : 8u) << 20;
     if (kind == SIEVE_DNA) {
         const uint32_t lists = kSieveList * 16;
