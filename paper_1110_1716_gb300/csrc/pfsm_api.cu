@@ -770,7 +770,11 @@ int ensure_words(uint32_t **buf, size_t *have, size_t need) {
     return PFSM_OK;
 }
 
-Slot *get_slot(pfsm_ctx *ctx, cudaStream_t s) {
+// The slot of stream `s`; a new one comes with the candidate list when
+// automaton `aut`'s scans need it, and with the tile kernel's bitsets (16 warps
+// per SM) for a sieved NFA, where there is room for them (one allocation for
+// all: each further one cost a context's first scan 100 us).
+Slot *get_slot(pfsm_ctx *ctx, cudaStream_t s, int aut) {
     std::lock_guard<std::mutex> g(ctx->mu);
     auto it = ctx->slots.find(s);
     if (it != ctx->slots.end()) return &it->second;
@@ -778,7 +782,20 @@ Slot *get_slot(pfsm_ctx *ctx, cudaStream_t s) {
     void *p = nullptr;
     constexpr size_t head = 128;   // status, carry counters, the sieve's counters
     const size_t bytes = head + static_cast<size_t>(kCarryCap) * 16;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    const auto m = ctx->machines.find(aut);
+    if (m != ctx->machines.end() && (m->second.sv_kind || m->second.lives)) {
+        const size_t words = m->second.kind == 1 && m->second.sv_kind ? static_cast<size_t>(ctx->nsm) * 16 * 2 * ((m->second.Q + 31) / 32) : 0;
+        if (cudaMalloc(&p, bytes + kCandBytes + words * 4) == cudaSuccess) {
+            sl.inside = true;
+            sl.cand = reinterpret_cast<uint2 *>(static_cast<uint8_t *>(p) + bytes);
+            sl.coop_words = words;
+            if (words) sl.coop = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(p) + bytes + kCandBytes);
+            sl.coop_inside = words != 0;
+        } else {
+            cudaGetLastError();
+        }
+    }
+    if (!sl.inside && cudaMalloc(&p, bytes) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
@@ -1033,10 +1050,10 @@ static Route route_of(const pfsm_ctx *ctx, const Machine &m, uint64_t n, cudaStr
 }
 
 // Whether the stream has the sieve's candidate list (also the scratch of
-// long-lived scans), allocated by the first scan that needs it. Where there is
-// no room for it the tile kernel takes the scan.
+// long-lived scans), allocated with the slot or by the first scan that needs
+// it. Where there is no room for it the tile kernel takes the scan.
 static bool have_cand(Slot *slot) {
-    if (!slot->cand && cudaMalloc(&slot->cand, static_cast<size_t>(kCandCap) * sizeof(uint2)) != cudaSuccess) {
+    if (!slot->cand && cudaMalloc(&slot->cand, kCandBytes) != cudaSuccess) {
         cudaGetLastError();
         slot->cand = nullptr;
     }
@@ -1083,6 +1100,17 @@ static int walk_enqueue(pfsm_ctx *ctx, const Machine &m, const uint8_t *text, ui
     });
 }
 
+// At least `need` words of warp-wide bitsets (those that came with the slot stay
+// allocated with it when they do not do).
+static int ensure_coop(Slot *slot, size_t need) {
+    if (need > slot->coop_words && slot->coop_inside) {
+        slot->coop = nullptr;
+        slot->coop_words = 0;
+        slot->coop_inside = false;
+    }
+    return ensure_words(&slot->coop, &slot->coop_words, need);
+}
+
 // Warp-wide bitsets in global memory for a scan by the tile kernel.
 static int tile_coop(pfsm_ctx *ctx, const Machine &m, Slot *slot, Plan &pl) {
     if (m.kind != 1 || pl.a.coop_smem) return PFSM_OK;
@@ -1091,7 +1119,7 @@ static int tile_coop(pfsm_ctx *ctx, const Machine &m, Slot *slot, Plan &pl) {
     size_t warps = static_cast<size_t>(pl.grid) * (pl.threads / 32);
     if (pl.a.carry_cap) warps = std::max(warps, static_cast<size_t>(ctx->nsm) * (std::min(pl.threads, 256) / 32));
     const size_t need = warps * 2 * m.dm.Wq;
-    if (ensure_words(&slot->coop, &slot->coop_words, need)) return PFSM_E_NOMEM;
+    if (ensure_coop(slot, need)) return PFSM_E_NOMEM;
     pl.a.coop_g = slot->coop;
     return PFSM_OK;
 }
@@ -1172,7 +1200,7 @@ static int sieve_enqueue(pfsm_ctx *ctx, const Machine &m, const uint8_t *text, u
     if (smem > most) smem = layout_finish_nfa(f, 0, 0);
     if (!f.coop_smem) {
         const size_t words = static_cast<size_t>(2 * ctx->nsm) * warps * 2 * m.dm.Wq;
-        if (ensure_words(&slot->coop, &slot->coop_words, words)) return PFSM_E_NOMEM;
+        if (ensure_coop(slot, words)) return PFSM_E_NOMEM;
         f.coop_g = slot->coop;
     }
     return launch([&] { return launch_finish_nfa(f, a, smem, ctx->nsm, ctx->smem_set, s); });
@@ -1325,9 +1353,9 @@ int pfsm_ctx_destroy(pfsm_ctx *ctx) {
         for (int i = 0; i < kUseRing; ++i)
             if (kv.second.ev[i]) cudaEventDestroy(kv.second.ev[i]);
     for (auto &kv : ctx->slots) {
-        cudaFree(kv.second.coop);
+        if (!kv.second.coop_inside) cudaFree(kv.second.coop);
         cudaFree(kv.second.status);
-        cudaFree(kv.second.cand);
+        if (!kv.second.inside) cudaFree(kv.second.cand);
         cudaFreeHost(kv.second.host_status);
         for (int i = 0; i < 2 * kEventRing; ++i) cudaEventDestroy(kv.second.ev[i]);
     }
@@ -1597,7 +1625,7 @@ int pfsm_scan_async(pfsm_ctx *ctx, pfsm_aut aut, const uint8_t *text_dev, uint64
     if ((n > 0 && !text_dev) || (cap > 0 && !out_dev)) return PFSM_E_INVAL;
     DeviceGuard g(ctx->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    Slot *slot = get_slot(ctx, s);
+    Slot *slot = get_slot(ctx, s, aut);
     if (!slot) return PFSM_E_NOMEM;
     return scan_enqueue(ctx, aut, text_dev, n, reinterpret_cast<uint32_t *>(out_dev), cap,
                         reinterpret_cast<unsigned long long *>(status_dev), slot, s);
@@ -1610,7 +1638,7 @@ int pfsm_scan(pfsm_ctx *ctx, pfsm_aut aut, const uint8_t *text_dev, uint64_t n,
     if ((n > 0 && !text_dev) || (cap > 0 && !out_dev)) return PFSM_E_INVAL;
     DeviceGuard g(ctx->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    Slot *slot = get_slot(ctx, s);
+    Slot *slot = get_slot(ctx, s, aut);
     if (!slot) return PFSM_E_NOMEM;
     bool in_host = false;
     int st = scan_enqueue(ctx, aut, text_dev, n, reinterpret_cast<uint32_t *>(out_dev), cap,

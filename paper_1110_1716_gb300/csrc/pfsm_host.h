@@ -16,6 +16,7 @@ namespace pfsm {
 constexpr uint64_t kDefaultBudget = 8ull << 30;
 constexpr uint32_t kCarryCap = 1u << 20;     // carry entries per stream slot
 constexpr uint32_t kCandCap = 1u << 22;      // sieve candidates per stream slot (32 MB)
+constexpr size_t kCandBytes = kCandCap * sizeof(uint2);
 constexpr uint32_t kSmemMax = 232448;        // opt-in shared memory per CTA
 constexpr uint32_t kSmemStatic = 1024;       // room left for static shared memory (single-text kernels: none)
 constexpr uint32_t kBatchSmemStatic = 2048;  // the batch class kernels' static shared memory (1.5 KB)
@@ -98,6 +99,7 @@ struct Slot {   // per-stream scratch
     uint32_t *carry_n = nullptr;
     uint32_t *carry = nullptr;              // kCarryCap entries of 4 words
     uint2 *cand = nullptr;                  // kCandCap candidates of the sieve, when a scan has needed them
+    bool inside = false;                    // they lie behind the carry buffer, in one allocation
     // the sieve's counters, zero between scans: {matches, error bits} and
     // {candidates, CTAs done}
     unsigned long long *sv_status = nullptr;
@@ -106,6 +108,7 @@ struct Slot {   // per-stream scratch
     unsigned long long *host_status = nullptr;   // pinned [2]
     uint32_t *coop = nullptr;               // warp-wide NFA bitsets
     size_t coop_words = 0;
+    bool coop_inside = false;               // behind the candidates, likewise
     // automata (by the low bits of their ids) and the text length that `coop`
     // has been sized for (reserve_coop)
     struct { int id; uint64_t n; } coop_for[8] = {};
@@ -208,7 +211,7 @@ void drop_host_image(Machine &m);
 void sweep_retired(pfsm_ctx *ctx);
 int make_resident(pfsm_ctx *ctx, int id, Machine &m, cudaStream_t s, bool core = false);
 int mark_use(pfsm_ctx *ctx, cudaStream_t s, Machine *const *ms, size_t k);
-Slot *get_slot(pfsm_ctx *ctx, cudaStream_t s);
+Slot *get_slot(pfsm_ctx *ctx, cudaStream_t s, int aut = 0);
 int ensure_words(uint32_t **buf, size_t *have, size_t need);
 void collect_timing(pfsm_ctx *ctx, Slot *slot, int keep);
 int finish_status(const unsigned long long *hs, uint64_t cap, uint64_t *n_matches);

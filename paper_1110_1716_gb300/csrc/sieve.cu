@@ -204,14 +204,73 @@ static __device__ __forceinline__ void run_items(const OView &ov, const MView &m
     }
 }
 
+// Where the list is incomplete, each warp uses a part of its place for starts
+// that the bitmap leaves (kEveryLeft) and those with a record (kEveryFound).
+constexpr uint32_t kEveryLeft = 160, kEveryFound = 64;
+struct EveryState {
+    uint2 *left;           // the warp's part
+    uint64_t x0;           // the next start to look at
+    uint32_t cnt, ready;   // entries of both
+};
+// Collects candidates until a warp is full of them or the text ends, and takes
+// up to 32 from the end: their number is returned, `ready` is where they lie. A
+// function of its own, for the kernel's sake where lists are complete.
+static __device__ __noinline__ uint32_t every_fill(const SieveArgs &sv, EveryState &ev, uint32_t *ready_n, uint64_t warps,
+                                                   int lane) {
+    const uint64_t pol_keep = policy_evict_last();
+    const uint32_t n = sv.n;
+    uint2 *left = ev.left, *found = left + kEveryLeft;
+    uint64_t x0 = ev.x0;
+    uint32_t cnt = ev.cnt, ready = ev.ready;
+    SieveArgs lv = sv;
+    lv.cand = found;
+    lv.cand_n = ready_n;
+    lv.cand_cap = kEveryFound;
+    while (ready < 32 && (cnt || x0 < n)) {
+        if (cnt < 32 && x0 < n) {
+            const uint64_t first = x0 + 4 * lane;
+            const uint32_t keep = starts_left(sv.text, n, first, n, sv.surv2, SIEVE_DEEP_M, 2, pol_keep);
+            uint32_t g0 = 0, g1 = 0;
+            if (keep) pack32_at(sv.text, n, static_cast<uint32_t>(first), g0, g1);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const uint32_t m = __ballot_sync(FULLMASK, (keep >> r) & 1u);
+                if ((keep >> r) & 1u)
+                    left[cnt + __popc(m & lanemask_lt())] =
+                        make_uint2(static_cast<uint32_t>(first) + r, __funnelshift_r(g0, g1, 2 * r));
+                cnt += __popc(m);
+            }
+            x0 += warps * 128;
+            continue;
+        }
+        const uint32_t k = min(cnt, 32u);
+        cnt -= k;
+        __syncwarp();
+        if (sv.l3) {
+            sieve_levels<false>(lv, left + cnt, k, lane, pol_keep);
+            __syncwarp();
+            ready = *static_cast<volatile uint32_t *>(ready_n);
+        } else {
+            if (static_cast<uint32_t>(lane) < k) found[ready + lane] = make_uint2(left[cnt + lane].x, SIEVE_NO_RECORD);
+            ready += k;
+        }
+        __syncwarp();
+    }
+    const uint32_t k = min(ready, 32u);
+    ready -= k;
+    __syncwarp();
+    if (lane == 0) *ready_n = ready;
+    __syncwarp();
+    ev.x0 = x0;
+    ev.cnt = cnt;
+    ev.ready = ready;
+    return k;
+}
+
 // The candidates of an NFA, a warp's 32 at a time: those that come with a
 // second-level record report its matches and run on from its set, split into
 // strands (run_items); the others (near the end of the text, machines without
-// such tables, records of many states) take the general exact path. Where the
-// list is incomplete, each warp uses a part of its place for starts that the
-// bitmap leaves (kEveryLeft) and those with a record (kEveryFound), and takes
-// its candidates from there.
-constexpr uint32_t kEveryLeft = 160, kEveryFound = 64;
+// such tables, records of many states) take the general exact path.
 constexpr uint32_t kQueueBytes = WARP_QUEUE * 6 + WARP_QUEUE / 8;   // of a warp (smem_regions)
 static_assert(kQueueBytes % 4 == 0, "the counters behind the queues are aligned");
 __global__ void __launch_bounds__(kFinishThreads, 2) finish_nfa(const ScanArgs a, const SieveArgs sv) {
@@ -242,66 +301,30 @@ __global__ void __launch_bounds__(kFinishThreads, 2) finish_nfa(const ScanArgs a
     const uint32_t mask = (1u << (2 * kk)) - 1;
     uint2 *items = reinterpret_cast<uint2 *>(smem + a.sm_list) + wid * kRunItems;   // {lane << 16 | base, mask}
     uint32_t sn = 0, wq_n = 0;
-    const uint32_t each = every ? 128u : per;
     const uint64_t warp = static_cast<uint64_t>(wid) * gridDim.x + blockIdx.x;
-    // (every) the warp's part of the list's place, and the entries of both lists
-    uint2 *left = sv.cand + warp * (kEveryLeft + kEveryFound);
-    uint32_t *found_sm = reinterpret_cast<uint32_t *>(smem + a.sm_queue + nw * kQueueBytes);
-    uint32_t cnt = 0, ready = 0;
-    SieveArgs lv = sv;
-    lv.cand = left + kEveryLeft;
-    lv.cand_n = found_sm + wid;
-    lv.cand_cap = kEveryFound;
-    if (every && lane == 0) found_sm[wid] = 0;
+    uint32_t *ready_n = reinterpret_cast<uint32_t *>(smem + a.sm_queue + nw * kQueueBytes) + wid;
+    EveryState ev;
+    if (every) {
+        ev.left = sv.cand + warp * (kEveryLeft + kEveryFound);
+        ev.x0 = warp * 128;
+        ev.cnt = ev.ready = 0;
+        if (lane == 0) *ready_n = 0;
+    }
     bool done = false;
-    for (uint64_t x0 = warp * each; !done && (every || x0 < total);) {
+    for (uint64_t x0 = warp * per; !done && (every || x0 < total);) {
         bool have;
         uint2 c = make_uint2(0u, SIEVE_NO_RECORD);
         if (!every) {
             have = static_cast<uint32_t>(lane) < per && x0 + lane < total;
             if (have) c = sv.cand[x0 + lane];
-            x0 += warps * each;
+            x0 += warps * per;
             done = x0 >= total;
         } else {
-            while (ready < 32 && (cnt || x0 < total)) {
-                if (cnt < 32 && x0 < total) {
-                    const uint64_t first = x0 + 4 * lane;
-                    const uint32_t keep = starts_left(a.text, n, first, total, sv.surv2, SIEVE_DEEP_M, 2, pol_keep);
-                    uint32_t g0 = 0, g1 = 0;
-                    if (keep) pack32_at(a.text, n, static_cast<uint32_t>(first), g0, g1);
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const uint32_t m = __ballot_sync(FULLMASK, (keep >> r) & 1u);
-                        if ((keep >> r) & 1u)
-                            left[cnt + __popc(m & lanemask_lt())] =
-                                make_uint2(static_cast<uint32_t>(first) + r, __funnelshift_r(g0, g1, 2 * r));
-                        cnt += __popc(m);
-                    }
-                    x0 += warps * each;
-                    continue;
-                }
-                const uint32_t k = min(cnt, 32u);
-                cnt -= k;
-                __syncwarp();
-                if (sv.l3) {
-                    sieve_levels<false>(lv, left + cnt, k, lane, pol_keep);
-                    __syncwarp();
-                    ready = *static_cast<volatile uint32_t *>(found_sm + wid);
-                } else {
-                    if (static_cast<uint32_t>(lane) < k)
-                        lv.cand[ready + lane] = make_uint2(left[cnt + lane].x, SIEVE_NO_RECORD);
-                    ready += k;
-                }
-                __syncwarp();
-            }
-            const uint32_t k = min(ready, 32u);
-            ready -= k;
+            const uint32_t k = every_fill(sv, ev, ready_n, warps, lane);
             have = static_cast<uint32_t>(lane) < k;
-            if (have) c = lv.cand[ready + lane];
+            if (have) c = ev.left[kEveryLeft + ev.ready + lane];
             __syncwarp();
-            if (lane == 0) found_sm[wid] = ready;
-            __syncwarp();
-            done = ready == 0 && cnt == 0 && x0 >= total;
+            done = ev.ready == 0 && ev.cnt == 0 && ev.x0 >= total;
         }
         uint32_t e = PT_SKIP;      // entry for the exact path
         bool from_l2 = false;
@@ -481,7 +504,7 @@ uint32_t layout_finish_nfa(ScanArgs &a, uint32_t band_bytes, uint32_t coop_bytes
     a.sm_band = take(band_bytes);
     a.band_smem = band_bytes > 0;
     a.sm_list = take(nw * kRunItems * sizeof(uint2));
-    a.sm_queue = take(nw * (kQueueBytes + 4));   // the warps' queues, then their counters (found_sm)
+    a.sm_queue = take(nw * (kQueueBytes + 4));   // the warps' queues, then their counters (ready_n)
     a.sm_stage = take(nw * a.stage_n * 16);
     a.sm_slots = take(nw * 2 * NFA_SLOT * 32 * 2);
     a.sm_coop = take(coop_bytes);

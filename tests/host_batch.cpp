@@ -34,7 +34,7 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 int ensure_words(uint32_t **, size_t *, size_t) { return PFSM_OK; }
 int make_resident(pfsm_ctx *, int, Machine &m, cudaStream_t, bool) { return m.full = true, PFSM_OK; }
 int mark_use(pfsm_ctx *, cudaStream_t, Machine *const *, size_t k) { return seen.used = static_cast<int64_t>(k), PFSM_OK; }
-Slot *get_slot(pfsm_ctx *, cudaStream_t) { return nullptr; }
+Slot *get_slot(pfsm_ctx *, cudaStream_t, int) { return nullptr; }
 void collect_timing(pfsm_ctx *, Slot *, int) {}
 int finish_status(const unsigned long long *hs, uint64_t, uint64_t *n) { return *n = hs[0], PFSM_OK; }
 
