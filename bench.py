@@ -507,6 +507,8 @@ def compact_configs(main_name, main, others, detail):
         if r:
             out["f2_" + key] = {"lazy_ms": r4(r["lazy"]["ms"]), "chained_ms": r4(r["chained"]["ms"]),
                                 "matches": r["matches"]}
+            if "default" in r:
+                out["f2_" + key]["default_ms"] = r4(r["default"]["ms"])
     sv = others.get("serving")
     if sv:
         out["c4_serving"] = {
@@ -694,8 +696,10 @@ def measure_partitioning(P, pf, torch, dev, kind="dfa", n=16 << 10, steps=10):
     status = torch.zeros(2, dtype=torch.int64, device=dev)
     s = torch.cuda.Stream(device=dev)
     res = {"desc": desc, "bytes": n, "matches": int(cnt)}
-    for name, part in (("lazy", 1), ("chained", 2)):
-        P.pfsm_set_params(pf.ctx, aid, {"partition": part, "tile": 4096})
+    # by the tile kernel, both ways, and by default parameters (segments)
+    for name, params in (("lazy", {"partition": 1, "tile": 4096}), ("chained", {"partition": 2, "tile": 4096}),
+                         ("default", None)):
+        P.pfsm_set_params(pf.ctx, aid, params)
         ms = []
         for i in range(steps + 2):
             e0 = torch.cuda.Event(enable_timing=True)
