@@ -125,3 +125,13 @@ def test_sieve_needs_finals_past_its_step(pf):
         trie, _ = W.trie_dfa(sigs)
         t = np.random.default_rng(1).integers(0, 10, 20_001).astype(np.uint8)
         assert np.array_equal(scan_at(pf, pf.load(trie), t, 2), oracle.scan(trie, t))
+
+
+@pytest.mark.parametrize("n", [(3 << 20) - 1, (3 << 20) + 77])
+def test_dna_sieve_on_both_sides_of_3_mib(pf, n):
+    """2-bit symbols have the near bitmap in shared memory from 3 MiB on."""
+    nfa, motifs = motif(11, 90)
+    t = motif_text(motifs, n, 4000, 12)
+    assert np.array_equal(scan_at(pf, pf.load(nfa), t, 9), oracle.scan(nfa, t))
+    trie, _ = W.trie_dfa([bytes(x & 3 for x in s) for s in W.signature_set(13, n_sigs=60, len_lo=12, len_hi=20)], S=4)
+    assert np.array_equal(scan_at(pf, pf.load(trie), t, 2), oracle.scan(trie, t))
