@@ -297,21 +297,25 @@ __device__ __forceinline__ void flat_nfa(const FlatArgs &A, FlatOut &out, bool a
     __syncwarp();
 }
 
-// Candidates of the fallback, collected per warp: starts that the bitmap of
-// single starts leaves, then (NFA) those with a record.
-struct FlatEvery {
-    uint2 starts[64];      // {start, its first 16 symbols}
-    uint4 found[64];       // as the list of the front kernel has them
-    unsigned long long n;  // entries of found
-};
+// The fallback's candidates, collected per warp in a part of the place of the
+// list that overflowed: starts that the bitmap of single starts leaves
+// (kEveryLeft), then (NFA) those with a record (kEveryFound). Each warp's runs
+// are called from one place: with one for every way to fill a warp the code
+// outgrew the instruction cache, and warps waited for instructions half of the
+// time (256 MiB, 48 motifs: 7.0 ms, now 3.6).
+constexpr uint32_t kEveryLeft = 160, kEveryFound = 64;
+constexpr uint32_t kEveryPlace = kEveryLeft / 2 + kEveryFound;   // entries of 16 bytes
 
 // The starts [from, to) of one NFA's text, as the front kernel and the list
 // would have brought them: four starts per lane through the bitmap, then the
 // records and the runs of full warps of what is left.
-__device__ __forceinline__ void flat_every_nfa(const FlatArgs &A, uint32_t j, uint64_t from, uint64_t to, FlatEvery &E,
-                                               uint4 *items, FlatOut &out, int lane, uint64_t pol_keep) {
+__device__ __forceinline__ void flat_every_nfa(const FlatArgs &A, uint32_t j, uint64_t from, uint64_t to, uint4 *place,
+                                               unsigned long long *ready_n, uint4 *items, FlatOut &out, int lane,
+                                               uint64_t pol_keep) {
     const BatchJob &J = A.jobs[j];
     const DevMachine &M = A.machs[J.mach];
+    uint2 *left = reinterpret_cast<uint2 *>(place);   // {start, its first 16 symbols}
+    uint4 *found = place + kEveryLeft / 2;            // as the list of the front kernel has them
     SieveArgs a{};
     a.text = J.text;
     a.n = J.n;
@@ -321,55 +325,54 @@ __device__ __forceinline__ void flat_every_nfa(const FlatArgs &A, uint32_t j, ui
     a.l2tab = M.l2tab;
     a.l3 = M.sv_l3;
     a.job = j;
-    a.cand = reinterpret_cast<uint2 *>(E.found);
-    a.cand_sum = &E.n;
-    a.cand_cap = 64;
+    a.cand = reinterpret_cast<uint2 *>(found);
+    a.cand_sum = ready_n;
+    a.cand_cap = kEveryFound;
     const uint32_t *surv2 = M.surv2;
-    uint32_t cnt = 0;   // entries of E.starts
-    // runs the last entries of E.found, full warps of them (all at the end)
-    auto run = [&](bool all) {
-        __syncwarp();
-        uint32_t n = static_cast<uint32_t>(*static_cast<volatile unsigned long long *>(&E.n));
-        while (n >= 32 || (all && n)) {
-            const uint32_t k = min(n, 32u);
-            n -= k;
-            const uint4 c = E.found[n + min(static_cast<uint32_t>(lane), k - 1)];
-            flat_nfa(A, out, static_cast<uint32_t>(lane) < k, c.x, c.y, c.z, items, lane);
-        }
-        if (lane == 0) E.n = n;
-        __syncwarp();
-    };
-    for (; from < to; from += 128) {
-        const uint64_t first = from + 4 * lane;
-        const uint32_t keep = starts_left(a.text, a.n, first, to, surv2, SIEVE_DEEP_M, 2, pol_keep);
-        uint32_t g0 = 0, g1 = 0;
-        if (keep) pack32_at(a.text, a.n, static_cast<uint32_t>(first), g0, g1);
+    uint32_t cnt = 0, ready = 0;   // entries of both
+    while (true) {
+        while (ready < 32 && (cnt || from < to)) {
+            if (cnt < 32 && from < to) {
+                const uint64_t first = from + 4 * lane;
+                const uint32_t keep = starts_left(a.text, a.n, first, to, surv2, SIEVE_DEEP_M, 2, pol_keep);
+                uint32_t g0 = 0, g1 = 0;
+                if (keep) pack32_at(a.text, a.n, static_cast<uint32_t>(first), g0, g1);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const uint32_t m = __ballot_sync(FULLMASK, (keep >> r) & 1u);
-            if ((keep >> r) & 1u)
-                E.starts[cnt + __popc(m & lanemask_lt())] =
-                    make_uint2(static_cast<uint32_t>(first) + r, __funnelshift_r(g0, g1, 2 * r));
-            cnt += __popc(m);
-            if (cnt >= 32) {
-                cnt -= 32;
-                __syncwarp();
-                sieve_levels<true>(a, E.starts + cnt, 32, lane, pol_keep);
-                run(false);
+                for (int r = 0; r < 4; ++r) {
+                    const uint32_t m = __ballot_sync(FULLMASK, (keep >> r) & 1u);
+                    if ((keep >> r) & 1u)
+                        left[cnt + __popc(m & lanemask_lt())] =
+                            make_uint2(static_cast<uint32_t>(first) + r, __funnelshift_r(g0, g1, 2 * r));
+                    cnt += __popc(m);
+                }
+                from += 128;
+                continue;
             }
+            const uint32_t k = min(cnt, 32u);
+            cnt -= k;
+            __syncwarp();
+            sieve_levels<true>(a, left + cnt, k, lane, pol_keep);
+            __syncwarp();
+            ready = static_cast<uint32_t>(*static_cast<volatile unsigned long long *>(ready_n));
+            __syncwarp();
         }
+        if (ready == 0) break;
+        const uint32_t k = min(ready, 32u);
+        ready -= k;
+        const uint4 c = found[ready + min(static_cast<uint32_t>(lane), k - 1)];
+        __syncwarp();
+        if (lane == 0) *ready_n = ready;
+        __syncwarp();
+        flat_nfa(A, out, static_cast<uint32_t>(lane) < k, c.x, c.y, c.z, items, lane);
     }
-    __syncwarp();
-    if (cnt) sieve_levels<true>(a, E.starts, cnt, lane, pol_keep);
-    run(true);
 }
 
 // The same for a DFA.
-__device__ __forceinline__ void flat_every_dfa(const FlatArgs &A, uint32_t j, uint64_t from, uint64_t to, FlatEvery &E,
+__device__ __forceinline__ void flat_every_dfa(const FlatArgs &A, uint32_t j, uint64_t from, uint64_t to, uint4 *place,
                                                FlatOut &out, int lane, uint64_t pol_keep) {
     const BatchJob &J = A.jobs[j];
     const DevMachine &M = A.machs[J.mach];
-    uint32_t *left = reinterpret_cast<uint32_t *>(E.found), cnt = 0;   // (160 of its 256 words)
+    uint32_t *left = reinterpret_cast<uint32_t *>(place), cnt = 0;
     while (from < to || cnt) {
         for (; cnt < 32 && from < to; from += 128) {
             const uint64_t first = from + 4 * lane;
@@ -395,10 +398,11 @@ __device__ __forceinline__ void flat_every_dfa(const FlatArgs &A, uint32_t j, ui
 // turn to `warps` warps (this one is the me-th): texts may be long, and what a
 // start costs differs from place to place. A function of its own, so that the
 // kernel needs no more registers than the candidates do.
-static __device__ __noinline__ void flat_every(const FlatArgs &A, uint32_t kind, uint64_t me, uint64_t warps, FlatEvery &E,
-                                               uint4 *items, uint32_t *rows, int lane) {
+static __device__ __noinline__ void flat_every(const FlatArgs &A, uint32_t kind, uint64_t me, uint64_t warps,
+                                               unsigned long long *ready_n, uint4 *items, uint32_t *rows, int lane) {
     const uint64_t pol_keep = policy_evict_last();
-    if (lane == 0) E.n = 0;
+    uint4 *place = A.cand[kind] + me * kEveryPlace;
+    if (lane == 0) *ready_n = 0;
     FlatOut out{A, rows, 0u};
     for (int c = 0; c < FLAT_WALK; ++c) {
         const uint64_t span = flat_step(c, false);   // (the same in both forms)
@@ -412,8 +416,8 @@ static __device__ __noinline__ void flat_every(const FlatArgs &A, uint32_t kind,
                 s0 = j + 1 < A.job_hi[c] ? min(s1, A.jobs[j + 1].unit_begin) : s1;
                 if (b0 >= b1 || static_cast<uint32_t>(A.machs[J.mach].kind) != kind) continue;
                 const uint64_t to = min(static_cast<uint64_t>(J.n), b1 * span);
-                if (kind == 1) flat_every_nfa(A, j, b0 * span, to, E, items, out, lane, pol_keep);
-                else flat_every_dfa(A, j, b0 * span, to, E, out, lane, pol_keep);
+                if (kind == 1) flat_every_nfa(A, j, b0 * span, to, place, ready_n, items, out, lane, pol_keep);
+                else flat_every_dfa(A, j, b0 * span, to, place, out, lane, pol_keep);
             }
         }
     }
@@ -422,14 +426,13 @@ static __device__ __noinline__ void flat_every(const FlatArgs &A, uint32_t kind,
 
 // Even CTAs run the DFA candidates, odd ones the NFA candidates. A list that
 // overflowed (2 M) is replaced by every start of the texts of its kind: 256 MiB
-// dense in matches, class kernels and these, ms: 1000-signature trie 4.1, 2.6;
-// DNA trie 4.5, 2.4; 256 motifs 3.9, 4.1 and 6.4, 7.5; 48 motifs 5.7, 7.0 (a run
-// reads its band rows through L1 here, from shared memory there). All CTAs for
-// one kind where the other has no candidates: no faster there, and unions of
-// motif sets 593 -> 625 us.
+// dense in matches, class kernels and these, ms: 1000-signature trie 4.1, 2.3;
+// DNA trie 4.5, 2.2; 256 motifs 3.9, 2.7 and 6.4, 4.1; 48 motifs 5.7, 3.6. All
+// CTAs for one kind where the other has no candidates: unions of motif sets
+// 593 -> 625 us.
 __global__ void __launch_bounds__(256, 4) flat_finish(const __grid_constant__ FlatArgs A) {
     __shared__ uint4 items_sm[8][32 * SIEVE_PARTS];
-    __shared__ FlatEvery every_sm[8];
+    __shared__ unsigned long long ready_sm[8];   // flat_every
     __shared__ uint32_t rows_sm[8][kOutRows * 4];
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -439,7 +442,7 @@ __global__ void __launch_bounds__(256, 4) flat_finish(const __grid_constant__ Fl
     const uint64_t warps = static_cast<uint64_t>(ctas) * 8, me = static_cast<uint64_t>(wid) * ctas + blockIdx.x / 2;
     uint4 *items = items_sm[wid];
     if (found > A.cand_cap) {
-        flat_every(A, kind, me, warps, every_sm[wid], items, rows_sm[wid], lane);
+        flat_every(A, kind, me, warps, ready_sm + wid, items, rows_sm[wid], lane);
         return;
     }
     FlatOut out{A, rows_sm[wid], 0u};
