@@ -21,7 +21,7 @@
 //
 // Should the candidates outgrow their list (4 M), the finishing kernel takes
 // every start of the text that the bitmap of single starts leaves instead: same
-// result, in 0.4 - 0.7 of the tile kernel's time (finish.cuh).
+// result, in 0.4 - 0.75 of the tile kernel's time (finish.cuh).
 #include <atomic>
 
 #include "finish.cuh"
